@@ -58,27 +58,35 @@ __global__ void self_scale_kernel(SelfHighArgs A) {
 }
 
 // Psi[beta] = sum_m a_m psi0[m + beta] for 1 <= |beta| <= 2M (psi0 vanishes at
-// odd indices, so only m of the parity of beta contribute).
+// odd indices, so only m of the parity of beta contribute).  One warp per
+// beta, the lanes take its columns m in turn: one thread per beta ran up to
+// 961 dependent multiply-adds on 58 CTAs (92 us at M = 60).
 __global__ void self_psi_kernel(SelfHighArgs A) {
-  const int b = blockIdx.x * blockDim.x + threadIdx.x;
-  if (b >= A.NB) return;
+  const int b = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
+  if (b >= A.NB) return;  // whole warps
   const int bn = order_of_col(b + 1);  // bcol(b1, b2) = tri(|beta|) + b2 - 1
   const int b2 = b + 1 - tri(bn), b1 = bn - b2;
   double acc = 0.0;
   for (int m1 = b1 & 1; m1 <= A.M; m1 += 2)
-    for (int m2 = b2 & 1; m1 + m2 <= A.M; m2 += 2) {
+    for (int m2 = (b2 & 1) + 2 * lane; m1 + m2 <= A.M; m2 += 64) {
       const int a1 = m1 + b1, a2 = m2 + b2;
       acc = fma(A.at[mcol(m1, m2)], A.psi0[tri(a1 + a2) + a2], acc);
     }
-  A.Psi[b] = acc;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+  if (lane == 0) A.Psi[b] = acc;
 }
 
-// pass 1: U1[k2][l2][b1] (Gamma^I), U2[k2][l2][b1] (Gamma^II)
+// pass 1: U1[k2][l2][b1] (Gamma^I), U2[k2][l2][b1] (Gamma^II).  Pass 3 reads
+// V[k2][l1][b1] at b1 <= k1 + l1 + 1 with k1 <= M - k2 only, and pass 2 sums U
+// over l1 + l2 <= M, so b1 <= 2M - k2 - l2 + 1 covers all that is used (half
+// of the array).
 __global__ void self_pass1_kernel(SelfHighArgs A) {
   const int M = A.M, W = 2 * M + 1;
   const int idx = blockIdx.x * blockDim.x + threadIdx.x;
   if (idx >= (M + 1) * (M + 1) * W) return;
   const int b1 = idx % W, l2 = (idx / W) % (M + 1), k2 = idx / (W * (M + 1));
+  if (b1 > 2 * M - k2 - l2 + 1) return;
   // C(l2, q) g(k2 - q) and C(l2, q) g(k2 - 1 - q), q = 0, 1, ...
   const double* c1 = A.cg + ((size_t)l2 * (M + 1) + k2) * (M + 1);
   double u1 = 0.0, u2 = 0.0;
@@ -97,12 +105,13 @@ __global__ void self_pass1_kernel(SelfHighArgs A) {
   A.U2[idx] = u2;
 }
 
-// pass 2: V[k2][l1][b1] = sum_{l2 <= M - l1} (-1)^{l2} a_{l1,l2} U[k2][l2][b1]
+// pass 2 (b1 <= M - k2 + l1 + 1, see pass 1): V[k2][l1][b1] = sum_{l2 <= M - l1} (-1)^{l2} a_{l1,l2} U[k2][l2][b1]
 __global__ void self_pass2_kernel(SelfHighArgs A) {
   const int M = A.M, W = 2 * M + 1;
   const int idx = blockIdx.x * blockDim.x + threadIdx.x;
   if (idx >= (M + 1) * (M + 1) * W) return;
   const int b1 = idx % W, l1 = (idx / W) % (M + 1), k2 = idx / (W * (M + 1));
+  if (b1 > M - k2 + l1 + 1) return;
   const double* u1 = A.U1 + (size_t)k2 * (M + 1) * W + b1;
   const double* u2 = A.U2 + (size_t)k2 * (M + 1) * W + b1;
   double v1 = 0.0, v2 = 0.0;
@@ -186,7 +195,7 @@ cudaError_t launch_self_high(SelfHighArgs A, double* scratch, cudaStream_t st) {
   A.V2 = A.V1 + P;
   const int T = 128;
   self_scale_kernel<<<(A.K + T - 1) / T, T, 0, st>>>(A);
-  self_psi_kernel<<<(A.NB + T - 1) / T, T, 0, st>>>(A);
+  self_psi_kernel<<<(A.NB * 32 + T - 1) / T, T, 0, st>>>(A);
   self_pass1_kernel<<<(int)((P + T - 1) / T), T, 0, st>>>(A);
   self_pass2_kernel<<<(int)((P + T - 1) / T), T, 0, st>>>(A);
   self_pass3_kernel<<<(A.K * 32 + T - 1) / T, T, 0, st>>>(A);
