@@ -83,7 +83,7 @@ struct mmvm_ctx {
   cudaStream_t own = nullptr, st = nullptr;
   DevBuf<double> x, m, xs, ms, xsum, msum, rdx, rdm, scal, partial;
   DevBuf<unsigned char> rec, order_tmp;
-  DevBuf<int> flags, k_off, e_l, e_b, perm;
+  DevBuf<int> flags, perm;
   DevBuf<float> gbox;  // group records (gdata_len(M) floats per kGroup sorted positions)
   // cumulative work of the all-pairs kernel: near pairs, far pairs source by
   // source, tile expansions evaluated, pairs those expansions covered
@@ -95,7 +95,9 @@ struct mmvm_ctx {
   DevBuf<double> dk;                  // adaptive steps: 7 stage derivatives
   DevBuf<unsigned long long> derr;    // adaptive steps: error of the step (bits)
   int order_launches = 0;  // kernels launched by one spatial ordering
-  DevBuf<double> e_c, psi0;
+  DevBuf<unsigned char> ftab;  // finish tables (blob of tables.h)
+  mmvm::FinishTab ft;
+  int sms = 1;                 // multiprocessors of the device
   mmvm::PairEntry pe;
   // interaction-list form of the all-pairs kernels (FP32 with the far field):
   // near lists (G x G entries, G counts), far-field partials (lfar blocks of
@@ -113,7 +115,6 @@ struct mmvm_ctx {
   int lc = 0, tfar = 1;
   int S = 32;            // sources per shared-memory tile
   int chunks = 1;        // source chunks of the pair kernel
-  int finish_tb = 1;     // targets per finish block
   bool graph_ok = false;
   cudaGraph_t graph = nullptr;
   cudaGraphExec_t gexec = nullptr;
@@ -327,7 +328,7 @@ int enqueue_rhs(mmvm_ctx* c, int mode, const double* xin, const double* min_, do
     H.K = c->K;
     H.NB = c->NB;
     H.Min = min_;
-    H.psi0 = c->psi0.p;
+    H.psi0 = c->ft.psi0;
     H.binom = c->sbinom.p;
     H.g = c->sg.p;
     H.cg = c->scg.p;
@@ -341,8 +342,8 @@ int enqueue_rhs(mmvm_ctx* c, int mode, const double* xin, const double* min_, do
     H.out_dM = out_dM;
     H.y_x = c->x.p;
     H.y_M = c->m.p;
-    H.ys_x = c->xs.p;
-    H.ys_M = c->ms.p;
+    H.ys_x = mode == 2 ? c->rdx.p : c->xs.p;
+    H.ys_M = mode == 2 ? c->rdm.p : c->ms.p;
     H.sum_x = c->xsum.p;
     H.sum_M = c->msum.p;
     MMVM_CK(mmvm::launch_self_high(H, c->sscr.p, c->st));
@@ -360,15 +361,10 @@ int enqueue_rhs(mmvm_ctx* c, int mode, const double* xin, const double* min_, do
     A.nfar = c->tree ? c->tfar : c->lfar;
     A.n_edge = c->le.far.n_edge;
   }
-  A.targets_per_block = c->finish_tb;
   A.partial = n > 1 ? c->partial.p : nullptr;
   A.perm = perm;
   A.Min = min_;
-  A.k_off = c->k_off.p;
-  A.e_l = c->e_l.p;
-  A.e_b = c->e_b.p;
-  A.e_c = c->e_c.p;
-  A.psi0 = c->psi0.p;
+  A.tab = c->ft;
   A.lam0sq = lam0sq;
   A.four_nu = four_nu;
   A.t_dev = c->t_dev();
@@ -379,11 +375,12 @@ int enqueue_rhs(mmvm_ctx* c, int mode, const double* xin, const double* min_, do
   A.out_dM = out_dM;
   A.y_x = c->x.p;
   A.y_M = c->m.p;
-  A.ys_x = c->xs.p;
-  A.ys_M = c->ms.p;
+  // stage 2 writes the RHS buffers, so that no stage overwrites its input
+  A.ys_x = mode == 2 ? c->rdx.p : c->xs.p;
+  A.ys_M = mode == 2 ? c->rdm.p : c->ms.p;
   A.sum_x = c->xsum.p;
   A.sum_M = c->msum.p;
-  MMVM_CK(mmvm::launch_finish(A, c->st));
+  MMVM_CK(mmvm::launch_finish(A, c->sms, c->st));
   c->launches += 1;
   return MMVM_OK;
 }
@@ -393,7 +390,7 @@ int enqueue_step(mmvm_ctx* c) {
   double* dt = c->dt_dev();
   if ((rc = enqueue_rhs(c, 1, c->x.p, c->m.p, 0.0, dt))) return rc;
   if ((rc = enqueue_rhs(c, 2, c->xs.p, c->ms.p, 0.5, dt))) return rc;
-  if ((rc = enqueue_rhs(c, 3, c->xs.p, c->ms.p, 0.5, dt))) return rc;
+  if ((rc = enqueue_rhs(c, 3, c->rdx.p, c->rdm.p, 0.5, dt))) return rc;
   if ((rc = enqueue_rhs(c, 4, c->xs.p, c->ms.p, 1.0, dt))) return rc;
   MMVM_CK(mmvm::launch_advance_time(c->t_dev(), dt, c->st));
   c->launches += 1;
@@ -723,8 +720,8 @@ int mmvm_create(const mmvm_config* cfg, mmvm_ctx** out) {
       return fail(MMVM_E_UNSUPPORTED, "pair kernel variant not compiled");
     }
   }
-  const int K = c->K;
-  c->finish_tb = std::max(1, 128 / (((K + 31) / 32) * 32));
+  cudaDeviceGetAttribute(&c->sms, cudaDevAttrMultiProcessorCount, cfg->device);
+  c->sms = std::max(c->sms, 1);
   c->S = mmvm::kGroup;
   auto bail = [&](int rc) {
     mmvm_destroy(c);
@@ -751,25 +748,15 @@ int mmvm_create(const mmvm_config* cfg, mmvm_ctx** out) {
                         cudaMemcpyHostToDevice)) != cudaSuccess)
       return bail(cuda_fail(e, "separable tables"));
   }
-  if ((e = c->k_off.ensure(T.k_off.size())) != cudaSuccess ||
-      (e = c->e_l.ensure(T.e_l.size())) != cudaSuccess ||
-      (e = c->e_b.ensure(T.e_b.size())) != cudaSuccess ||
-      (e = c->e_c.ensure(T.e_c.size())) != cudaSuccess ||
-      (e = c->psi0.ensure(T.psi0.size())) != cudaSuccess ||
-      (e = c->scal.ensure(2)) != cudaSuccess || (e = c->flags.ensure(2)) != cudaSuccess ||
-      (e = c->counts.ensure(4)) != cudaSuccess)
+  const std::vector<unsigned char> tb = T.blob();
+  if ((e = c->ftab.ensure(tb.size())) != cudaSuccess || (e = c->scal.ensure(2)) != cudaSuccess ||
+      (e = c->flags.ensure(2)) != cudaSuccess || (e = c->counts.ensure(4)) != cudaSuccess)
     return bail(cuda_fail(e, "cudaMalloc(tables)"));
-  auto up = [&](void* d, const void* h, size_t bytes) {
-    return bytes ? cudaMemcpy(d, h, bytes, cudaMemcpyHostToDevice) : cudaSuccess;
-  };
-  if ((e = up(c->k_off.p, T.k_off.data(), T.k_off.size() * sizeof(int))) != cudaSuccess ||
-      (e = up(c->e_l.p, T.e_l.data(), T.e_l.size() * sizeof(int))) != cudaSuccess ||
-      (e = up(c->e_b.p, T.e_b.data(), T.e_b.size() * sizeof(int))) != cudaSuccess ||
-      (e = up(c->e_c.p, T.e_c.data(), T.e_c.size() * sizeof(double))) != cudaSuccess ||
-      (e = up(c->psi0.p, T.psi0.data(), T.psi0.size() * sizeof(double))) != cudaSuccess ||
+  if ((e = cudaMemcpy(c->ftab.p, tb.data(), tb.size(), cudaMemcpyHostToDevice)) != cudaSuccess ||
       (e = cudaMemset(c->scal.p, 0, 2 * sizeof(double))) != cudaSuccess ||
       (e = cudaMemset(c->counts.p, 0, 4 * sizeof(unsigned long long))) != cudaSuccess)
     return bail(cuda_fail(e, "cudaMemcpy(tables)"));
+  c->ft = mmvm::finish_tab(T, c->ftab.p);
   if (c->pe.nslices && (e = mmvm::pair_prepare(c->pe, c->S)) != cudaSuccess)
     return bail(cuda_fail(e, "pair kernel shared-memory limit"));
   *out = c;
@@ -788,7 +775,7 @@ void mmvm_destroy(mmvm_ctx* c) {
     for (auto& e : pr)
       if (e) cudaEventDestroy(e);
   for (auto* b : {&c->x, &c->m, &c->xs, &c->ms, &c->xsum, &c->msum, &c->rdx, &c->rdm, &c->scal,
-                  &c->partial, &c->e_c, &c->psi0, &c->sbinom, &c->sg, &c->scg, &c->sscr, &c->dpts, &c->dval, &c->dring, &c->dk,
+                  &c->partial, &c->sbinom, &c->sg, &c->scg, &c->sscr, &c->dpts, &c->dval, &c->dring, &c->dk,
                   &c->fpart})
     b->release();
   c->tnodes.release();
@@ -802,9 +789,7 @@ void mmvm_destroy(mmvm_ctx* c) {
   c->perm.release();
   c->gbox.release();
   c->flags.release();
-  c->k_off.release();
-  c->e_l.release();
-  c->e_b.release();
+  c->ftab.release();
   if (c->own) cudaStreamDestroy(c->own);
   delete c;
 }

@@ -41,7 +41,7 @@ namespace {
 constexpr int kMaxN = 4096;
 constexpr int kMaxOrder = 8;
 constexpr int kChunks = 2;
-// tables region: k_off, e_l, e_b (int) and e_c, psi0 (double), sized for order 8
+// tables region: the finish tables (blob of tables.h), sized for order 8
 constexpr size_t kTableBytes = 1u << 20;
 // largest record: FP64 order 8, 48 doubles = 384 bytes (FP32: 68 floats)
 constexpr size_t kRecBytes = (size_t)kMaxN * 384;
@@ -56,7 +56,8 @@ struct DeviceScratch {
   bool ready = false;
   unsigned char* base = nullptr;  // device address of g_scratch on this device
   int tables_order = -1;          // order whose tables are resident
-  int off_koff = 0, off_el = 0, off_eb = 0, off_ec = 0, off_psi0 = 0;
+  mmvm::FinishTab tab;
+  int sms = 1;
 };
 std::mutex g_mu;
 DeviceScratch g_dev[64];
@@ -69,8 +70,6 @@ int set_err(int code, const std::string& m) {
   mmvm::set_last_error(m.c_str());
   return code;
 }
-
-size_t align256(size_t v) { return (v + 255) & ~(size_t)255; }
 
 }  // namespace
 
@@ -105,6 +104,7 @@ extern "C" int mmvm_rhs_noalloc(const mmvm_config* cfg, int64_t n, double t, con
     if (e != cudaSuccess)
       return set_err(MMVM_E_DEVICE, std::string("cudaGetSymbolAddress: ") + cudaGetErrorString(e));
     ds.base = static_cast<unsigned char*>(p);
+    cudaDeviceGetAttribute(&ds.sms, cudaDevAttrMultiProcessorCount, dev);
     ds.ready = true;
   }
   if (ds.tables_order != M) {  // upload the finish tables of this order
@@ -114,36 +114,15 @@ extern "C" int mmvm_rhs_noalloc(const mmvm_config* cfg, int64_t n, double t, con
         return set_err(MMVM_E_DEVICE, std::string("synchronize: ") + cudaGetErrorString(e));
     }
     FinishTables T = build_finish_tables(M);
-    size_t off = 0;
-    ds.off_koff = (int)off;
-    off = align256(off + T.k_off.size() * sizeof(int));
-    ds.off_el = (int)off;
-    off = align256(off + T.e_l.size() * sizeof(int));
-    ds.off_eb = (int)off;
-    off = align256(off + T.e_b.size() * sizeof(int));
-    ds.off_ec = (int)off;
-    off = align256(off + T.e_c.size() * sizeof(double));
-    ds.off_psi0 = (int)off;
-    off = align256(off + T.psi0.size() * sizeof(double));
-    if (off > kTableBytes) return set_err(MMVM_E_UNSUPPORTED, "tables exceed the fixed scratch");
-    struct Up {
-      int off;
-      const void* src;
-      size_t bytes;
-    } ups[] = {{ds.off_koff, T.k_off.data(), T.k_off.size() * sizeof(int)},
-               {ds.off_el, T.e_l.data(), T.e_l.size() * sizeof(int)},
-               {ds.off_eb, T.e_b.data(), T.e_b.size() * sizeof(int)},
-               {ds.off_ec, T.e_c.data(), T.e_c.size() * sizeof(double)},
-               {ds.off_psi0, T.psi0.data(), T.psi0.size() * sizeof(double)}};
-    for (const Up& u : ups) {
-      if (!u.bytes) continue;
-      e = cudaMemcpyAsync(ds.base + u.off, u.src, u.bytes, cudaMemcpyHostToDevice, st);
-      if (e != cudaSuccess)
-        return set_err(MMVM_E_DEVICE, std::string("table upload: ") + cudaGetErrorString(e));
-    }
+    const std::vector<unsigned char> tb = T.blob();
+    if (tb.size() > kTableBytes) return set_err(MMVM_E_UNSUPPORTED, "tables exceed the fixed scratch");
+    e = cudaMemcpyAsync(ds.base, tb.data(), tb.size(), cudaMemcpyHostToDevice, st);
+    if (e != cudaSuccess)
+      return set_err(MMVM_E_DEVICE, std::string("table upload: ") + cudaGetErrorString(e));
     e = cudaStreamSynchronize(st);  // the host vectors go out of scope here
     if (e != cudaSuccess)
       return set_err(MMVM_E_DEVICE, std::string("table upload: ") + cudaGetErrorString(e));
+    ds.tab = finish_tab(T, ds.base);
     ds.tables_order = M;
   }
   unsigned char* base = ds.base;
@@ -172,14 +151,9 @@ extern "C" int mmvm_rhs_noalloc(const mmvm_config* cfg, int64_t n, double t, con
   A.K = K;
   A.NB = NB;
   A.nchunks = chunks;
-  A.targets_per_block = std::max(1, 128 / (((K + 31) / 32) * 32));  // as for a context
   A.partial = n > 1 ? partial : nullptr;
   A.Min = d_moments;
-  A.k_off = reinterpret_cast<const int*>(base + ds.off_koff);
-  A.e_l = reinterpret_cast<const int*>(base + ds.off_el);
-  A.e_b = reinterpret_cast<const int*>(base + ds.off_eb);
-  A.e_c = reinterpret_cast<const double*>(base + ds.off_ec);
-  A.psi0 = reinterpret_cast<const double*>(base + ds.off_psi0);
+  A.tab = ds.tab;
   A.lam0sq = lam0sq;
   A.four_nu = four_nu;
   A.t_dev = t_dev;
@@ -188,7 +162,7 @@ extern "C" int mmvm_rhs_noalloc(const mmvm_config* cfg, int64_t n, double t, con
   A.mode = 0;
   A.out_dx = d_dxdt;
   A.out_dM = d_dMdt;
-  if ((e = launch_finish(A, st)) != cudaSuccess)
+  if ((e = launch_finish(A, ds.sms, st)) != cudaSuccess)
     return set_err(MMVM_E_DEVICE, std::string("finish: ") + cudaGetErrorString(e));
   return MMVM_OK;
 }

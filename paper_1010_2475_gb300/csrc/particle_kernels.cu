@@ -189,25 +189,45 @@ __global__ void group_multipole_kernel(int n, const float* __restrict__ rec,
   }
 }
 
-// Shared-memory layout per block: for each of TB targets, Psi[NB], a[K], X[2],
-// M_00 (read before any in-place stage write), then the powers c^{-s/2}.
-// The block handles sorted positions j0 .. j0 + TB - 1 (those below A.n); all
-// its threads call this, and it ends with the block's last writes to shared
-// memory behind no barrier (a caller that loops must add one).
-__device__ __forceinline__ void finish_block(const FinishArgs& A, int j0, double* sm) {
-  const int TB = A.targets_per_block;
-  const int NB = A.NB, K = A.K, M = A.M;
-  double* psi = sm;                       // TB * NB
-  double* at = psi + TB * NB;             // TB * K
-  double* X = at + TB * K;                // TB * 2
-  double* m00s = X + TB * 2;              // TB
-  double* cpow = m00s + TB;               // c^{-s/2}, s = 0..2M+2
+// The finish of TG targets (sorted positions j0 .. j0 + TG - 1, those below
+// A.n) by one CTA, moment rows [k0, k1) with the table pieces [p0, p1).
+//
+// Bound: FP64 arithmetic (2 FMA per cycle and SM here, 1/64 of FP32).  Per
+// target: the sums over the partial blocks, NB K / 4 multiply-adds of the
+// self pair and one multiply-add per table entry and (k, l) group (4214 at
+// M = 6; the form c a_l Psi took 6916).  A thread takes whole pieces of the
+// table for one target, so that rows of very different length (0 to 260
+// entries at M = 6) do not leave lanes idle, and the entries are read by
+// neighbouring threads side by side.  TG = 32 makes the entry stream of a warp
+// uniform; small n takes smaller TG so that every SM has work
+// (finish_targets).  Shared memory holds [column][target] arrays: Psi (NB), a
+// (K), X (2), M_00, the powers c^{-s/2} and the pieces' sums.  Every global
+// read of the stage input precedes the first write behind a barrier.  All
+// threads of the CTA call this; a caller that loops must add a barrier.
+template <int TG>
+__device__ __forceinline__ void finish_block(const FinishArgs& A, int j0, int k0, int k1,
+                                             double* sm) {
+  const int NB = A.NB, K = A.K, M = A.M, NT = blockDim.x;
+  const int p0 = A.tab.row_off[k0], p1 = A.tab.row_off[k1];
+  double* psi = sm;                 // NB * TG
+  double* at = psi + NB * TG;       // K * TG
+  double* X = at + K * TG;          // 2 * TG
+  double* m00s = X + 2 * TG;        // TG
+  double* cpow = m00s + TG;         // c^{-s/2}, s = 0..M
+  double* pres = cpow + M + 1;      // (p1 - p0) * TG
   const double c = stage_c(A.t_dev, A.dt_dev, A.cs, A.lam0sq, A.four_nu);
-  for (int s = threadIdx.x; s <= 2 * M + 2; s += blockDim.x) cpow[s] = pow(c, -0.5 * s);
+  if (threadIdx.x <= M) {  // c^{-s/2} by repeated squaring of 1/c: a few roundings
+    double base = 1.0 / c, v = (threadIdx.x & 1) ? 1.0 / sqrt(c) : 1.0;
+    for (int e = threadIdx.x >> 1; e; e >>= 1) {
+      if (e & 1) v *= base;
+      base *= base;
+    }
+    cpow[threadIdx.x] = v;
+  }
   __syncthreads();
-  // 1. Psi_excl = sum over source chunks (fixed order), scaled moments
-  for (int idx = threadIdx.x; idx < TB * NB; idx += blockDim.x) {
-    const int tt = idx / NB, b = idx % NB, j = j0 + tt;
+  // 1. Psi_excl = sum over the partial blocks (fixed order), scaled moments
+  for (int idx = threadIdx.x; idx < TG * NB; idx += NT) {
+    const int tt = idx % TG, b = idx / TG, j = j0 + tt;
     double v = 0.0;
     if (j < A.n && A.partial) {
       for (int ch = 0; ch < A.nchunks; ++ch) v += A.partial[((size_t)ch * NB + b) * A.n + j];
@@ -221,82 +241,107 @@ __device__ __forceinline__ void finish_block(const FinishArgs& A, int j0, double
         }
       }
     }
-    psi[idx] = v;
+    psi[b * TG + tt] = v;
   }
-  __syncthreads();
-  // 1b. the pair kernels leave Psi itself only in the edge columns beta1 <= 1;
-  //     a column beta1 >= 2 holds R[beta] = sum_m a_m D^{m + beta - 2 e1} Lap psi.
-  //     D_1^2 = Lap - D_2^2 gives Psi[beta] = R[beta] - Psi[beta - 2 e1 + 2 e2],
-  //     taken per order in increasing beta1.
-  const int BM = bmax_of(M);
-  for (int idx = threadIdx.x; idx < TB * BM; idx += blockDim.x) {
-    const int tt = idx / BM, k = idx % BM + 1;
-    double* ps = psi + tt * NB;
-    for (int b1 = 2; b1 <= k; ++b1) ps[bcol(b1, k - b1)] -= ps[bcol(b1 - 2, k - b1 + 2)];
-  }
-  for (int idx = threadIdx.x; idx < TB * K; idx += blockDim.x) {
+  for (int idx = threadIdx.x; idx < TG * K; idx += NT) {
     const int tt = idx / K, m = idx % K, p = j0 + tt;
     int s = 0;
-    while ((s + 1) * (s + 2) / 2 <= m) ++s;  // total order of column m
+    while (tri(s + 1) <= m) ++s;  // total order of column m
     const int j = p < A.n ? (A.perm ? A.perm[p] : p) : 0;
     const double mv = (p < A.n) ? A.Min[(size_t)j * K + m] : 0.0;
-    at[idx] = mv * cpow[s];
+    at[m * TG + tt] = mv * cpow[s];
     if (m == 0) m00s[tt] = (p < A.n) ? mv : 1.0;
   }
   __syncthreads();
-  // 2. centroid sums X_c = sum_m (-1)^{|m|} a_m What_c[m], What_1[m] = -Psi[m+e2],
-  //    What_2[m] = Psi[m+e1]  (eq:xjdot_Final in c = 1 units, self pair excluded)
-  for (int idx = threadIdx.x; idx < TB * 2; idx += blockDim.x) {
-    const int tt = idx >> 1, comp = idx & 1;
-    double acc = 0.0;
-    int col = 0;
-    for (int s = 0; s <= M; ++s) {
-      const double sg = (s & 1) ? -1.0 : 1.0;
-      for (int m2 = 0; m2 <= s; ++m2, ++col) {
-        const int m1 = s - m2;
-        const double a = at[tt * K + col];
-        if (comp == 0) acc -= sg * a * psi[tt * NB + bcol(m1, m2 + 1)];
-        else acc += sg * a * psi[tt * NB + bcol(m1 + 1, m2)];
-      }
+  if (A.partial) {
+    // 1b. the pair kernels leave Psi itself only in the edge columns beta1 <= 1;
+    //     a column beta1 >= 2 holds R[beta] = sum_m a_m D^{m + beta - 2 e1} Lap psi.
+    //     D_1^2 = Lap - D_2^2 gives Psi[beta] = R[beta] - Psi[beta - 2 e1 + 2 e2],
+    //     taken per order in increasing beta1.
+    const int BM = bmax_of(M);
+    for (int idx = threadIdx.x; idx < TG * BM; idx += NT) {
+      const int tt = idx % TG, k = idx / TG + 1;
+      double* ps = psi + tt;
+      for (int b1 = 2; b1 <= k; ++b1)
+        ps[bcol(b1, k - b1) * TG] -= ps[bcol(b1 - 2, k - b1 + 2) * TG];
     }
-    X[idx] = acc;
+    __syncthreads();
+    // 2. centroid sums X_c = sum_m (-1)^{|m|} a_m What_c[m], What_1[m] = -Psi[m+e2],
+    //    What_2[m] = Psi[m+e1]  (eq:xjdot_Final in c = 1 units, self pair excluded);
+    //    the columns m of one (target, component) are split over q lanes
+    const int q = min(32, NT / (2 * TG));
+    if (threadIdx.x < 2 * TG * q) {  // whole warps: 2 TG q is a multiple of 32 here
+      const int part = threadIdx.x % q, tt = (threadIdx.x / q) >> 1, comp = (threadIdx.x / q) & 1;
+      double acc = 0.0;
+      for (int col = part; col < K; col += q) {
+        int s = 0;
+        while (tri(s + 1) <= col) ++s;
+        const int m2 = col - tri(s), m1 = s - m2;
+        const double a = ((s & 1) == comp) ? -at[col * TG + tt] : at[col * TG + tt];
+        acc = fma(a, psi[(comp == 0 ? bcol(m1, m2 + 1) : bcol(m1 + 1, m2)) * TG + tt], acc);
+      }
+      for (int o = q >> 1; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+      if (part == 0) X[2 * tt + comp] = acc;
+    }
+    __syncthreads();
+  } else if (threadIdx.x < 2 * TG) {
+    X[threadIdx.x] = 0.0;
   }
-  __syncthreads();
-  // 3. add the self pair: Psi_self[beta] = sum_m a_m psi0[m + beta]
-  for (int idx = threadIdx.x; idx < TB * NB; idx += blockDim.x) {
-    const int tt = idx / NB, b = idx % NB;
+  // 3. add the self pair: Psi_self[beta] = sum_m a_m psi0[m + beta] (psi0
+  //    vanishes at odd indices: only m of the parity of beta contribute)
+  for (int idx = threadIdx.x; idx < TG * NB; idx += NT) {
+    const int tt = idx % TG, b = idx / TG;
     int bn = 1;
     while (tri(bn + 1) - 1 <= b) ++bn;
     const int b2 = b + 1 - tri(bn), b1 = bn - b2;
     double acc = 0.0;
-    int col = 0;
-    for (int s = 0; s <= M; ++s) {
-      for (int m2 = 0; m2 <= s; ++m2, ++col) {
-        const int a1 = s - m2 + b1, a2 = m2 + b2;
-        if ((a1 | a2) & 1) continue;  // psi0 vanishes at odd indices
-        acc += at[tt * K + col] * A.psi0[tri(a1 + a2) + a2];
+    for (int m1 = b1 & 1; m1 <= M; m1 += 2)
+      for (int m2 = b2 & 1; m1 + m2 <= M; m2 += 2) {
+        const int a2 = m2 + b2;
+        acc = fma(at[mcol(m1, m2) * TG + tt], __ldg(A.tab.psi0 + tri(m1 + b1 + a2) + a2), acc);
       }
-    }
-    psi[idx] += acc;
+    psi[b * TG + tt] += acc;
   }
   __syncthreads();
-  // 4. moment equation and centroid velocity per (target, k)
-  for (int idx = threadIdx.x; idx < TB * K; idx += blockDim.x) {
-    const int tt = idx / K, k = idx % K, p = j0 + tt;
+  // 4. the table: sum_l a_l (sum_beta c Psi[beta]) over each piece
+  {
+    const int tt = threadIdx.x % TG, np = A.tab.np;
+    const double* ps = psi + tt;
+    const double* a = at + tt;
+    for (int p = p0 + threadIdx.x / TG; p < p1; p += NT / TG) {
+      const int len = __ldg(A.tab.piece_len + p);
+      const double2* e = reinterpret_cast<const double2*>(A.tab.tab) + p;
+      double R = 0.0, g = 0.0;
+#pragma unroll 4
+      for (int j = 0; j < len; ++j) {
+        const double2 v = __ldg(e + (size_t)j * np);  // (c, packed b and l)
+        const long long bl = __double_as_longlong(v.y);
+        const int b = (int)(bl & 0xffffffffll), l = (int)(bl >> 32);
+        g = fma(v.x, ps[b * TG], g);
+        if (l >= 0) {
+          R = fma(a[l * TG], g, R);
+          g = 0.0;
+        }
+      }
+      pres[(p - p0) * TG + tt] = R;
+    }
+  }
+  __syncthreads();
+  // 5. moment equation and stage update per (target, k)
+  const int nk = k1 - k0;
+  for (int idx = threadIdx.x; idx < TG * nk; idx += NT) {
+    const int tt = idx / nk, k = k0 + idx % nk, p = j0 + tt;
     if (p >= A.n) continue;
     const int j = A.perm ? A.perm[p] : p;
     int kn = 0;
-    while ((kn + 1) * (kn + 2) / 2 <= k) ++kn;
-    const int k2 = k - tri(kn), k1 = kn - k2;
-    const double* a = at + tt * K;
-    const double* ps = psi + tt * NB;
+    while (tri(kn + 1) <= k) ++kn;
+    const int k2 = k - tri(kn), k1c = kn - k2;
     double R = 0.0;
-    for (int e = A.k_off[k]; e < A.k_off[k + 1]; ++e) R += A.e_c[e] * a[A.e_l[e]] * ps[A.e_b[e]];
-    const double m00 = m00s[tt];
+    for (int e = A.tab.row_off[k]; e < A.tab.row_off[k + 1]; ++e) R += pres[(e - p0) * TG + tt];
     double ctr = 0.0;
-    if (k1 >= 1) ctr += X[2 * tt] * a[mcol(k1 - 1, k2)];
-    if (k2 >= 1) ctr += X[2 * tt + 1] * a[mcol(k1, k2 - 1)];
-    const double dm = (R + ctr / m00) / (cpow[kn] * c);  // c^{|k|/2 - 1}
+    if (k1c >= 1) ctr += X[2 * tt] * at[mcol(k1c - 1, k2) * TG + tt];
+    if (k2 >= 1) ctr += X[2 * tt + 1] * at[mcol(k1c, k2 - 1) * TG + tt];
+    const double dm = (R + ctr / m00s[tt]) / (cpow[kn] * c);  // c^{|k|/2 - 1}
     const size_t o = (size_t)j * K + k;
     if (A.mode == 0) {
       A.out_dM[o] = dm;
@@ -309,12 +354,13 @@ __device__ __forceinline__ void finish_block(const FinishArgs& A, int j0, double
       if (A.mode == 4) { A.y_M[o] = A.sum_M[o] + h / 6.0 * dm; }
     }
   }
-  // 5. centroid velocity xdot_c = c^{-1/2} X_c / M_00 and its stage update
-  for (int idx = threadIdx.x; idx < TB * 2; idx += blockDim.x) {
+  // 6. centroid velocity xdot_c = c^{-1/2} X_c / M_00 and its stage update
+  if (k0 != 0) return;
+  for (int idx = threadIdx.x; idx < TG * 2; idx += NT) {
     const int tt = idx >> 1, comp = idx & 1, p = j0 + tt;
     if (p >= A.n) continue;
     const int j = A.perm ? A.perm[p] : p;
-    const double dx = X[idx] * cpow[1] / m00s[tt];
+    const double dx = X[idx] / (sqrt(c) * m00s[tt]);
     const size_t ox = (size_t)j * 2 + comp;
     if (A.mode == 0) {
       A.out_dx[ox] = dx;
@@ -329,9 +375,15 @@ __device__ __forceinline__ void finish_block(const FinishArgs& A, int j0, double
   }
 }
 
-__global__ void finish_kernel(FinishArgs A) {
+constexpr int kFinishThreads = 256;
+
+// Grid: (target blocks, row blocks); row blocks are used for n == 1 only.
+template <int TG>
+__global__ void __launch_bounds__(kFinishThreads) finish_kernel(FinishArgs A) {
   extern __shared__ double sm[];
-  finish_block(A, blockIdx.x * A.targets_per_block, sm);  // sorted positions
+  const bool split = gridDim.y > 1;
+  finish_block<TG>(A, blockIdx.x * TG, split ? A.tab.rb_off[blockIdx.y] : 0,
+                   split ? A.tab.rb_off[blockIdx.y + 1] : A.K, sm);
 }
 
 __global__ void advance_time_kernel(double* t_dev, const double* dt_dev) {
@@ -407,8 +459,9 @@ __global__ void prep_batch_kernel(int M, int K, int R, const BatchInst* __restri
 }
 
 // Finish of every instance of a batch: item (instance, first target) per
-// block of TB targets; blocks loop over the items.
-__global__ void finish_batch_kernel(BatchFinishArgs B) {
+// block of TG targets; blocks loop over the items.
+template <int TG>
+__global__ void __launch_bounds__(kFinishThreads) finish_batch_kernel(BatchFinishArgs B) {
   extern __shared__ double sm[];
   const int total = *B.n_items;
   for (int it = blockIdx.x; it < total; it += gridDim.x) {
@@ -421,15 +474,10 @@ __global__ void finish_batch_kernel(BatchFinishArgs B) {
     A.K = B.K;
     A.NB = B.NB;
     A.nchunks = I.n > 1 ? I.chunks : 0;
-    A.targets_per_block = B.targets_per_block;
     A.partial = I.n > 1 ? B.partial + I.part_off : nullptr;
     A.perm = B.perm_local ? B.perm_local + I.slot0 : nullptr;
     A.Min = inst_stage_m(I, B.K, B.src);
-    A.k_off = B.k_off;
-    A.e_l = B.e_l;
-    A.e_b = B.e_b;
-    A.e_c = B.e_c;
-    A.psi0 = B.psi0;
+    A.tab = B.tab;
     A.lam0sq = I.lam0sq;
     A.four_nu = I.four_nu;
     A.t_dev = &I.t;
@@ -442,7 +490,7 @@ __global__ void finish_batch_kernel(BatchFinishArgs B) {
     A.ys_M = I.state + blk + 2 * (size_t)I.n;
     A.sum_x = I.state + 2 * blk;
     A.sum_M = I.state + 2 * blk + 2 * (size_t)I.n;
-    finish_block(A, w.y, sm);
+    finish_block<TG>(A, w.y, 0, B.K, sm);
     __syncthreads();  // shared memory is reused by the next item
   }
 }
@@ -495,20 +543,40 @@ cudaError_t launch_prep_batch(int precision, int M, const BatchInst* inst, const
   return cudaGetLastError();
 }
 
-size_t finish_smem_bytes(int M, int targets_per_block) {
-  const int K = n_moments(M), NB = n_beta(M);
-  return sizeof(double) * ((size_t)targets_per_block * (NB + K + 3) + 2 * M + 3);
+// Shared memory of a finish CTA of TG targets and np pieces.
+size_t finish_smem_bytes(int M, int TG, int np) {
+  return sizeof(double) * ((size_t)TG * (n_beta(M) + n_moments(M) + 3 + np) + M + 1);
 }
 
-cudaError_t launch_finish_batch(const BatchFinishArgs& B, int grid, cudaStream_t st) {
-  const size_t smem = finish_smem_bytes(B.M, B.targets_per_block);
-  if (smem > 48 * 1024) {
-    cudaError_t e = cudaFuncSetAttribute(finish_batch_kernel,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
+// Call f(kernel of TG targets) for the run-time TG in {1, 4, 8, 16, 32}.
+template <typename F>
+cudaError_t with_targets(int TG, F&& f) {
+  switch (TG) {
+    case 1: return f(std::integral_constant<int, 1>{});
+    case 4: return f(std::integral_constant<int, 4>{});
+    case 8: return f(std::integral_constant<int, 8>{});
+    case 16: return f(std::integral_constant<int, 16>{});
+    default: return f(std::integral_constant<int, 32>{});
   }
-  finish_batch_kernel<<<std::max(1, grid), 128, smem, st>>>(B);
-  return cudaGetLastError();
+}
+
+// Targets per batch item: instances of 64 to 8192 particles give 8-target
+// items enough CTAs; orders above the pair limit hold one particle.
+int finish_batch_targets(int M) { return M > 8 ? 1 : 8; }
+
+cudaError_t launch_finish_batch(const BatchFinishArgs& B, int grid, cudaStream_t st) {
+  const int TG = finish_batch_targets(B.M);
+  const size_t smem = finish_smem_bytes(B.M, TG, B.tab.np);
+  return with_targets(TG, [&](auto tg) {
+    constexpr int T = decltype(tg)::value;
+    if (smem > 48 * 1024) {
+      cudaError_t e = cudaFuncSetAttribute(
+          finish_batch_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+      if (e != cudaSuccess) return e;
+    }
+    finish_batch_kernel<T><<<std::max(1, grid), kFinishThreads, smem, st>>>(B);
+    return cudaGetLastError();
+  });
 }
 
 cudaError_t launch_advance_batch(BatchInst* inst, const int* n_inst, int max_inst,
@@ -557,17 +625,29 @@ cudaError_t launch_prep(int precision, int n, int M, const int* perm, const doub
   return cudaGetLastError();
 }
 
-cudaError_t launch_finish(const FinishArgs& A, cudaStream_t st) {
-  const int TB = A.targets_per_block;
-  const size_t smem = sizeof(double) * ((size_t)TB * (A.NB + A.K + 3) + 2 * A.M + 3);
-  if (smem > 48 * 1024) {
-    cudaError_t e = cudaFuncSetAttribute(finish_kernel,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-  }
-  const int blocks = (A.n + TB - 1) / TB;
-  finish_kernel<<<blocks, 128, smem, st>>>(A);
-  return cudaGetLastError();
+// Targets per finish CTA: the largest of 32, 16, 8, 4, 1 that still gives 4
+// CTAs per SM (the FP64 pipe of every SM then has work to the end).
+int finish_targets(int n, int sms) {
+  for (int TG : {32, 16, 8, 4})
+    if ((n + TG - 1) / TG >= 4 * sms) return TG;
+  return 1;
+}
+
+cudaError_t launch_finish(const FinishArgs& A, int sms, cudaStream_t st) {
+  const int TG = finish_targets(A.n, sms);
+  const int rb = A.n == 1 ? A.tab.nrb : 1;
+  // row blocks hold a part of the pieces each; the bound covers any of them
+  const size_t smem = finish_smem_bytes(A.M, TG, A.tab.np);
+  return with_targets(TG, [&](auto tg) {
+    constexpr int T = decltype(tg)::value;
+    if (smem > 48 * 1024) {
+      cudaError_t e = cudaFuncSetAttribute(
+          finish_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+      if (e != cudaSuccess) return e;
+    }
+    finish_kernel<T><<<dim3((A.n + T - 1) / T, rb), kFinishThreads, smem, st>>>(A);
+    return cudaGetLastError();
+  });
 }
 
 cudaError_t launch_advance_time(double* t_dev, const double* dt_dev, cudaStream_t st) {

@@ -6,23 +6,19 @@
 #include <vector>
 
 #include "common.cuh"
+#include "tables.h"
 
 namespace mmvm {
 
 struct FinishArgs {
   int n = 0, M = 0, K = 0, NB = 0;
   int nchunks = 0;                  // number of pair partials (0: single particle)
-  int targets_per_block = 1;
   const double* partial = nullptr;  // [nchunks][NB][n] by sorted position
   const double* fpart = nullptr;    // far-field blocks [nfar][n_edge][n] (list form; nullable):
   int nfar = 0, n_edge = 0;         // edge column e = 2 (|beta| - 1) + beta1, beta1 <= 1
   const int* perm = nullptr;        // sorted position -> particle (null: identity)
   const double* Min = nullptr;      // stage moments (n x K)
-  const int* k_off = nullptr;       // finish tables (tables.h)
-  const int* e_l = nullptr;
-  const int* e_b = nullptr;
-  const double* e_c = nullptr;
-  const double* psi0 = nullptr;
+  FinishTab tab;                    // finish tables (tables.h)
   double lam0sq = 0, four_nu = 0;   // lambda^2 = lam0sq + four_nu * t
   const double* t_dev = nullptr;    // step start time
   const double* dt_dev = nullptr;   // step size (null: 0)
@@ -39,21 +35,16 @@ struct FinishArgs {
 };
 
 // Finish of a batch of one order (see BatchInst): items (instance, first
-// target) of targets_per_block targets each; src selects the stage input
+// target) of finish_batch_targets(M) targets each; src selects the stage input
 // (0: y, 1: ys); mode 1..4 is the RK4 stage (mode 0 is not used by batches).
 struct BatchFinishArgs {
   int M = 0, K = 0, NB = 0;
-  int targets_per_block = 1;
   const BatchInst* inst = nullptr;
   const int2* items = nullptr;
   const int* n_items = nullptr;     // device count of items
   const double* partial = nullptr;  // the batch's partials (BatchInst::part_off)
   const int* perm_local = nullptr;  // batch order (null: identity)
-  const int* k_off = nullptr;       // finish tables of the order (tables.h)
-  const int* e_l = nullptr;
-  const int* e_b = nullptr;
-  const double* e_c = nullptr;
-  const double* psi0 = nullptr;
+  FinishTab tab;                    // finish tables of the order (tables.h)
   int src = 0;
   double cs = 0;
   int mode = 1;
@@ -73,7 +64,7 @@ cudaError_t launch_batch_order(int slot_cap, const int* n_slots, const BatchInst
                                unsigned long long* kin, unsigned long long* kout, int* iin,
                                int* iout, void* temp, size_t temp_bytes, int* perm_local,
                                cudaStream_t st);
-size_t finish_smem_bytes(int M, int targets_per_block);
+int finish_batch_targets(int M);  // targets per item of launch_finish_batch
 // flags[i] = 1 if instance i's step-start state holds a non-finite value.
 cudaError_t launch_scan_batch(int M, const BatchInst* inst, const int* n_inst, int max_inst,
                               int* flags, cudaStream_t st);
@@ -146,7 +137,9 @@ cudaError_t launch_group_multipole(int M, int n, const void* rec, void* gdata,
 size_t spatial_order_temp_bytes(int n);
 cudaError_t launch_spatial_order(int n, const double* x, void* temp, size_t temp_bytes,
                                  int* perm, cudaStream_t st);
-cudaError_t launch_finish(const FinishArgs& A, cudaStream_t st);
+// sms: multiprocessors of the device (sets the targets per CTA).  In modes 1-3
+// A.Min must not alias A.ys_M when n == 1 (several CTAs share the particle).
+cudaError_t launch_finish(const FinishArgs& A, int sms, cudaStream_t st);
 cudaError_t launch_advance_time(double* t_dev, const double* dt_dev, cudaStream_t st);
 cudaError_t launch_scan(int n, int K, const double* x, const double* mom, int* flags,
                         cudaStream_t st);

@@ -85,8 +85,6 @@ int chunk_len_for(int64_t n, int chunks) {
   return mmvm::round_up((int)((n + chunks - 1) / chunks), kGroup);
 }
 
-int finish_tb(int K) { return std::max(1, 128 / (((K + 31) / 32) * 32)); }
-
 int size_class(int64_t n) { return n <= 256 ? 0 : n <= 1024 ? 1 : n <= 4096 ? 2 : 3; }
 
 size_t rec_bytes(int M, int precision) {
@@ -159,8 +157,8 @@ struct Batch {
   std::vector<Request*> incoming;  // admitted, state on its way, joining at the next tick
   bool dirty = true;
   bool tuned = false;
-  DBuf<int> k_off, e_l, e_b;
-  DBuf<double> e_c, psi0;
+  DBuf<unsigned char> ftab;  // finish tables (blob of tables.h)
+  mmvm::FinishTab ft;
   DBuf<unsigned char> rec;
   DBuf<double> partial;
   DBuf<BatchInst> inst;
@@ -185,10 +183,8 @@ struct Batch {
   int grid = 1;               // persistent CTAs of the pair kernel
   int64_t pairs_per_rhs = 0;  // sum of n^2 over the members
   void release() {
-    for (auto* b : {&k_off, &e_l, &e_b, &slot_inst, &counts, &bad, &perm, &iin, &iout})
-      b->release();
-    e_c.release();
-    psi0.release();
+    for (auto* b : {&slot_inst, &counts, &bad, &perm, &iin, &iout}) b->release();
+    ftab.release();
     rec.release();
     partial.release();
     inst.release();
@@ -256,23 +252,14 @@ void finish_request(mmvm_server* s, Request* r, int status, const std::string& e
 
 cudaError_t upload_tables(Batch& b) {
   mmvm::FinishTables T = mmvm::build_finish_tables(b.M);
+  const std::vector<unsigned char> tb = T.blob();
   bool g = false;
   cudaError_t e;
-  if ((e = b.k_off.ensure(T.k_off.size(), &g)) != cudaSuccess ||
-      (e = b.e_l.ensure(std::max<size_t>(T.e_l.size(), 1), &g)) != cudaSuccess ||
-      (e = b.e_b.ensure(std::max<size_t>(T.e_b.size(), 1), &g)) != cudaSuccess ||
-      (e = b.e_c.ensure(std::max<size_t>(T.e_c.size(), 1), &g)) != cudaSuccess ||
-      (e = b.psi0.ensure(T.psi0.size(), &g)) != cudaSuccess)
+  if ((e = b.ftab.ensure(tb.size(), &g)) != cudaSuccess ||
+      (e = cudaMemcpyAsync(b.ftab.p, tb.data(), tb.size(), cudaMemcpyHostToDevice, b.st)) !=
+          cudaSuccess)
     return e;
-  auto up = [&](void* d, const void* h, size_t bytes) {
-    return bytes ? cudaMemcpyAsync(d, h, bytes, cudaMemcpyHostToDevice, b.st) : cudaSuccess;
-  };
-  if ((e = up(b.k_off.p, T.k_off.data(), T.k_off.size() * sizeof(int))) != cudaSuccess ||
-      (e = up(b.e_l.p, T.e_l.data(), T.e_l.size() * sizeof(int))) != cudaSuccess ||
-      (e = up(b.e_b.p, T.e_b.data(), T.e_b.size() * sizeof(int))) != cudaSuccess ||
-      (e = up(b.e_c.p, T.e_c.data(), T.e_c.size() * sizeof(double))) != cudaSuccess ||
-      (e = up(b.psi0.p, T.psi0.data(), T.psi0.size() * sizeof(double))) != cudaSuccess)
-    return e;
+  b.ft = mmvm::finish_tab(T, b.ftab.p);
   return cudaStreamSynchronize(b.st);  // the host tables go out of scope
 }
 
@@ -421,17 +408,12 @@ cudaError_t enqueue_batch_step(const mmvm_server* s, Batch& b) {
     B.M = b.M;
     B.K = b.K;
     B.NB = b.NB;
-    B.targets_per_block = b.tb;
     B.inst = b.inst.p;
     B.items = b.fitems.p;
     B.n_items = b.counts.p + 2;
     B.partial = b.partial.p;
     B.perm_local = far ? b.perm.p : nullptr;
-    B.k_off = b.k_off.p;
-    B.e_l = b.e_l.p;
-    B.e_b = b.e_b.p;
-    B.e_c = b.e_c.p;
-    B.psi0 = b.psi0.p;
+    B.tab = b.ft;
     B.src = src;
     B.cs = cs[stage - 1];
     B.mode = stage;
@@ -540,7 +522,7 @@ Batch& batch_of(mmvm_server* s, int M, int64_t n, cudaError_t* e) {
   b.M = M;
   b.K = mmvm::n_moments(M);
   b.NB = mmvm::n_beta(M);
-  b.tb = finish_tb(b.K);
+  b.tb = mmvm::finish_batch_targets(M);
   b.pe = mmvm::PairEntry();
   if (M <= MMVM_MAX_ORDER_PAIRS) {
     b.pe = mmvm::pair_entry(M, s->cfg.precision, 0);

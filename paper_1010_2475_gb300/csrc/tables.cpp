@@ -2,6 +2,7 @@
 #include "tables.h"
 
 #include <algorithm>
+#include <cstring>
 #include <map>
 #include <tuple>
 
@@ -31,7 +32,98 @@ long double pow4l(int e) {
   return r;
 }
 
+// Pieces, their interleaved layout and the row blocks of t from the rows'
+// entries (FinEntry::l holds the group on entry).
+void cut_rows(FinishTables& t, const std::vector<std::vector<FinEntry>>& rows) {
+  size_t total = 0;
+  for (const auto& r : rows) total += r.size();
+  // ~128 pieces keep the threads of a CTA busy; longer rows of the high
+  // orders get more pieces instead of longer ones
+  const size_t piece = std::min<size_t>(std::max<size_t>(total / 128, 8), 96);
+  std::vector<std::vector<FinEntry>> ps;
+  t.row_off.assign(1, 0);
+  for (const auto& r : rows) {
+    const size_t cnt = (r.size() + piece - 1) / piece;
+    for (size_t i = 0; i < cnt; ++i) {
+      const size_t e0 = i * r.size() / cnt, e1 = (i + 1) * r.size() / cnt;
+      std::vector<FinEntry> p(r.begin() + e0, r.begin() + e1);
+      for (size_t e = 0; e + 1 < p.size(); ++e)
+        if (p[e].l == p[e + 1].l) p[e].l = -1;  // only the last entry of a group closes it
+      ps.push_back(std::move(p));
+    }
+    t.row_off.push_back((int)ps.size());
+  }
+  t.np = (int)ps.size();
+  size_t plen = 0;
+  for (const auto& p : ps) plen = std::max(plen, p.size());
+  t.tab.assign(plen * ps.size(), FinEntry{0.0, 0, -1});
+  t.piece_len.clear();
+  for (size_t p = 0; p < ps.size(); ++p) {
+    t.piece_len.push_back((int)ps[p].size());
+    for (size_t j = 0; j < ps[p].size(); ++j) t.tab[j * ps.size() + p] = ps[p][j];
+  }
+  // row blocks of ~1500 entries: a CTA's threads then hold a few entries each
+  const int want = (int)std::min<size_t>(std::max<size_t>(total / 1500, 1), 64);
+  t.rb_off.assign(1, 0);
+  size_t run = 0;
+  for (int k = 0; k < t.K; ++k) {
+    run += rows.size() ? rows[k].size() : 0;
+    if (run * want >= total * t.rb_off.size() && (int)t.rb_off.size() < want)
+      t.rb_off.push_back(k + 1);
+  }
+  if (t.rb_off.back() != t.K) t.rb_off.push_back(t.K);
+  t.nrb = (int)t.rb_off.size() - 1;
+}
+
+struct BlobOffsets {
+  size_t tab, piece_len, row_off, rb_off, psi0, bytes;
+};
+BlobOffsets blob_offsets(const FinishTables& t) {
+  BlobOffsets o;
+  size_t off = 0;
+  auto take = [&](size_t bytes) {
+    const size_t at = off;
+    off = (off + bytes + 255) & ~(size_t)255;
+    return at;
+  };
+  o.tab = take(t.tab.size() * sizeof(FinEntry));
+  o.piece_len = take(t.piece_len.size() * sizeof(int));
+  o.row_off = take(t.row_off.size() * sizeof(int));
+  o.rb_off = take(t.rb_off.size() * sizeof(int));
+  o.psi0 = take(t.psi0.size() * sizeof(double));
+  o.bytes = off;
+  return o;
+}
+
 }  // namespace
+
+std::vector<unsigned char> FinishTables::blob() const {
+  const BlobOffsets o = blob_offsets(*this);
+  std::vector<unsigned char> b(o.bytes, 0);
+  auto put = [&](size_t at, const void* src, size_t bytes) {
+    if (bytes) std::memcpy(b.data() + at, src, bytes);
+  };
+  put(o.tab, tab.data(), tab.size() * sizeof(FinEntry));
+  put(o.piece_len, piece_len.data(), piece_len.size() * sizeof(int));
+  put(o.row_off, row_off.data(), row_off.size() * sizeof(int));
+  put(o.rb_off, rb_off.data(), rb_off.size() * sizeof(int));
+  put(o.psi0, psi0.data(), psi0.size() * sizeof(double));
+  return b;
+}
+
+FinishTab finish_tab(const FinishTables& t, const void* base) {
+  const BlobOffsets o = blob_offsets(t);
+  const unsigned char* p = static_cast<const unsigned char*>(base);
+  FinishTab f;
+  f.tab = reinterpret_cast<const FinEntry*>(p + o.tab);
+  f.piece_len = reinterpret_cast<const int*>(p + o.piece_len);
+  f.row_off = reinterpret_cast<const int*>(p + o.row_off);
+  f.rb_off = reinterpret_cast<const int*>(p + o.rb_off);
+  f.psi0 = reinterpret_cast<const double*>(p + o.psi0);
+  f.np = t.np;
+  f.nrb = t.nrb;
+  return f;
+}
 
 FinishTables build_finish_tables(int M, bool entries) {
   FinishTables t;
@@ -39,7 +131,7 @@ FinishTables build_finish_tables(int M, bool entries) {
   t.K = n_moments(M);
   t.NB = n_beta(M);
   t.NJ = jet_order(M);
-  t.k_off.assign(t.K + 1, 0);
+  std::vector<std::vector<FinEntry>> rows(t.K);  // entries by row, grouped by l
   for (int kn = 0, kcol = 0; entries && kn <= M; ++kn) {
     for (int k2 = 0; k2 <= kn; ++k2, ++kcol) {
       const int k1 = kn - k2;
@@ -73,13 +165,11 @@ FinishTables build_finish_tables(int M, bool entries) {
       }
       for (auto& kv : acc) {
         if (kv.second == 0.0L) continue;
-        t.e_l.push_back(kv.first.first);
-        t.e_b.push_back(kv.first.second);
-        t.e_c.push_back((double)kv.second);
+        rows[kcol].push_back({(double)kv.second, kv.first.second, kv.first.first});
       }
-      t.k_off[kcol + 1] = (int)t.e_l.size();
     }
   }
+  cut_rows(t, rows);
   // psi0 (jet of the Gaussian-vortex stream function at the origin, c = 1)
   t.psi0.assign(tri(t.NJ + 1), 0.0);
   const long double inv4pi = 0.0795774715459476678844418816862571810L;

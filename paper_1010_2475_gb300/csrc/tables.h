@@ -26,14 +26,41 @@
 
 namespace mmvm {
 
+// One (k, l, beta) entry.  The entries of a row k are grouped by l, so that a
+// row is sum_l a_l (sum_beta c Psi[beta]): one multiply-add per entry and one
+// per (k, l) group.
+struct FinEntry {
+  double c;  // coefficient
+  int b;     // Psi column beta (bcol)
+  int l;     // moment column l on the last entry of a group, else -1
+};
+
+// The rows are cut into pieces of similar length (whole groups or parts of
+// one), one thread sums a piece.  Entry j of piece p sits at tab[j * np + p],
+// so threads on neighbouring pieces read neighbouring entries; row k owns the
+// pieces [row_off[k], row_off[k + 1]).  Row blocks [rb_off[i], rb_off[i + 1])
+// split the rows of a single particle over several CTAs (similar entry counts).
 struct FinishTables {
   int M = 0, K = 0, NB = 0, NJ = 0;
-  std::vector<int> k_off;    // K+1 offsets into the entry arrays, grouped by k
-  std::vector<int> e_l;      // moment column l
-  std::vector<int> e_b;      // Psi column beta (bcol)
-  std::vector<double> e_c;   // coefficient
-  std::vector<double> psi0;  // psi0 for |alpha| <= NJ, column q(|alpha|) + alpha_2
+  int np = 0, nrb = 1;
+  std::vector<FinEntry> tab;
+  std::vector<int> piece_len;  // np
+  std::vector<int> row_off;    // K + 1
+  std::vector<int> rb_off;     // nrb + 1
+  std::vector<double> psi0;    // psi0 for |alpha| <= NJ, column q(|alpha|) + alpha_2
+  std::vector<unsigned char> blob() const;  // all of them, 256-byte aligned parts
 };
+
+// Device view of a blob() copied to `base`.
+struct FinishTab {
+  const FinEntry* tab = nullptr;
+  const int* piece_len = nullptr;
+  const int* row_off = nullptr;
+  const int* rb_off = nullptr;
+  const double* psi0 = nullptr;
+  int np = 0, nrb = 1;
+};
+FinishTab finish_tab(const FinishTables& t, const void* base);
 
 // entries = false leaves out the (k, l, beta) entries (their number grows
 // like M^6; the separable single-particle path does not use them).
