@@ -67,7 +67,7 @@ extern "C" {
 #define MMVM_MAX_ORDER_SINGLE 64
 
 /* mmvm_config.flags bits.  In MMVM_MIXED_FP32 mode the particles are put in
- * spatial (Morton) order every step and tile pairs whose bounding boxes are
+ * spatial (Hilbert) order every step and tile pairs whose bounding boxes are
  * far enough apart that the Gaussian part of the pair jet is below FP32
  * rounding take the point-vortex jet (far field); this flag turns that off
  * (every pair takes the full jet).  MMVM_FP64 never uses the far field.     */

@@ -1,10 +1,14 @@
 // Spatial ordering of the particles for the all-pairs kernel: consecutive
 // positions are close in space, so the 32-particle groups (source tiles and
 // target warps) have small bounding boxes and the far-field test of the pair
-// kernel can take the point-vortex jet for whole tiles.  Morton (Z-order)
-// keys of the centres quantised to 16 bits per axis over the bounding box,
-// sorted with a stable radix sort (ties keep the index order), so the order
-// is deterministic.
+// kernel can take the point-vortex jet for whole tiles.  Keys: the position
+// along a Hilbert curve of the centres quantised to 16 bits per axis over the
+// bounding square, sorted with a stable radix sort (ties keep the index
+// order), so the order is deterministic.  Neighbours on a Hilbert curve are
+// always neighbours in the plane; a Z-order curve jumps across the plane, and
+// the groups that straddle a jump have boxes many times larger (two patches,
+// n = 65536: median group radius 0.60 core units against 1.06, mean box area
+// 0.88 against 1.96).
 #include <cub/device/device_radix_sort.cuh>
 
 #include <algorithm>
@@ -16,6 +20,33 @@ namespace mmvm {
 
 namespace {
 
+// Distance along the order-16 Hilbert curve of the cell (x, y), both below
+// 2^16: per level the quadrant's rank along the curve, then the rotation or
+// reflection that maps the quadrant's curve onto the parent's.
+__device__ __forceinline__ unsigned hilbert16(unsigned x, unsigned y) {
+  unsigned d = 0;
+#pragma unroll
+  for (int b = 15; b >= 0; --b) {
+    const unsigned rx = (x >> b) & 1u, ry = (y >> b) & 1u;
+    d = (d << 2) | ((3u * rx) ^ ry);
+    if (!ry) {
+      if (rx) {
+        x = 65535u - x;
+        y = 65535u - y;
+      }
+      const unsigned t = x;
+      x = y;
+      y = t;
+    }
+  }
+  return d;
+}
+
+// Morton (Z-order) code of a centre, each axis scaled to its own extent: the
+// server's order.  Its batched kernel gains 2 % from the Hilbert order, which
+// is less than what a change of summation order moves in the results of long
+// served runs (1e-9 relative after 4 steps of an order-8 disk), so served
+// results keep the order they always had.
 __device__ __forceinline__ unsigned spread16(unsigned v) {
   v &= 0xffffu;
   v = (v | (v << 8)) & 0x00ff00ffu;
@@ -23,6 +54,21 @@ __device__ __forceinline__ unsigned spread16(unsigned v) {
   v = (v | (v << 2)) & 0x33333333u;
   v = (v | (v << 1)) & 0x55555555u;
   return v;
+}
+__device__ __forceinline__ unsigned morton_key(double x1, double x2, const double4 b) {
+  const double s1 = fmax(b.z - b.x, 1e-300), s2 = fmax(b.w - b.y, 1e-300);
+  const double q1 = fmin(fmax((x1 - b.x) / s1, 0.0), 1.0) * 65535.0;
+  const double q2 = fmin(fmax((x2 - b.y) / s2, 0.0), 1.0) * 65535.0;
+  return spread16((unsigned)q1) | (spread16((unsigned)q2) << 1);
+}
+
+// Hilbert key of the centre (x1, x2) in the box (min1, min2, max1, max2).
+__device__ __forceinline__ unsigned order_key(double x1, double x2, double lo1, double lo2,
+                                              double hi1, double hi2) {
+  const double s = fmax(fmax(hi1 - lo1, hi2 - lo2), 1e-300);
+  const double q1 = fmin(fmax((x1 - lo1) / s, 0.0), 1.0) * 65535.0;
+  const double q2 = fmin(fmax((x2 - lo2) / s, 0.0), 1.0) * 65535.0;
+  return hilbert16((unsigned)q1, (unsigned)q2);
 }
 
 // One block: bounding box of all centres -> box[0..3] = (min1, min2, max1, max2).
@@ -71,14 +117,11 @@ __global__ void bbox_kernel(int n, const double* __restrict__ x, double* __restr
   }
 }
 
-__global__ void morton_kernel(int n, const double* __restrict__ x, const double* __restrict__ box,
+__global__ void keys_kernel(int n, const double* __restrict__ x, const double* __restrict__ box,
                               unsigned* __restrict__ keys, int* __restrict__ idx) {
   const int j = blockIdx.x * blockDim.x + threadIdx.x;
   if (j >= n) return;
-  const double s1 = fmax(box[2] - box[0], 1e-300), s2 = fmax(box[3] - box[1], 1e-300);
-  const double q1 = fmin(fmax((x[2 * j] - box[0]) / s1, 0.0), 1.0) * 65535.0;
-  const double q2 = fmin(fmax((x[2 * j + 1] - box[1]) / s2, 0.0), 1.0) * 65535.0;
-  keys[j] = spread16((unsigned)q1) | (spread16((unsigned)q2) << 1);
+  keys[j] = order_key(x[2 * j], x[2 * j + 1], box[0], box[1], box[2], box[3]);
   idx[j] = j;
 }
 
@@ -141,7 +184,7 @@ __global__ void bbox_batch_kernel(const BatchInst* __restrict__ inst, const int*
 // Key of slot p: (instance << 32) | Morton code in the instance's own box;
 // padding slots of an instance sort after its particles, slots past the
 // batch after everything.
-__global__ void morton_batch_kernel(int slot_cap, const int* __restrict__ n_slots,
+__global__ void keys_batch_kernel(int slot_cap, const int* __restrict__ n_slots,
                                     const BatchInst* __restrict__ inst,
                                     const int* __restrict__ slot_inst,
                                     const double4* __restrict__ ibox,
@@ -155,11 +198,7 @@ __global__ void morton_batch_kernel(int slot_cap, const int* __restrict__ n_slot
       const int j = p - I.slot0;
       unsigned code = 0xffffffffu;
       if (j < I.n) {
-        const double4 b = ibox[i];
-        const double s1 = fmax(b.z - b.x, 1e-300), s2 = fmax(b.w - b.y, 1e-300);
-        const double q1 = fmin(fmax((I.state[2 * j] - b.x) / s1, 0.0), 1.0) * 65535.0;
-        const double q2 = fmin(fmax((I.state[2 * j + 1] - b.y) / s2, 0.0), 1.0) * 65535.0;
-        code = spread16((unsigned)q1) | (spread16((unsigned)q2) << 1);
+        code = morton_key(I.state[2 * j], I.state[2 * j + 1], ibox[i]);
       }
       key = ((unsigned long long)i << 32) | code;
     }
@@ -201,7 +240,7 @@ cudaError_t launch_batch_order(int slot_cap, const int* n_slots, const BatchInst
   bbox_batch_kernel<<<std::max(1, std::min(inst_cap, 1024)), 256, 0, st>>>(
       inst, n_inst, static_cast<double4*>(ibox));
   const int blocks = std::max(1, std::min((slot_cap + 255) / 256, 4096));
-  morton_batch_kernel<<<blocks, 256, 0, st>>>(slot_cap, n_slots, inst, slot_inst,
+  keys_batch_kernel<<<blocks, 256, 0, st>>>(slot_cap, n_slots, inst, slot_inst,
                                               static_cast<const double4*>(ibox), kin, iin);
   cudaError_t e = cub::DeviceRadixSort::SortPairs(temp, cb, kin, kout, iin, iout, slot_cap, 0, 64,
                                                   st);
@@ -229,7 +268,7 @@ cudaError_t launch_spatial_order(int n, const double* x, void* temp, size_t temp
   size_t cb = cub_bytes(n);
   if (off + cb > temp_bytes) return cudaErrorInvalidValue;
   bbox_kernel<<<1, 1024, 0, st>>>(n, x, box);
-  morton_kernel<<<(n + 255) / 256, 256, 0, st>>>(n, x, box, kin, iin);
+  keys_kernel<<<(n + 255) / 256, 256, 0, st>>>(n, x, box, kin, iin);
   return cub::DeviceRadixSort::SortPairs(base + off, cb, kin, kout, iin, perm, n, 0, 32, st);
 }
 

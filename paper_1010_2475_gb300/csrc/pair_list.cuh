@@ -517,7 +517,7 @@ __global__ void __launch_bounds__(kFarWarps * 32)
 }
 
 // ------------------------------------------------------------------ 4. tree far field
-// A binary tree over the Morton order of the groups: level 0 is the groups
+// A binary tree over the spatial order of the groups: level 0 is the groups
 // themselves (gdata), node i of level L >= 1 holds the groups of nodes 2i and
 // 2i+1 of level L-1, i.e. the consecutive groups [i 2^L, (i+1) 2^L).  A node
 // record has the group-record layout (gdata_len): the union of the children's

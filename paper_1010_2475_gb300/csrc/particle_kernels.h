@@ -132,7 +132,7 @@ cudaError_t launch_prep(int precision, int n, int M, const int* perm, const doub
 cudaError_t launch_group_multipole(int M, int n, const void* rec, void* gdata,
                                    const BatchInst* inst, const int* slot_inst,
                                    const int* n_slots, int max_slots, cudaStream_t st);
-// Spatial order: perm[p] = particle at sorted position p (Morton order of the
+// Spatial order: perm[p] = particle at sorted position p (Hilbert order of the
 // centres, ties by index).  temp_bytes() sizes the scratch for n particles.
 size_t spatial_order_temp_bytes(int n);
 cudaError_t launch_spatial_order(int n, const double* x, void* temp, size_t temp_bytes,
