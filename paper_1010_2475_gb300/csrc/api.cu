@@ -1067,17 +1067,18 @@ int mmvm_vorticity(mmvm_ctx* c, int64_t npts, const double* pts, double* omega) 
     return fail(MMVM_E_UNSUPPORTED, "order above the diagnostics limit (64)");
   if (npts == 0) return MMVM_OK;
   MMVM_CK(cudaSetDevice(c->cfg.device));
+  const int vch = mmvm::vorticity_chunks((int)c->n, c->M, (int)npts, c->sms);
   MMVM_CK(c->dpts.ensure(2 * (size_t)npts));
-  MMVM_CK(c->dval.ensure((size_t)npts));
+  MMVM_CK(c->dval.ensure((size_t)npts * (vch > 1 ? 1 + vch : 1)));
   MMVM_CK(cudaMemcpyAsync(c->dpts.p, pts, 2 * (size_t)npts * sizeof(double),
                           cudaMemcpyHostToDevice, c->st));
   MMVM_CK(mmvm::launch_vorticity((int)c->n, c->M, c->x.p, c->m.p, c->t_dev(),
                                  c->cfg.lambda0 * c->cfg.lambda0, 4.0 * c->cfg.nu, (int)npts,
-                                 c->dpts.p, c->dval.p, c->st));
+                                 c->dpts.p, c->dval.p, c->dval.p + npts, vch, c->st));
   MMVM_CK(cudaMemcpyAsync(omega, c->dval.p, (size_t)npts * sizeof(double),
                           cudaMemcpyDeviceToHost, c->st));
   MMVM_CK(cudaStreamSynchronize(c->st));
-  c->launches += 1;
+  c->launches += vch > 1 ? 2 : 1;
   return MMVM_OK;
 }
 
@@ -1105,19 +1106,20 @@ int mmvm_nonaxi_enstrophy(mmvm_ctx* c, double cx, double cy, double r_max, int32
   }
   MMVM_CK(cudaSetDevice(c->cfg.device));
   MMVM_CK(c->dpts.ensure(2 * np));
-  MMVM_CK(c->dval.ensure(np));
+  const int vch = mmvm::vorticity_chunks((int)c->n, c->M, (int)np, c->sms);
+  MMVM_CK(c->dval.ensure(np * (vch > 1 ? 1 + vch : 1)));
   MMVM_CK(c->dring.ensure((size_t)nr));
   MMVM_CK(cudaMemcpyAsync(c->dpts.p, pts.data(), 2 * np * sizeof(double), cudaMemcpyHostToDevice,
                           c->st));
   MMVM_CK(mmvm::launch_vorticity((int)c->n, c->M, c->x.p, c->m.p, c->t_dev(),
                                  c->cfg.lambda0 * c->cfg.lambda0, 4.0 * c->cfg.nu, (int)np,
-                                 c->dpts.p, c->dval.p, c->st));
+                                 c->dpts.p, c->dval.p, c->dval.p + np, vch, c->st));
   MMVM_CK(mmvm::launch_ring_deviation(nr, ntheta, c->dval.p, c->dring.p, c->st));
   std::vector<double> ring(nr);
   MMVM_CK(cudaMemcpyAsync(ring.data(), c->dring.p, nr * sizeof(double), cudaMemcpyDeviceToHost,
                           c->st));
   MMVM_CK(cudaStreamSynchronize(c->st));
-  c->launches += 2;
+  c->launches += vch > 1 ? 3 : 2;
   double e = 0.0;  // sum over rings of (r dr weight) x (angle sum) x (2 pi / ntheta)
   for (int i = 0; i < nr; ++i) {
     const double r = 0.5 * r_max * (xg[i] + 1.0);

@@ -104,7 +104,9 @@ cudaError_t launch_self_high(SelfHighArgs A, double* scratch, cudaStream_t st); 
 int diag_max_order();
 cudaError_t launch_vorticity(int n, int M, const double* x, const double* mom, const double* t_dev,
                              double lam0sq, double four_nu, int npts, const double* pts,
-                             double* out, cudaStream_t st);
+                             double* out, double* work, int chunks, cudaStream_t st);
+// Particle chunks for launch_vorticity; work holds chunks * npts values (unused if 1).
+int vorticity_chunks(int n, int M, int npts, int sms);
 cudaError_t launch_ring_deviation(int nr, int ntheta, const double* v, double* ring,
                                   cudaStream_t st);
 void gauss_legendre(int n, std::vector<double>& xs, std::vector<double>& ws);
