@@ -70,7 +70,9 @@ extern "C" {
  * spatial (Hilbert) order every step and tile pairs whose bounding boxes are
  * far enough apart that the Gaussian part of the pair jet is below FP32
  * rounding take the point-vortex jet (far field); this flag turns that off
- * (every pair takes the full jet).  MMVM_FP64 never uses the far field.     */
+ * (every pair takes the full jet).  MMVM_FP64 uses no tiles or expansions;
+ * a pair whose Gaussian part is below FP64 rounding (2^-54 of the jet) takes
+ * the point-vortex jet, which is the same value, unless this flag is set.   */
 #define MMVM_FLAG_NO_FAR_FIELD 1u
 /* Single particle: evaluate the self term by the separable route (the
  * coefficient sums of eq:FinalSingleI/II taken one index at a time, no

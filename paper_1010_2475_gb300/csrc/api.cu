@@ -89,6 +89,15 @@ struct mmvm_ctx {
   // source, tile expansions evaluated, pairs those expansions covered
   DevBuf<unsigned long long> counts;
   bool far = false;    // FP32 and not MMVM_FLAG_NO_FAR_FIELD: sort + far-field tiles
+  bool far64 = false;  // FP64 and not that flag: pairs beyond x_far64 take the point-vortex jet
+  // FP64 sorts from this n on: below it a warp's targets span the problem
+  static constexpr int kSortMin64 = 256;
+  bool sorted() const { return n > 1 && (far || (far64 && n >= kSortMin64)); }
+  // what the direct form's far argument gets: group records, or (FP64) any
+  // non-null pointer while the records are in spatial order
+  const void* far_arg() const {
+    return far ? (const void*)gbox.p : sorted() ? (const void*)perm.p : nullptr;
+  }
   bool high = false;   // single particle through the separable self term (self_high.cu)
   DevBuf<double> sbinom, sg, scg, sscr;  // its factor tables and scratch
   DevBuf<double> dpts, dval, dring;  // diagnostics: points, values, ring sums
@@ -201,6 +210,15 @@ int pair_launches(const mmvm_ctx* c) {
 
 int choose_chunks(const mmvm_ctx* c, int64_t n) {
   const int per_sm = c->pe.nslices ? mmvm::pair_occupancy(c->pe, c->S) : 1;
+  if (c->cfg.precision == MMVM_FP64) {
+    // ~6 waves of CTAs, down to one source per chunk: an FP64 pair keeps an
+    // SM's pipe busy for microseconds, so a small problem must spread its
+    // sources over the SMs (n = 36, M = 2: one chunk took 646 us); the
+    // finish adds NB values per chunk and target, 3 % of one source's pair
+    const int64_t tiles = (n + c->pe.tpc - 1) / c->pe.tpc;
+    const int64_t ch = (6 * (int64_t)c->sms * std::max(per_sm, 1) + tiles - 1) / tiles;
+    return (int)std::min<int64_t>(std::max<int64_t>(ch, 1), n);
+  }
   return chunks_for(n, c->pe.tpc, per_sm, c->cfg.device, c->S);
 }
 
@@ -249,9 +267,11 @@ int ensure_buffers(mmvm_ctx* c, int64_t n) {
         MMVM_CK(c->errf.ensure(1));
         MMVM_CK(cudaMemset(c->errf.p, 0, sizeof(int)));
       }
-      MMVM_CK(grow(c->perm, (size_t)n));
       MMVM_CK(grow(c->gbox, (size_t)mmvm::gdata_len(c->M) *
                                 ((n + mmvm::kGroup - 1) / mmvm::kGroup)));
+    }
+    if (c->sorted()) {
+      MMVM_CK(grow(c->perm, (size_t)n));
       MMVM_CK(grow(c->order_tmp, mmvm::spatial_order_temp_bytes((int)n)));
       if (realloc) {
         // count the kernels one ordering launches (the sort's are the library's)
@@ -293,9 +313,9 @@ int enqueue_rhs(mmvm_ctx* c, int mode, const double* xin, const double* min_, do
   if (!out_dM) out_dM = c->rdm.p;
   const double lam0sq = c->cfg.lambda0 * c->cfg.lambda0;
   const double four_nu = 4.0 * c->cfg.nu;
-  const int* perm = (n > 1 && c->far) ? c->perm.p : nullptr;
+  const int* perm = c->sorted() ? c->perm.p : nullptr;
   if (n > 1) {
-    if (c->far && (mode == 0 || mode == 1)) {  // order from the step-start centres
+    if (c->sorted() && (mode == 0 || mode == 1)) {  // order from the step-start centres
       MMVM_CK(mmvm::launch_spatial_order(n, xin, c->order_tmp.p, c->order_tmp.cap, c->perm.p,
                                          c->st));
       c->launches += c->order_launches;
@@ -312,9 +332,8 @@ int enqueue_rhs(mmvm_ctx* c, int mode, const double* xin, const double* min_, do
                                 c->st, c->timing ? c->evm[slot] : nullptr));
       if (c->timing) c->evm_pending[slot] = true;
     } else {
-      MMVM_CK(mmvm::pair_launch(c->pe, c->rec.p, n, c->chunks, c->S,
-                                c->far ? c->gbox.p : nullptr, c->partial.p, 0, c->st,
-                                c->counts.p));
+      MMVM_CK(mmvm::pair_launch(c->pe, c->rec.p, n, c->chunks, c->S, c->far_arg(), c->partial.p,
+                                0, c->st, c->counts.p));
     }
     if (c->timing) {
       MMVM_CK(cudaEventRecord(c->ev[slot][1], c->st));
@@ -710,6 +729,7 @@ int mmvm_create(const mmvm_config* cfg, mmvm_ctx** out) {
   mmvm_ctx* c = new mmvm_ctx();
   c->cfg = *cfg;
   c->far = cfg->precision == MMVM_MIXED_FP32 && !(cfg->flags & MMVM_FLAG_NO_FAR_FIELD);
+  c->far64 = cfg->precision == MMVM_FP64 && !(cfg->flags & MMVM_FLAG_NO_FAR_FIELD);
   c->M = cfg->order;
   c->K = mmvm::n_moments(c->M);
   c->NB = mmvm::n_beta(c->M);
@@ -825,6 +845,7 @@ static int set_state_common(mmvm_ctx* c, int64_t n, const double* x, const doubl
     if (rc) return rc;
   }
   MMVM_CK(cudaStreamSynchronize(c->st));
+  if (n != c->n) c->drop_graph();  // the captured step holds launches for the old n
   c->n = n;
   int rc = ensure_buffers(c, n);
   if (rc) return rc;
@@ -937,7 +958,7 @@ int mmvm_step(mmvm_ctx* c, double dt, int64_t nsteps) {
     c->graph_ok = true;
   }
   const int per_step =
-      (c->n > 1 ? 4 * ((c->far ? 2 : 1) + pair_launches(c) + 1) + (c->far ? c->order_launches : 0)
+      (c->n > 1 ? 4 * ((c->far ? 2 : 1) + pair_launches(c) + 1) + (c->sorted() ? c->order_launches : 0)
                 : (c->high ? 20 : 4)) +
       1;
   for (int64_t s = 0; s < nsteps; ++s) {

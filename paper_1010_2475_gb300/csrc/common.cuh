@@ -94,6 +94,15 @@ __host__ __device__ constexpr float x_far(int M) {
        : M == 5 ? 66.f : M == 6 ? 74.f : M == 7 ? 80.f : 88.f;
 }
 
+// The same threshold for FP64 pairs: beyond it the Gaussian part of every jet
+// entry of order <= 3M is below 2^-54 of the largest entry of that order
+// (maximum over all directions; 6 units of margin added), so the point-vortex
+// jet equals the full jet to FP64 rounding.
+__host__ __device__ constexpr float x_far64(int M) {
+  return M <= 0 ? 44.f : M == 1 ? 52.f : M == 2 ? 63.f : M == 3 ? 72.f : M == 4 ? 81.f
+       : M == 5 ? 90.f : M == 6 ? 98.f : M == 7 ? 107.f : 115.f;
+}
+
 // Far source tiles seen from far enough away are summed through one
 // multipole expansion about the tile's centre instead of source by source.
 // With u = 1/w, w = target - centre, delta_s = source - centre and

@@ -59,85 +59,53 @@ namespace mmvm {
 constexpr double kInvPi = 0.31830988618379067154;
 constexpr double kInv4Pi = 0.07957747154594766788;
 
-// 1/i, correctly rounded (compile-time), for the Kummer series below: the
-// loop index is a run-time value, and a table read is cheaper than a
-// correctly rounded reciprocal at run time.
-struct RecipTable {
-  float f[128];
-  double d[128];
-};
-constexpr RecipTable make_recip_table() {
-  RecipTable t{};
-  for (int i = 1; i < 128; ++i) {
-    t.f[i] = 1.0f / (float)i;
-    t.d[i] = 1.0 / (double)i;
-  }
-  return t;
-}
-static __constant__ RecipTable kRecip = make_recip_table();
-
-template <typename T> __device__ __forceinline__ T recip_of(int i);
-template <> __device__ __forceinline__ float recip_of<float>(int i) { return kRecip.f[i]; }
-template <> __device__ __forceinline__ double recip_of<double>(int i) { return kRecip.d[i]; }
-
-// Terms of the FP32 Kummer series at order P: the smallest KN with
-// prod_{j=1}^{KN} P / (P + 1 + j) below 2^-26, so that the terms dropped are
-// below FP32 rounding of the sum for every x <= P (the series is only used
-// there, or for x < 1).
-constexpr int kummer_terms(int P) {
+// Terms of the Kummer series at order P: the smallest KN with
+// prod_{j=1}^{KN} P / (P + 1 + j) below 2^-BITS, so that the terms dropped are
+// below rounding of the sum for every x <= P (the series is only used there,
+// or for x < 1).  BITS: 26 in FP32, 56 in FP64.
+constexpr int kummer_terms(int P, int bits) {
+  double eps = 1.0;
+  for (int i = 0; i < bits; ++i) eps *= 0.5;
   double t = 1.0;
   int k = 0;
-  while (t >= 1.0 / 67108864.0 && k < 120) {
+  while (t >= eps && k < 160) {
     ++k;
     t *= (double)(P > 0 ? P : 1) / (double)(P + 1 + k);
   }
   return k + 1;
 }
-// Coefficients of the FP32 Horner form in y = x / Ps (Ps = max(P, 1)):
+// Coefficients of the Horner form in y = x / Ps (Ps = max(P, 1)):
 // d_k = Ps^k / ((P+1)(P+2)...(P+k+1)), all in (0, 1/(P+1)] and far inside the
 // FP32 range (the unscaled 1 / ((P+1)...(P+k+1)) underflows it).
-template <int P>
+template <int P, typename T>
 struct KummerCoef {
-  static constexpr int KN = kummer_terms(P);
+  static constexpr int KN = kummer_terms(P, sizeof(T) == 4 ? 26 : 56);
   static constexpr int PS = P > 0 ? P : 1;
-  float c[KN];
+  T c[KN];
   constexpr KummerCoef() : c() {
     double v = 1.0;
     for (int k = 0; k < KN; ++k) {
       v = v * (k > 0 ? (double)PS : 1.0) / (double)(P + 1 + k);
-      c[k] = (float)v;
+      c[k] = (T)v;
     }
   }
 };
 
-// sum_{k>=0} x^k / ((P+1)(P+2)...(P+k+1)) so that I_P(x) = e^{-x} * sum (x < P).
-// FP32: a fixed Horner form (every coefficient positive, so it is as
-// accurate as the term-by-term sum; no data-dependent trip count that would
-// split the lanes of a warp).
+// sum_{k>=0} x^k / ((P+1)(P+2)...(P+k+1)) so that I_P(x) = e^{-x} * sum (x < P),
+// as a fixed Horner form: every coefficient is positive, so it is as accurate
+// as the term-by-term sum, costs one multiply-add per term (the FP64 loop
+// took three operations and a test) and has no data-dependent trip count that
+// would split the lanes of a warp.
 template <int P, typename T>
 __device__ __forceinline__ T kummer_sum(T x) {
-  constexpr bool f32 = std::is_same<T, float>::value;
-  if constexpr (f32) {
-    constexpr KummerCoef<P> kc{};
-    const T y = x * T(1.0 / KummerCoef<P>::PS);
-    T s = T(kc.c[KummerCoef<P>::KN - 1]);
-    static_for_down<0, KummerCoef<P>::KN - 1>([&](auto ic) {
-      constexpr int k = decltype(ic)::value;
-      s = fma(s, y, T(kc.c[k]));
-    });
-    return s;
-  }
-  const T eps = f32 ? T(2e-8) : T(5e-18);
-  constexpr int kmax = f32 ? 48 : 80;
-  static_assert(P + kmax < 128, "reciprocal table too short");
-  T term = T(1.0 / (P + 1));
-  T s = term;
-#pragma unroll 1
-  for (int k = 1; k < kmax; ++k) {
-    term = term * x * recip_of<T>(P + 1 + k);
-    s += term;
-    if (term <= eps * s) break;
-  }
+  using KC = KummerCoef<P, T>;
+  constexpr KC kc{};
+  const T y = x * T(1.0 / KC::PS);
+  T s = kc.c[KC::KN - 1];
+  static_for_down<0, KC::KN - 1>([&](auto ic) {
+    constexpr int k = decltype(ic)::value;
+    s = fma(s, y, kc.c[k]);
+  });
   return s;
 }
 
@@ -145,8 +113,12 @@ __device__ __forceinline__ T kummer_sum(T x) {
 // up to n = P + 1 in FP32: there I_P(x) ~ P! / x^(P+1) stays above 1e-35 and
 // |zbar|^(P+1) below 1e30, inside the normal FP32 range (I_17(300) ~ 1e-30,
 // I_23(200) ~ 1e-33).  In FP32 the two forms agree to ~2e-6 of |w_n| at
-// n = 18 over 20 <= x <= 400.
-__host__ __device__ constexpr float table_x(int P) { return P <= 17 ? 300.f : 200.f; }
+// n = 18 over 20 <= x <= 400.  In FP64 x < 1e6 keeps |zbar|^24 and
+// I_23(x) ~ 23! / x^24 far inside the range.
+template <typename T>
+__host__ __device__ constexpr float table_x(int P) {
+  return sizeof(T) == 8 ? 1e6f : P <= 17 ? 300.f : 200.f;
+}
 
 // Outputs of one order slice: Psi[beta] with LO <= |beta| <= HI, i.e. the
 // columns [B0, B1).  They need the jet orders LO .. HI + M only.  PART 1
@@ -173,13 +145,18 @@ struct PairNear {
   // used for the self pair, whose separation the caller moves far away).
   __device__ __forceinline__ static void run(T b1, T b2, T l1, T l2, T wmask,
                                              const T (&a)[K], T (&acc)[NBL]) {
+    constexpr bool f32 = std::is_same<T, float>::value;
     // squares (b_hi + b_lo)^2 = s_d + q_d + 2 b_hi b_lo (q_d: rounding of s_d)
     const T s1 = b1 * b1;
     const T s2 = b2 * b2;
     const T q1 = fma(b1, b1, -s1);
     const T q2 = fma(b2, b2, -s2);
-    const T sl1 = q1 + T(2) * b1 * l1;
-    const T sl2 = q2 + T(2) * b2 * l2;
+    // (FP64 has no lo part: l1 = l2 = 0, and its terms are left out)
+    T sl1 = q1, sl2 = q2;
+    if constexpr (f32) {
+      sl1 = q1 + T(2) * b1 * l1;
+      sl2 = q2 + T(2) * b2 * l2;
+    }
     // x = xh + xl (TwoSum of the two squares plus the small corrections)
     const T xh = s1 + s2;
     const T bv = xh - s1;
@@ -189,7 +166,8 @@ struct PairNear {
     const T eh1 = dexp(-s1) * (T(1) - q1);
     const T eh2 = dexp(-s2) * (T(1) - q2);
     // ... and e^{-x} at the full separation
-    const T E = eh1 * (T(1) - T(2) * b1 * l1) * (eh2 * (T(1) - T(2) * b2 * l2));
+    T E = eh1 * eh2;
+    if constexpr (f32) E = eh1 * (T(1) - T(2) * b1 * l1) * (eh2 * (T(1) - T(2) * b2 * l2));
     // Hermite functions at b_hi, one order beyond what is used, then the
     // first-order correction to b = b_hi + b_lo: hx[k] = h_k(b1)/pi, hy[k] = h_k(b2)
     T hx[HN + 1], hy[HN + 1];
@@ -202,11 +180,13 @@ struct PairNear {
       hx[k + 1] = T(-2) * b1 * hx[k] - T(2 * k) * hx[k - 1];
       hy[k + 1] = T(-2) * b2 * hy[k] - T(2 * k) * hy[k - 1];
     });
-    static_for<0, HN>([&](auto kc) {
-      constexpr int k = decltype(kc)::value;
-      hx[k] = fma(l1, hx[k + 1], hx[k]);
-      hy[k] = fma(l2, hy[k + 1], hy[k]);
-    });
+    if constexpr (f32) {
+      static_for<0, HN>([&](auto kc) {
+        constexpr int k = decltype(kc)::value;
+        hx[k] = fma(l1, hx[k + 1], hx[k]);
+        hy[k] = fma(l2, hy[k + 1], hy[k]);
+      });
+    }
 
     if constexpr (PART != 2) {
     // The holomorphic edge w_n = zbar^n I_{n-1}(x) is formed one order at a
@@ -217,7 +197,7 @@ struct PairNear {
     // threshold, so the lanes of a warp agree and the per-order test does
     // not split the warp.
     constexpr int P = NJ - 1;
-    const bool small = x < T(table_x(P));
+    const bool small = x < T(table_x<T>(P));
     const T rxh = T(1) / x;  // inf at x == 0: those entries are replaced below
     const T rx = rxh * (T(1) - xl * rxh);
     T I[P + 1];
@@ -255,8 +235,14 @@ struct PairNear {
       T w_r, w_i;
       if (small) {
         if constexpr (n > 1) {  // (zr + i zi) * ((b1 + l1) - i (b2 + l2)), two-term
-          const T tr = fma(zr, b1, fma(zi, b2, fma(zr, l1, zi * l2)));
-          const T ti = fma(zi, b1, fma(-zr, b2, fma(zi, l1, -zr * l2)));
+          T tr, ti;
+          if constexpr (f32) {
+            tr = fma(zr, b1, fma(zi, b2, fma(zr, l1, zi * l2)));
+            ti = fma(zi, b1, fma(-zr, b2, fma(zi, l1, -zr * l2)));
+          } else {
+            tr = fma(zr, b1, zi * b2);
+            ti = fma(zi, b1, -zr * b2);
+          }
           zr = tr;
           zi = ti;
         }
@@ -389,11 +375,13 @@ struct FarSums {
                                              T (&yi)[NY]) {
     const T inv = T(1) / (b1 * b1 + b2 * b2);
     T ur = b1 * inv, ui = -b2 * inv;  // 1 / z_hi
-    // u = 1/(z_hi + l) = uh (1 - l uh) to first order in the low part l = l1 + i l2
-    const T tr = l1 * ur - l2 * ui, ti = l1 * ui + l2 * ur;
-    const T nr = ur - (ur * tr - ui * ti), ni = ui - (ur * ti + ui * tr);
-    ur = nr;
-    ui = ni;
+    if constexpr (std::is_same<T, float>::value) {
+      // u = 1/(z_hi + l) = uh (1 - l uh) to first order in the low part l = l1 + i l2
+      const T tr = l1 * ur - l2 * ui, ti = l1 * ui + l2 * ur;
+      const T nr = ur - (ur * tr - ui * ti), ni = ui - (ur * ti + ui * tr);
+      ur = nr;
+      ui = ni;
+    }
     T ar[NA], ai[NA];
 #pragma unroll
     for (int n = 0; n < NA; ++n) {

@@ -67,6 +67,7 @@ __device__ __forceinline__ void near_source(const T* r, int src, int j, T tz1, T
     l1 = T(0);
     l2 = T(0);
     wm = T(0);
+    if constexpr (!std::is_same<T, float>::value) b1 = T(1e3);  // inside the table form
   }
   PN::run(b1, b2, l1, l2, wm, a, accr);
 }
@@ -149,6 +150,43 @@ __device__ __forceinline__ void far_source(const float* r, float tz1, float tz2,
   PairFar<M, float, LO, HI>::run(b1, b2, l1, l2, r + HDR + K, yr, yi);
 }
 
+// One far source in FP64: the source's multipoles af (A'_n of the tile's
+// source, tile_multipoles), added to the edge columns of acc.
+template <int M, int LO, int HI>
+__device__ __forceinline__ void far_source64(const double* r, const double* af, double tz1,
+                                             double tz2, double* acc) {
+  double yr[HI - LO + 1], yi[HI - LO + 1];
+#pragma unroll
+  for (int b = 0; b < HI - LO + 1; ++b) {
+    yr[b] = 0.0;
+    yi[b] = 0.0;
+  }
+  PairFar<M, double, LO, HI>::run(tz1 - r[0], tz2 - r[1], 0.0, 0.0, af, yr, yi);
+  fold_far<M, double, LO, HI>(yr, yi, acc);
+}
+
+// A'_n = sum_{|m|=n} a_m (-i)^{m1+n}, n = 0..M, of an FP64 record (FP32
+// records carry them).
+template <int M>
+__device__ __forceinline__ void tile_multipoles(const double* r, double* af) {
+  constexpr int HDR = Rec<double>::HDR;
+  static_for<0, M + 1>([&](auto nc) {
+    constexpr int n = decltype(nc)::value;
+    double fr = 0.0, fi = 0.0;
+    static_for<0, n + 1>([&](auto kc) {
+      constexpr int k2 = decltype(kc)::value;
+      constexpr int q = (n - k2 + n) & 3;
+      const double a = r[HDR + mcol(n - k2, k2)];
+      if constexpr (q == 0) fr += a;
+      if constexpr (q == 1) fi -= a;
+      if constexpr (q == 2) fr -= a;
+      if constexpr (q == 3) fi += a;
+    });
+    af[2 * n] = fr;
+    af[2 * n + 1] = fi;
+  });
+}
+
 // Group record g (see gdata_len in common.cuh).
 template <int M>
 __device__ __forceinline__ const float* group_rec(const float* __restrict__ gdata, int g) {
@@ -219,12 +257,19 @@ __device__ __forceinline__ void m2p_tile(const float* __restrict__ gdata, int sg
   flush_edge_sums<M, LO, HI, PART, TPC>(tmp, acc_hi, acc_lo, slot);
 }
 
+// Doubles of far-field multipoles per source of an FP64 tile.
+__host__ __device__ constexpr int tile_far64(int M) { return 2 * (M + 1); }
+
 // The work of one CTA: targets tile0 .. tile0 + TPC - 1 (those below n) of
 // one instance against its sources c0 .. c1 - 1.  rec holds the instance's n
 // records (indices are local to it); gdata: one record per group of kGroup
 // consecutive records (box of the hi parts, centre, radius, expansion about
-// the centre; see gdata_len), null disables the far-field path (FP64
-// always).  A far tile is summed through its expansion when it is far enough
+// the centre; see gdata_len), null disables the far-field path.  FP64 reads no
+// group record: with gdata non-null (the records are in spatial order), a
+// source beyond x_far64(M) of the box of the warp's targets takes the
+// point-vortex jet, which equals the full jet to FP64 rounding there (n = 2048,
+// M = 6 two patches: 2 of 3 pairs, at about 430 instead of 2500 operations).
+// FP32: A far tile is summed through its expansion when it is far enough
 // for it (tile_takes_m2p), else source by source with the point-vortex jet.
 // out: this chunk's block [NB][n] of the partial sums (coalesced FP64
 // stores); only the slice's columns are written.  counts (nullable):
@@ -273,6 +318,7 @@ __device__ __forceinline__ void pair_tile_work(const T* __restrict__ rec, int n,
   // far tiles: skipped by every part; summed (pass 1) by parts 0 and 1 (the
   // Laplacian columns of a far tile are zero)
   const bool use_far = f32 && gdata != nullptr;
+  const bool far64 = !f32 && gdata != nullptr;
   // this thread's target: pairs on each path, tile expansions evaluated
   unsigned n_near = 0, n_far = 0, n_m2p = 0, n_m2p_pairs = 0;
   // did this warp accumulate anything? (warp-uniform; a warp that did not
@@ -351,6 +397,18 @@ __device__ __forceinline__ void pair_tile_work(const T* __restrict__ rec, int n,
   float4 tbox = make_float4(0.f, 0.f, 0.f, 0.f);
   if constexpr (f32) {
     if (use_far && warp_valid) tbox = *reinterpret_cast<const float4*>(group_rec<M>(gdata, tgroup));
+  } else if (far64) {
+    // box of the warp's targets, in FP32 (x_far64 has margin for the rounding)
+    float lo1 = j < n ? (float)tz1 : 3.4e38f, hi1 = j < n ? (float)tz1 : -3.4e38f;
+    float lo2 = j < n ? (float)tz2 : 3.4e38f, hi2 = j < n ? (float)tz2 : -3.4e38f;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      lo1 = fminf(lo1, __shfl_xor_sync(0xffffffffu, lo1, o));
+      hi1 = fmaxf(hi1, __shfl_xor_sync(0xffffffffu, hi1, o));
+      lo2 = fminf(lo2, __shfl_xor_sync(0xffffffffu, lo2, o));
+      hi2 = fmaxf(hi2, __shfl_xor_sync(0xffffffffu, hi2, o));
+    }
+    tbox = make_float4(lo1, hi1, lo2, hi2);
   }
 #pragma unroll 1
   for (int t0 = c0; t0 < c1; t0 += S) {
@@ -373,6 +431,14 @@ __device__ __forceinline__ void pair_tile_work(const T* __restrict__ rec, int n,
     if (__syncthreads_or(near)) {
       load_tile(t0, cnt);
       __syncthreads();
+      if constexpr (!f32 && PART != 2) {
+        if (far64) {
+          T* mf = tile + (size_t)S * R;
+          for (int s = threadIdx.x; s < cnt; s += blockDim.x)
+            tile_multipoles<M>(tile + s * R, mf + s * tile_far64(M));
+          __syncthreads();
+        }
+      }
       if constexpr (f32 && PART != 2) {
         if (m2p2) {
           work = true;
@@ -391,6 +457,11 @@ __device__ __forceinline__ void pair_tile_work(const T* __restrict__ rec, int n,
           bool sfar = sbs;  // every source of a far tile is far from the warp's box
           if constexpr (f32) {
             if (use_far && near) sfar = point_is_far<M>(tbox, rs[0], rs[1]);
+          } else if (far64) {
+            const float z1 = (float)rs[0], z2 = (float)rs[1];
+            const float dx = fmaxf(0.f, fmaxf(tbox.x - z1, z1 - tbox.y));
+            const float dy = fmaxf(0.f, fmaxf(tbox.z - z2, z2 - tbox.w));
+            sfar = dx * dx + dy * dy >= x_far64(M);
           }
           if (!sfar) {
             near_source<M, T, LO, HI, PART>(rs, t0 + s, j, tz1, tz2, tl1, tl2, acc);
@@ -404,9 +475,14 @@ __device__ __forceinline__ void pair_tile_work(const T* __restrict__ rec, int n,
             far_source<M, LO, HI>(reinterpret_cast<const float*>(rs), tz1, tz2, tl1, tl2, yr,
                                   yi);
             fold_far<M, float, LO, HI>(yr, yi, reinterpret_cast<float*>(acc));
+          } else if constexpr (!f32 && PART != 2) {
+            far_source64<M, LO, HI>(reinterpret_cast<const double*>(rs),
+                                    reinterpret_cast<const double*>(tile + (size_t)S * R) +
+                                        s * tile_far64(M),
+                                    tz1, tz2, reinterpret_cast<double*>(acc));
           }
           if (j < n) {
-            if (sfar)
+            if (f32 && sfar)  // FP64 pairs all count as near: the jet is the full one to rounding
               ++n_far;
             else
               ++n_near;
@@ -509,6 +585,8 @@ size_t pair_smem_bytes(int S) {  // shared memory of one CTA
   size_t b = (size_t)S * rec_len<T>(M) * sizeof(T);
   if (std::is_same<T, float>::value)
     b += 2 * (size_t)PartCols<LO, HI, PART>::NS * TPC * sizeof(float);
+  else if (PART != 2)
+    b += (size_t)S * tile_far64(M) * sizeof(T);
   return b;
 }
 

@@ -59,8 +59,10 @@ int pair_occupancy(const PairEntry& e, int S) {
 cudaError_t pair_launch(const PairEntry& e, const void* rec, int n, int chunks, int S,
                         const void* gbox, double* partial, int grid_y_limit, cudaStream_t st,
                         unsigned long long* counts) {
-  // chunks start on group boundaries so every source tile is one group
-  const int chunk_len = round_up((n + chunks - 1) / chunks, S);
+  // FP32 chunks start on group boundaries so every source tile is one group
+  // (its record decides near or far); FP64 reads no group records
+  const int len = (n + chunks - 1) / chunks;
+  const int chunk_len = e.precision == 1 ? round_up(len, S) : len;
   const int gy = (grid_y_limit > 0 && chunks > grid_y_limit) ? grid_y_limit : chunks;
   for (int s = 0; s < e.nslices; ++s) {
     cudaError_t r = e.slices[s].launch(rec, n, chunk_len, gy, S, gbox, partial, counts, st);

@@ -48,8 +48,9 @@ PairEntry pair_entry(int M, int precision, int v);
 cudaError_t pair_prepare(const PairEntry& e, int S);
 // CTAs per SM of the slice kernels (the smallest), 0 on error.
 int pair_occupancy(const PairEntry& e, int S);
-// Launch every slice.  gbox: float4 per group of kGroup records (null: every
-// pair takes the full jet); S must equal kGroup.  Sources are split into
+// Launch every slice.  gbox: group records (null: every pair takes the full
+// jet; FP64: only whether it is null is read, see pair_tile_work); S must
+// equal kGroup.  Sources are split into
 // `chunks` chunks of a multiple of S; `partial` holds min(chunks, grid_y_limit)
 // chunks (grid_y_limit > 0 launches only the first grid_y_limit chunks, used
 // when timing variants; 0 launches all of them).  counts (nullable) receives

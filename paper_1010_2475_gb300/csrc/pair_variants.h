@@ -38,17 +38,17 @@ constexpr int n_variants(int M, int prec) {
 }
 
 constexpr VariantSpec variant_spec(int M, int prec, int v) {
-  if (prec == 0) {  // FP64: narrow slices keep the FP64 accumulators in registers
+  // FP64: the edge and the Laplacian columns of all orders as two kernels from
+  // order 3 on.  The FP64 pipe is the bound (2 FMA per cycle and SM), so the
+  // fewest FP64 operations win over register pressure: order slices (the jet
+  // formed again for each) took 6600 operations per pair at M = 6, the parts
+  // take about 2500; the registers they spill cost little beside that.
+  if (prec == 0) {
     switch (M) {
       case 0: return {1, {{1, 1}}, 64, 1, 0};
       case 1: return {1, {{1, 2}}, 64, 1, 0};
       case 2: return {1, {{1, 4}}, 64, 1, 0};
-      case 3: return {1, {{1, 6}}, 64, 1, 0};
-      case 4: return {2, {{1, 5}, {6, 8}}, 64, 1, 0};
-      case 5: return {2, {{1, 6}, {7, 10}}, 64, 1, 0};
-      case 6: return {3, {{1, 7}, {8, 10}, {11, 12}}, 64, 1, 0};
-      case 7: return {4, {{1, 7}, {8, 10}, {11, 12}, {13, 14}}, 64, 1, 0};
-      default: return {4, {{1, 8}, {9, 11}, {12, 14}, {15, 16}}, 64, 1, 0};
+      default: return {2, {{1, 2 * M, 1}, {1, 2 * M, 2}}, 64, 1, 0};
     }
   }
   switch (M) {
