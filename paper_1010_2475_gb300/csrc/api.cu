@@ -122,6 +122,12 @@ struct mmvm_ctx {
   bool tree = false;
   DevBuf<float> tnodes;
   int lc = 0, tfar = 1;
+  // local expansions of compact groups (pair_local.cuh): group expansions and
+  // the target groups' fields of loc_seg list segments
+  bool local = false;
+  int loc_seg = 1;
+  DevBuf<float> gexp;
+  DevBuf<float2> fld, ffld;
   int S = 32;            // sources per shared-memory tile
   int chunks = 1;        // source chunks of the pair kernel
   bool graph_ok = false;
@@ -205,7 +211,7 @@ void list_shape(const mmvm_ctx* c, const mmvm::ListEntry& e, int64_t n, int* lse
 int pair_launches(const mmvm_ctx* c) {
   if (!c->list) return c->pe.nslices;
   const int G = (int)((c->n + mmvm::kGroup - 1) / mmvm::kGroup);
-  return 1 + (c->tree ? mmvm::tree_levels(G) + 1 : 1) + c->le.nslices;
+  return 1 + (c->tree ? mmvm::tree_levels(G) + 1 : 1) + (c->local ? 4 : 0) + c->le.nslices;
 }
 
 int choose_chunks(const mmvm_ctx* c, int64_t n) {
@@ -229,7 +235,8 @@ constexpr int kTuneChunks = 8;
 // Process-wide autotuning results: (device, M, precision, far, log2 n) -> variant.
 std::mutex g_tune_mu;
 std::map<std::tuple<int, int, int, int, int>, int> g_tuned;
-std::map<std::tuple<int, int, int, int, int>, int> g_tuned_tree;  // list form: tree far field
+std::map<std::tuple<int, int, int, int, int>, int> g_tuned_tree;   // list form: tree far field
+std::map<std::tuple<int, int, int, int, int>, int> g_tuned_local;  // list form: local expansions
 
 int ilog2(int64_t v) {
   int r = 0;
@@ -262,7 +269,7 @@ int ensure_buffers(mmvm_ctx* c, int64_t n) {
     if (c->far) {
       const size_t G = (size_t)((n + mmvm::kGroup - 1) / mmvm::kGroup);
       MMVM_CK(grow(c->lent, G * G));
-      MMVM_CK(grow(c->lcnt, G));
+      MMVM_CK(grow(c->lcnt, 2 * G));
       if (!c->errf.p) {
         MMVM_CK(c->errf.ensure(1));
         MMVM_CK(cudaMemset(c->errf.p, 0, sizeof(int)));
@@ -303,6 +310,31 @@ int ensure_buffers(mmvm_ctx* c, int64_t n) {
   return MMVM_OK;
 }
 
+// The context's buffers for a list-form evaluation of the given shape.
+mmvm::ListArgs list_args(mmvm_ctx* c, int n, int lseg, int lfar, bool tree, int lc, bool local,
+                         int loc_seg, unsigned long long* counts) {
+  mmvm::ListArgs A;
+  A.rec = reinterpret_cast<const float*>(c->rec.p);
+  A.n = n;
+  A.gdata = c->gbox.p;
+  A.ent = c->lent.p;
+  A.cnt = c->lcnt.p;
+  A.segments = lseg;
+  A.partial = c->partial.p;
+  A.far_ranges = lfar;
+  A.fpart = c->fpart.p;
+  A.tree = tree ? c->tnodes.p : nullptr;
+  A.Lc = lc;
+  A.local = local;
+  A.loc_segments = loc_seg;
+  A.gexp = c->gexp.p;
+  A.fld = c->fld.p;
+  A.ffld = c->ffld.p;
+  A.counts = counts;
+  A.err = c->errf.p;
+  return A;
+}
+
 // One RHS evaluation: mode 0 writes (rdx, rdm); modes 1..4 are RK4 stages.
 // out_dx / out_dM (mode 0 only): where the RHS goes (null: the context's own
 // rdx / rdm).
@@ -326,10 +358,10 @@ int enqueue_rhs(mmvm_ctx* c, int mode, const double* xin, const double* min_, do
     const int slot = mode == 0 ? 4 : mode - 1;
     if (c->timing) MMVM_CK(cudaEventRecord(c->ev[slot][0], c->st));
     if (c->list) {
-      MMVM_CK(mmvm::list_launch(c->le, reinterpret_cast<const float*>(c->rec.p), n, c->gbox.p,
-                                c->lent.p, c->lcnt.p, c->lseg, c->partial.p, c->lfar, c->fpart.p,
-                                c->tree ? c->tnodes.p : nullptr, c->lc, c->counts.p, c->errf.p,
-                                c->st, c->timing ? c->evm[slot] : nullptr));
+      MMVM_CK(mmvm::list_launch(
+          c->le,
+          list_args(c, n, c->lseg, c->lfar, c->tree, c->lc, c->local, c->loc_seg, c->counts.p),
+          c->st, c->timing ? c->evm[slot] : nullptr));
       if (c->timing) c->evm_pending[slot] = true;
     } else {
       MMVM_CK(mmvm::pair_launch(c->pe, c->rec.p, n, c->chunks, c->S, c->far_arg(), c->partial.p,
@@ -374,11 +406,16 @@ int enqueue_rhs(mmvm_ctx* c, int mode, const double* xin, const double* min_, do
   A.M = c->M;
   A.K = c->K;
   A.NB = c->NB;
-  A.nchunks = n > 1 ? (c->list ? c->lseg : c->chunks) : 0;
+  A.nchunks = n > 1 ? (c->list ? c->lseg + (c->local ? 1 : 0) : c->chunks) : 0;
   if (n > 1 && c->list) {
     A.fpart = c->fpart.p;
     A.nfar = c->tree ? c->tfar : c->lfar;
     A.n_edge = c->le.far.n_edge;
+    if (c->local) {  // groups with a local field have no far block
+      A.gdata = c->gbox.p;
+      A.gdata_len = mmvm::gdata_len(c->M);
+      A.rmax = c->le.far.loc_radius;
+    }
   }
   A.partial = n > 1 ? c->partial.p : nullptr;
   A.perm = perm;
@@ -445,16 +482,31 @@ static cudaError_t time_pair_variant(mmvm_ctx* c, const mmvm::PairEntry& e, int 
 
 // Make the list buffers hold list variant e's shape for n records; the
 // shape goes to *lseg / *lfar.
-static int ensure_list_buffers(mmvm_ctx* c, const mmvm::ListEntry& e, int n, int* lseg,
-                               int* lfar) {
+static int ensure_list_buffers(mmvm_ctx* c, const mmvm::ListEntry& e, int n, bool local,
+                               int* lseg, int* lfar, int* loc_seg) {
   list_shape(c, e, n, lseg, lfar);
+  const int64_t G = (n + mmvm::kGroup - 1) / mmvm::kGroup;
+  // ~4 waves of warps (8 per SM) of the local kernel
+  *loc_seg = (int)std::min<int64_t>(std::max<int64_t>((32 * (int64_t)c->sms + G - 1) / G, 1), 8);
+  if (local) {
+    const size_t ge = (size_t)G * e.far.loc_len;
+    const size_t fl = (size_t)*loc_seg * G * e.far.loc_rows * 32;
+    const size_t ff = (size_t)*lfar * G * 64;  // at most lfar nodes on the tree's start level
+    if (ge > c->gexp.cap || !c->gexp.p || fl > c->fld.cap || !c->fld.p || ff > c->ffld.cap ||
+        !c->ffld.p) {
+      MMVM_CK(c->gexp.ensure(std::max(ge, c->gexp.cap)));
+      MMVM_CK(c->fld.ensure(std::max(fl, c->fld.cap)));
+      MMVM_CK(c->ffld.ensure(std::max(ff, c->ffld.cap)));
+      c->drop_graph();
+    }
+  }
   const size_t tn = (size_t)mmvm::tree_nodes((n + mmvm::kGroup - 1) / mmvm::kGroup) *
                     mmvm::gdata_len(c->M);
   if (tn > c->tnodes.cap || !c->tnodes.p) {
     MMVM_CK(c->tnodes.ensure(std::max<size_t>(tn, 1)));
     c->drop_graph();
   }
-  const size_t part = (size_t)*lseg * c->NB * n;
+  const size_t part = (size_t)(*lseg + (local ? 1 : 0)) * c->NB * n;
   const size_t fp = (size_t)*lfar * e.far.n_edge * n;
   if (part > c->partial.cap || fp > c->fpart.cap || !c->fpart.p) {
     MMVM_CK(c->partial.ensure(std::max(part, c->partial.cap)));
@@ -466,20 +518,17 @@ static int ensure_list_buffers(mmvm_ctx* c, const mmvm::ListEntry& e, int n, int
 
 // Time one launch of list variant e on the context's current records (after
 // one untimed launch); *per_pair = milliseconds per pair.
-static int time_list_variant(mmvm_ctx* c, const mmvm::ListEntry& e, int n, bool tree,
+static int time_list_variant(mmvm_ctx* c, const mmvm::ListEntry& e, int n, bool tree, bool local,
                              cudaEvent_t e0, cudaEvent_t e1, double* per_pair) {
-  int lseg = 1, lfar = 1;
-  int rc = ensure_list_buffers(c, e, n, &lseg, &lfar);
+  int lseg = 1, lfar = 1, loc_seg = 1;
+  int rc = ensure_list_buffers(c, e, n, local, &lseg, &lfar, &loc_seg);
   if (rc) return rc;
-  const float* rec = reinterpret_cast<const float*>(c->rec.p);
   int tfar = 1;
   const int lc = mmvm::tree_chunk_level((n + mmvm::kGroup - 1) / mmvm::kGroup, lfar, &tfar);
-  float* tr = tree ? c->tnodes.p : nullptr;
-  MMVM_CK(mmvm::list_launch(e, rec, n, c->gbox.p, c->lent.p, c->lcnt.p, lseg, c->partial.p, lfar,
-                            c->fpart.p, tr, lc, nullptr, c->errf.p, c->st));
+  const mmvm::ListArgs A = list_args(c, n, lseg, lfar, tree, lc, local, loc_seg, nullptr);
+  MMVM_CK(mmvm::list_launch(e, A, c->st));
   MMVM_CK(cudaEventRecord(e0, c->st));
-  MMVM_CK(mmvm::list_launch(e, rec, n, c->gbox.p, c->lent.p, c->lcnt.p, lseg, c->partial.p, lfar,
-                            c->fpart.p, tr, lc, nullptr, c->errf.p, c->st));
+  MMVM_CK(mmvm::list_launch(e, A, c->st));
   MMVM_CK(cudaEventRecord(e1, c->st));
   MMVM_CK(cudaEventSynchronize(e1));
   float ms = 0.f;
@@ -488,8 +537,8 @@ static int time_list_variant(mmvm_ctx* c, const mmvm::ListEntry& e, int n, bool 
   if (const char* vb = std::getenv("MMVM_TUNE_VERBOSE"))
     if (std::atoi(vb))
       std::fprintf(stderr, "[mmvm tune] M=%d n=%d list variant %d (near kernels=%d, segments=%d, "
-                   "far %s, far blocks=%d): %.3f ms, %.3e pairs/s\n", c->M, n, e.variant,
-                   e.nslices, lseg, tree ? "tree" : "flat", tree ? tfar : lfar, ms,
+                   "far %s, far blocks=%d, local %d): %.3f ms, %.3e pairs/s\n", c->M, n, e.variant,
+                   e.nslices, lseg, tree ? "tree" : "flat", tree ? tfar : lfar, local ? 1 : 0, ms,
                    (double)n * n / (ms * 1e-3));
   return MMVM_OK;
 }
@@ -510,7 +559,7 @@ int tune_pair(mmvm_ctx* c) {
   if (n <= 1 || nv + nl <= 1) return MMVM_OK;
   const auto key = std::make_tuple(c->cfg.device, c->M, c->cfg.precision, c->far ? 1 : 0,
                                    ilog2(n));
-  int choice = -1, tree_choice = -1;
+  int choice = -1, tree_choice = -1, local_choice = -1;
   if (const char* f = std::getenv("MMVM_PAIR_VARIANT")) choice = std::atoi(f);
   if (choice < 0) {
     if (const char* a = std::getenv("MMVM_AUTOTUNE"))
@@ -581,6 +630,8 @@ int tune_pair(mmvm_ctx* c) {
       }
     }
     // the list form, every variant on its full launch
+    double best_list = 1e300;
+    int best_v = -1;
     for (int v = 0; v < nl; ++v) {
       mmvm::ListEntry e = mmvm::list_entry(c->M, v);
       if (e.M != c->M) continue;
@@ -589,49 +640,84 @@ int tune_pair(mmvm_ctx* c) {
         continue;
       }
       double per_pair = 0.0;
-      int rc = time_list_variant(c, e, n, false, e0, e1, &per_pair);
+      int rc = time_list_variant(c, e, n, false, false, e0, e1, &per_pair);
       if (rc) return rc;
-      if (per_pair < best_full) {
-        best_full = per_pair;
-        choice = nv + v;
+      if (per_pair < best_list) {
+        best_list = per_pair;
+        best_v = v;
       }
     }
-    // the far field of the best list variant through the tree
+    // the best list variant with the far field through the tree, and with
+    // compact near groups through local expansions
     tree_choice = 0;
-    if (choice >= nv) {
-      mmvm::ListEntry e = mmvm::list_entry(c->M, choice - nv);
+    local_choice = 0;
+    if (best_v >= 0) {
+      mmvm::ListEntry e = mmvm::list_entry(c->M, best_v);
       double per_pair = 0.0;
-      int rc = time_list_variant(c, e, n, true, e0, e1, &per_pair);
+      int rc = time_list_variant(c, e, n, true, false, e0, e1, &per_pair);
       if (rc) return rc;
-      if (per_pair < best_full) {
-        best_full = per_pair;
+      if (per_pair < best_list) {
+        best_list = per_pair;
         tree_choice = 1;
       }
+      MMVM_CK(e.far.loc_prepare());
+      rc = time_list_variant(c, e, n, true, true, e0, e1, &per_pair);
+      if (rc) return rc;
+      if (per_pair < best_list) {
+        best_list = per_pair;
+        tree_choice = local_choice = 1;
+        // short lists of close groups remain: the variants rank differently
+        for (int v = 0; v < nl; ++v) {
+          mmvm::ListEntry ev = mmvm::list_entry(c->M, v);
+          if (v == e.variant || ev.M != c->M) continue;
+          if (mmvm::list_prepare(ev) != cudaSuccess || mmvm::list_occupancy(ev) < 1) {
+            cudaGetLastError();
+            continue;
+          }
+          rc = time_list_variant(c, ev, n, true, true, e0, e1, &per_pair);
+          if (rc) return rc;
+          if (per_pair < best_list) {
+            best_list = per_pair;
+            best_v = v;
+          }
+        }
+      }
+      if (best_list < best_full) choice = nv + best_v;
     }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     std::lock_guard<std::mutex> lk(g_tune_mu);
     g_tuned[key] = choice;
     g_tuned_tree[key] = tree_choice;
+    g_tuned_local[key] = local_choice;
   }
   if (tree_choice < 0) {
     std::lock_guard<std::mutex> lk(g_tune_mu);
     auto it = g_tuned_tree.find(key);
     tree_choice = it != g_tuned_tree.end() ? it->second : 1;
   }
+  if (local_choice < 0) {
+    std::lock_guard<std::mutex> lk(g_tune_mu);
+    auto it = g_tuned_local.find(key);
+    local_choice = it != g_tuned_local.end() ? it->second : 1;
+  }
   if (const char* f = std::getenv("MMVM_FAR_TREE")) tree_choice = std::atoi(f) != 0;
+  if (const char* f = std::getenv("MMVM_LOCAL")) local_choice = std::atoi(f) != 0;
+  if (!tree_choice) local_choice = 0;  // the far part of the local form walks the tree
   if (choice >= nv) {  // list form
     if (choice >= nv + nl) return fail(MMVM_E_INVALID_ARG, "MMVM_PAIR_VARIANT out of range");
     mmvm::ListEntry e = mmvm::list_entry(c->M, choice - nv);
     if (e.M != c->M) return fail(MMVM_E_INVALID_ARG, "MMVM_PAIR_VARIANT out of range");
     MMVM_CK(mmvm::list_prepare(e));
-    int lseg = 1, lfar = 1;
-    int rc = ensure_list_buffers(c, e, n, &lseg, &lfar);
+    if (local_choice) MMVM_CK(e.far.loc_prepare());
+    int lseg = 1, lfar = 1, loc_seg = 1;
+    int rc = ensure_list_buffers(c, e, n, local_choice != 0, &lseg, &lfar, &loc_seg);
     if (rc) return rc;
     int tfar = 1;
     const int lc = mmvm::tree_chunk_level((n + mmvm::kGroup - 1) / mmvm::kGroup, lfar, &tfar);
     if (!c->list || e.variant != c->le.variant || lseg != c->lseg || lfar != c->lfar ||
-        c->tree != (tree_choice != 0) || lc != c->lc)
+        c->tree != (tree_choice != 0) || lc != c->lc || c->local != (local_choice != 0) ||
+        loc_seg != c->loc_seg)
       c->drop_graph();
     c->le = e;
     c->list = true;
@@ -640,6 +726,8 @@ int tune_pair(mmvm_ctx* c) {
     c->tree = tree_choice != 0;
     c->lc = lc;
     c->tfar = tfar;
+    c->local = local_choice != 0;
+    c->loc_seg = loc_seg;
     return MMVM_OK;
   }
   if (c->list) c->drop_graph();
@@ -799,6 +887,9 @@ void mmvm_destroy(mmvm_ctx* c) {
                   &c->fpart})
     b->release();
   c->tnodes.release();
+  c->gexp.release();
+  c->fld.release();
+  c->ffld.release();
   c->lent.release();
   c->lcnt.release();
   c->errf.release();
@@ -1184,7 +1275,7 @@ int mmvm_pair_config(const mmvm_ctx* c, int32_t* out) {
   if (!c || !out) return fail(MMVM_E_INVALID_ARG, "null argument");
   if (c->list) {
     out[0] = mmvm::pair_variant_count(c->M, c->cfg.precision) + c->le.variant;
-    out[1] = c->le.nslices + 2;
+    out[1] = c->le.nslices + 2 + (c->local ? 4 : 0);
     out[2] = c->le.slices[0].warps * 32;
     out[3] = mmvm::list_occupancy(c->le);
     out[4] = 1;

@@ -123,6 +123,20 @@ constexpr float kM2PTheta2 = 0.01f;  // theta^2
 // Re/Im B_j for j < m2p_terms(M); padded to whole float4s.
 __host__ __device__ constexpr int gdata_len(int M) { return round_up(8 + 2 * m2p_terms(M), 4); }
 
+// Local expansions (pair_local.cuh): extra orders of a group's expansion and of
+// a target group's field (2M + extra <= 31: one lane per order), and the widest
+// group they serve.  At these radii the truncation stays below the FP32
+// rounding of the pair sums (two patches, M = 6: moment rates of n = 65536,
+// 52000 and 40000 particles off by 1.8e-7, 1.9e-7 and 2.2e-7 of FP64, 1.9e-7,
+// 2.1e-7 and 2.2e-7 pair by pair; 2 more orders change nothing, 3 fewer add
+// 50 % where most groups are near the limit).
+__host__ __device__ constexpr int loc_extra(int M) {
+  return M <= 1 ? 13 : M == 2 ? 14 : M == 3 ? 15 : M == 4 ? 16 : M <= 7 ? 17 : 15;
+}
+__host__ __device__ constexpr float loc_radius(int M) {
+  return M <= 5 ? 0.95f : M == 6 ? 0.9f : M == 7 ? 0.8f : 0.7f;
+}
+
 // Binary tree over G groups of kGroup sorted records (the far field of the
 // list form): level L has ceil(G / 2^L) nodes, node i of level L >= 1 holds
 // nodes 2i and 2i+1 of level L-1, the top level one node; the node records

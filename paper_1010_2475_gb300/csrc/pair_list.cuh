@@ -98,22 +98,51 @@ __device__ __forceinline__ bool takes_m2p(const float4 tb, const float4 c) {
 // ent[tg * G + e] = (source group, near mask), e < cnt[tg], in increasing
 // source-group order; only groups with a non-empty mask are listed.  One warp
 // per target group; groups of kGroup sorted records, the last one partial.
+// With rmax > 0 (local expansions), a near group that loc_pair takes goes to
+// the other end of the row instead, ent[tg * G + G - 1 - e], e < mcnt[tg].
+//
+// loc_pair: do the target group (centre, radius) tc and the source group sc go
+// through local expansions (pair_local.cuh)?  Both must be compact, and their
+// centres at least sqrt(kLocMinX) core units apart: the rounding of an FP32
+// expansion is shared by the 1024 pairs of two groups, where pair by pair it
+// averages out (sqrt(32) times smaller), and the closest groups' terms are the
+// largest.  At n = 65536, M = 6 (two patches) the moment rates are off by
+// 1.0e-6 (2-norm, weighted) without the limit and 1.9e-7 pair by pair; at
+// x >= 8 an expansion's share is below 5e-8, and 1 of 8 near groups is closer.
+// The products are rounded one by one so that every kernel decides alike.
+constexpr float kLocMinX = 8.f;
+__device__ __forceinline__ bool loc_pair(float rmax, const float4 tc, const float4 sc) {
+  const float dx = tc.x - sc.x, dy = tc.y - sc.y;
+  return rmax > 0.f && tc.z <= rmax && sc.z <= rmax &&
+         __fadd_rn(__fmul_rn(dx, dx), __fmul_rn(dy, dy)) >= kLocMinX;
+}
 template <int M>
 __global__ void near_list_kernel(const float* __restrict__ rec, int n, int G,
-                                 const float* __restrict__ gdata, int2* __restrict__ ent,
-                                 int* __restrict__ cnt) {
+                                 const float* __restrict__ gdata, float rmax,
+                                 int2* __restrict__ ent, int* __restrict__ cnt,
+                                 int* __restrict__ mcnt) {
   constexpr int R = rec_len<float>(M), GL = gdata_len(M);
   const int lane = threadIdx.x & 31;
   const int nwarps = (gridDim.x * blockDim.x) >> 5;
   for (int tg = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; tg < G; tg += nwarps) {
     const float4 tb = *reinterpret_cast<const float4*>(gdata + (size_t)tg * GL);
-    int c = 0;
+    const float4 tc = *reinterpret_cast<const float4*>(gdata + (size_t)tg * GL + 4);
+    int c = 0, mc = 0;
     for (int gb = 0; gb < G; gb += 32) {
       const int g = gb + lane;
       bool nearg = false;
       if (g < G) {
         const float4 sb = *reinterpret_cast<const float4*>(gdata + (size_t)g * GL);
         nearg = box_dist2(tb, sb) < x_far(M);
+      }
+      if (rmax > 0.f && tc.z <= rmax) {
+        const bool loc =
+            nearg && loc_pair(rmax, tc, *reinterpret_cast<const float4*>(gdata + (size_t)g * GL + 4));
+        const unsigned lb = __ballot_sync(0xffffffffu, loc);
+        if (loc)
+          ent[(size_t)tg * G + G - 1 - mc - __popc(lb & ((1u << lane) - 1u))] = make_int2(g, 0);
+        mc += __popc(lb);
+        nearg = nearg && !loc;
       }
       unsigned bal = __ballot_sync(0xffffffffu, nearg);
       while (bal) {
@@ -132,7 +161,10 @@ __global__ void near_list_kernel(const float* __restrict__ rec, int n, int G,
         }
       }
     }
-    if (lane == 0) cnt[tg] = c;
+    if (lane == 0) {
+      cnt[tg] = c;
+      mcnt[tg] = mc;
+    }
   }
 }
 
@@ -604,7 +636,8 @@ constexpr int kTreeStack = 32;
 template <int M>
 __global__ void __launch_bounds__(kFarWarps * 32)
     far_tree_kernel(const float* __restrict__ rec, int n, int G, const float* __restrict__ gdata,
-                    const float* __restrict__ tree, int Lc, double* __restrict__ fpart,
+                    const float* __restrict__ tree, int Lc, float rmax,
+                    double* __restrict__ fpart,
                     unsigned long long* __restrict__ counts) {
   constexpr int R = rec_len<float>(M), K = n_moments(M), HDR = Rec<float>::HDR;
   constexpr int GL = gdata_len(M), NA = m2p_terms(M), BM = bmax_of(M), NE = n_edge(M);
@@ -624,6 +657,8 @@ __global__ void __launch_bounds__(kFarWarps * 32)
     tl2 = r[3];
   }
   const float4 tb = *reinterpret_cast<const float4*>(gdata + (size_t)tg * GL);
+  const float4 tc = *reinterpret_cast<const float4*>(gdata + (size_t)tg * GL + 4);
+  if (rmax > 0.f && tc.z <= rmax) return;  // loc_far_kernel's; the finish leaves its block out
   float yhr[BM], yhi[BM], ylr[BM], yli[BM], tyr[BM], tyi[BM];
 #pragma unroll
   for (int b = 0; b < BM; ++b) {

@@ -3,7 +3,7 @@
 // -DMMVM_INST_S so the kernels compile in parallel; with -DMMVM_INST_FAR
 // instead of -DMMVM_INST_V / -DMMVM_INST_S, the list build and the far
 // kernel of order MMVM_INST_M.
-#include "pair_list.cuh"
+#include "pair_local.cuh"
 #include "pair_registry.h"
 
 #if !defined(MMVM_INST_M)
@@ -16,10 +16,10 @@ namespace mmvm {
 
 namespace {
 constexpr int kM = MMVM_INST_M;
-cudaError_t build_fn(const float* rec, int n, int G, const float* gdata, int2* ent, int* cnt,
-                     cudaStream_t st) {
+cudaError_t build_fn(const float* rec, int n, int G, const float* gdata, float rmax, int2* ent,
+                     int* cnt, int* mcnt, cudaStream_t st) {
   const int blocks = (G + 7) / 8;  // 8 warps (target groups) per block
-  near_list_kernel<kM><<<blocks, 256, 0, st>>>(rec, n, G, gdata, ent, cnt);
+  near_list_kernel<kM><<<blocks, 256, 0, st>>>(rec, n, G, gdata, rmax, ent, cnt, mcnt);
   return cudaGetLastError();
 }
 cudaError_t far_fn(const float* rec, int n, int G, const float* gdata, int S, double* fpart,
@@ -46,9 +46,36 @@ cudaError_t tree_build_fn(const float* gdata, int n, int G, float* tree, cudaStr
   return cudaSuccess;
 }
 cudaError_t far_tree_fn(const float* rec, int n, int G, const float* gdata, const float* tree,
-                        int Lc, double* fpart, unsigned long long* counts, cudaStream_t st) {
+                        int Lc, float rmax, double* fpart, unsigned long long* counts,
+                        cudaStream_t st) {
   dim3 grid((G + kFarWarps - 1) / kFarWarps, tree_level_nodes(G, Lc));
-  far_tree_kernel<kM><<<grid, kFarWarps * 32, 0, st>>>(rec, n, G, gdata, tree, Lc, fpart, counts);
+  far_tree_kernel<kM><<<grid, kFarWarps * 32, 0, st>>>(rec, n, G, gdata, tree, Lc, rmax, fpart,
+                                                    counts);
+  return cudaGetLastError();
+}
+cudaError_t loc_prepare_fn() {
+  cudaError_t e = cudaFuncSetAttribute(
+      loc_near_kernel<kM>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)LocSmem<kM>::bytes);
+  if (e != cudaSuccess) return e;
+  return cudaFuncSetAttribute(loc_far_kernel<kM>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              (int)LocFarSmem<kM>::bytes);
+}
+cudaError_t loc_far_fn(const float* rec, int n, int G, const float* gdata, const float* tree,
+                       int Lc, float2* ffld, unsigned long long* counts, cudaStream_t st) {
+  const dim3 grid((G + kLocWarps - 1) / kLocWarps, tree_level_nodes(G, Lc));
+  loc_far_kernel<kM><<<grid, kLocWarps * 32, LocFarSmem<kM>::bytes, st>>>(rec, n, G, gdata, tree,
+                                                                          Lc, ffld, counts);
+  return cudaGetLastError();
+}
+cudaError_t loc_near_fn(const float* rec, int n, int G, const float* gdata, float* gexp,
+                        const int2* ent, const int* mcnt, int C, float2* fld, int nfar,
+                        const float2* ffld, double* out, unsigned long long* counts, int* err,
+                        cudaStream_t st) {
+  const int blocks = (G + kLocWarps - 1) / kLocWarps;
+  loc_expand_kernel<kM><<<(G + 3) / 4, 128, 0, st>>>(rec, n, G, gdata, gexp);
+  loc_near_kernel<kM><<<dim3(blocks, C), kLocWarps * 32, LocSmem<kM>::bytes, st>>>(
+      n, G, gdata, gexp, ent, mcnt, C, fld, counts, err);
+  loc_eval_kernel<kM><<<(G + 3) / 4, 128, 0, st>>>(rec, n, G, gdata, C, fld, nfar, ffld, out);
   return cudaGetLastError();
 }
 }  // namespace
@@ -65,6 +92,12 @@ ListFarEntry MMVM_FAR(MMVM_INST_M)() {
   e.tree_build = tree_build_fn;
   e.far_tree = far_tree_fn;
   e.n_edge = n_edge(kM);
+  e.loc_prepare = loc_prepare_fn;
+  e.loc_far = loc_far_fn;
+  e.loc_near = loc_near_fn;
+  e.loc_len = Loc<kM>::LEN;
+  e.loc_rows = Loc<kM>::FROWS;
+  e.loc_radius = loc_radius(kM);
   return e;
 }
 

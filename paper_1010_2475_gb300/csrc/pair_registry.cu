@@ -140,20 +140,25 @@ int tree_chunk_level(int G, int blocks, int* nodes) {
   return L;
 }
 
-cudaError_t list_launch(const ListEntry& e, const float* rec, int n, const float* gdata,
-                        int2* ent, int* cnt, int C, double* partial, int S, double* fpart,
-                        float* tree, int Lc, unsigned long long* counts, int* err,
-                        cudaStream_t st, cudaEvent_t* marks) {
-  const int G = (n + kGroup - 1) / kGroup;
-  cudaError_t r = e.far.build(rec, n, G, gdata, ent, cnt, st);
-  if (tree && r == cudaSuccess) r = e.far.tree_build(gdata, n, G, tree, st);
+cudaError_t list_launch(const ListEntry& e, const ListArgs& A, cudaStream_t st,
+                        cudaEvent_t* marks) {
+  const int n = A.n, G = (n + kGroup - 1) / kGroup;
+  const float rmax = A.local && A.tree ? e.far.loc_radius : 0.f;
+  cudaError_t r = e.far.build(A.rec, n, G, A.gdata, rmax, A.ent, A.cnt, A.cnt + G, st);
+  if (A.tree && r == cudaSuccess) r = e.far.tree_build(A.gdata, n, G, A.tree, st);
   if (marks && r == cudaSuccess) r = cudaEventRecord(marks[0], st);
   if (r == cudaSuccess)
-    r = tree ? e.far.far_tree(rec, n, G, gdata, tree, Lc, fpart, counts, st)
-             : e.far.far(rec, n, G, gdata, S, fpart, counts, st);
+    r = A.tree ? e.far.far_tree(A.rec, n, G, A.gdata, A.tree, A.Lc, rmax, A.fpart, A.counts, st)
+               : e.far.far(A.rec, n, G, A.gdata, A.far_ranges, A.fpart, A.counts, st);
+  if (rmax > 0.f && r == cudaSuccess)
+    r = e.far.loc_far(A.rec, n, G, A.gdata, A.tree, A.Lc, A.ffld, A.counts, st);
   if (marks && r == cudaSuccess) r = cudaEventRecord(marks[1], st);
+  if (rmax > 0.f && r == cudaSuccess)
+    r = e.far.loc_near(A.rec, n, G, A.gdata, A.gexp, A.ent, A.cnt + G, A.loc_segments, A.fld,
+                       tree_level_nodes(G, A.Lc), A.ffld,
+                       A.partial + (size_t)A.segments * n_beta(e.M) * n, A.counts, A.err, st);
   for (int s = 0; s < e.nslices && r == cudaSuccess; ++s) {
-    r = e.slices[s].launch(rec, n, G, ent, cnt, C, partial, counts, err, st);
+    r = e.slices[s].launch(A.rec, n, G, A.ent, A.cnt, A.segments, A.partial, A.counts, A.err, st);
     if (marks && r == cudaSuccess) r = cudaEventRecord(marks[2 + s], st);
   }
   return r;

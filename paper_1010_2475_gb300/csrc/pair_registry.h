@@ -81,8 +81,10 @@ struct ListSliceEntry {
 };
 // The list build and the far kernel of one order.
 struct ListFarEntry {
-  cudaError_t (*build)(const float* rec, int n, int G, const float* gdata, int2* ent, int* cnt,
-                       cudaStream_t st) = nullptr;
+  // rmax: widest group that takes local expansions (0: none); build() lists its
+  // near groups in mcnt, far_tree() leaves its far field to loc_far()
+  cudaError_t (*build)(const float* rec, int n, int G, const float* gdata, float rmax, int2* ent,
+                       int* cnt, int* mcnt, cudaStream_t st) = nullptr;
   // grid (target groups / 4, S source ranges); fpart: S blocks [n_edge][n]
   cudaError_t (*far)(const float* rec, int n, int G, const float* gdata, int S, double* fpart,
                      unsigned long long* counts, cudaStream_t st) = nullptr;
@@ -93,9 +95,24 @@ struct ListFarEntry {
   cudaError_t (*tree_build)(const float* gdata, int n, int G, float* tree,
                             cudaStream_t st) = nullptr;
   cudaError_t (*far_tree)(const float* rec, int n, int G, const float* gdata, const float* tree,
-                          int Lc, double* fpart, unsigned long long* counts,
+                          int Lc, float rmax, double* fpart, unsigned long long* counts,
                           cudaStream_t st) = nullptr;
   int n_edge = 0;  // edge columns of a far block (2 BMAX)
+  // local expansions (pair_local.cuh): expansions of the compact groups, the
+  // fields of the target groups from C list segments, and the block `out`
+  // [NB][n] of the partial sums.  gexp: G x loc_len floats, fld: C x G x
+  // loc_rows x 32 float2, ffld: far blocks x G x 64 float2 (loc_far, one block
+  // per node of level Lc).
+  cudaError_t (*loc_prepare)() = nullptr;
+  cudaError_t (*loc_far)(const float* rec, int n, int G, const float* gdata, const float* tree,
+                         int Lc, float2* ffld, unsigned long long* counts,
+                         cudaStream_t st) = nullptr;
+  cudaError_t (*loc_near)(const float* rec, int n, int G, const float* gdata, float* gexp,
+                          const int2* ent, const int* mcnt, int C, float2* fld, int nfar,
+                          const float2* ffld, double* out, unsigned long long* counts, int* err,
+                          cudaStream_t st) = nullptr;
+  int loc_len = 0, loc_rows = 0;
+  float loc_radius = 0.f;
 };
 struct ListEntry {
   int M = -1;  // -1: no such variant
@@ -111,18 +128,33 @@ ListEntry list_entry(int M, int v);
 cudaError_t list_prepare(const ListEntry& e);
 // CTAs per SM of the near kernels (the smallest), 0 on error.
 int list_occupancy(const ListEntry& e);
-// The whole list form of one right-hand side: list build, far field, near
-// kernels (C list segments into partial).  ent: G x G entries, cnt: G counts
-// (G = groups of kGroup records).  Far field: tree == nullptr: the flat far
-// kernel over S source ranges; else the tree (tree_nodes(G) node records)
-// built and walked from the nodes of level Lc (tree_level_nodes(G, Lc) far
-// blocks; S is ignored).
+// Buffers and shape of one list-form evaluation.
+struct ListArgs {
+  const float* rec = nullptr;
+  int n = 0;
+  const float* gdata = nullptr;
+  int2* ent = nullptr;       // G x G entries (G = groups of kGroup records)
+  int* cnt = nullptr;        // G near counts, then G local counts
+  int segments = 1;          // list segments of the near kernels
+  double* partial = nullptr; // segments (+ 1 with local expansions) blocks [NB][n]
+  int far_ranges = 1;        // source ranges of the flat far kernel
+  double* fpart = nullptr;   // far blocks [n_edge][n]
+  float* tree = nullptr;     // node records (null: the flat far kernel)
+  int Lc = 0;                // level the tree is walked from (one far block per node)
+  bool local = false;        // compact groups through local expansions (with the tree)
+  int loc_segments = 1;
+  float* gexp = nullptr;
+  float2 *fld = nullptr, *ffld = nullptr;
+  unsigned long long* counts = nullptr;
+  int* err = nullptr;
+};
+// The whole list form of one right-hand side: list build, far field, local
+// expansions, near kernels.
 // marks (nullable, 2 + nslices events): recorded after the list build and
-// tree, after the far kernel and after each near kernel (per-kernel timing).
-cudaError_t list_launch(const ListEntry& e, const float* rec, int n, const float* gdata,
-                        int2* ent, int* cnt, int C, double* partial, int S, double* fpart,
-                        float* tree, int Lc, unsigned long long* counts, int* err,
-                        cudaStream_t st, cudaEvent_t* marks = nullptr);
+// tree, after the far kernel, and after each near kernel (the local expansions
+// count to the first).
+cudaError_t list_launch(const ListEntry& e, const ListArgs& A, cudaStream_t st,
+                        cudaEvent_t* marks = nullptr);
 // Node records of levels >= 1 of the tree over G groups.
 long long tree_nodes(int G);
 // Level whose node count is closest to (not above) `blocks`, and its count.

@@ -231,7 +231,9 @@ __device__ __forceinline__ void finish_block(const FinishArgs& A, int j0, int k0
     double v = 0.0;
     if (j < A.n && A.partial) {
       for (int ch = 0; ch < A.nchunks; ++ch) v += A.partial[((size_t)ch * NB + b) * A.n + j];
-      if (A.fpart) {  // far field of the list form: edge columns only
+      // far field of the list form: edge columns only
+      if (A.fpart &&
+          !(A.rmax > 0.f && A.gdata[(size_t)(j / kGroup) * A.gdata_len + 6] <= A.rmax)) {
         int bn = 1;
         while (tri(bn + 1) - 1 <= b) ++bn;
         const int b1 = bn - (b + 1 - tri(bn));

@@ -16,6 +16,9 @@ struct FinishArgs {
   const double* partial = nullptr;  // [nchunks][NB][n] by sorted position
   const double* fpart = nullptr;    // far-field blocks [nfar][n_edge][n] (list form; nullable):
   int nfar = 0, n_edge = 0;         // edge column e = 2 (|beta| - 1) + beta1, beta1 <= 1
+  const float* gdata = nullptr;     // with rmax > 0: group records of gdata_len floats; groups of
+  int gdata_len = 0;                // radius <= rmax have no far blocks (local expansions)
+  float rmax = 0.f;
   const int* perm = nullptr;        // sorted position -> particle (null: identity)
   const double* Min = nullptr;      // stage moments (n x K)
   FinishTab tab;                    // finish tables (tables.h)
