@@ -124,17 +124,24 @@ constexpr float kM2PTheta2 = 0.01f;  // theta^2
 __host__ __device__ constexpr int gdata_len(int M) { return round_up(8 + 2 * m2p_terms(M), 4); }
 
 // Local expansions (pair_local.cuh): extra orders of a group's expansion and of
-// a target group's field (2M + extra <= 31: one lane per order), and the widest
-// group they serve.  At these radii the truncation stays below the FP32
-// rounding of the pair sums (two patches, M = 6: moment rates of n = 65536,
-// 52000 and 40000 particles off by 1.8e-7, 1.9e-7 and 2.2e-7 of FP64, 1.9e-7,
-// 2.1e-7 and 2.2e-7 pair by pair; 2 more orders change nothing, 3 fewer add
-// 50 % where most groups are near the limit).
+// a target group's field (2M + extra <= 31: one lane per order), the widest
+// group they serve, and the least separation x = |t0 - s0|^2 of two groups, the
+// wider of radius r: the further apart, the faster the expansions converge.
+// Measured against FP64 on two patches and disks (2-norm of the moment rates,
+// with / without expansions): M = 6, n = 65536: 1.8e-7 / 1.9e-7, n = 40000:
+// 2.1e-7 / 2.1e-7, M = 4 disk, n = 8192: 2.7e-7 / 3.3e-7.  A limit of 2.0 at
+// M = 6 lets single particles reach 7e-6 (n = 8192), 1.4 at M = 8 1e-4.
 __host__ __device__ constexpr int loc_extra(int M) {
   return M <= 1 ? 13 : M == 2 ? 14 : M == 3 ? 15 : M == 4 ? 16 : M <= 7 ? 17 : 15;
 }
 __host__ __device__ constexpr float loc_radius(int M) {
-  return M <= 5 ? 0.95f : M == 6 ? 0.9f : M == 7 ? 0.8f : 0.7f;
+  return M <= 5 ? 2.0f : M == 6 ? 1.7f : M == 7 ? 1.1f : 0.85f;
+}
+__host__ __device__ constexpr float loc_core(int M) {  // up to this radius kLocMinX is enough
+  return M <= 6 ? 0.9f : M == 7 ? 0.8f : 0.7f;
+}
+__host__ __device__ constexpr float loc_slope(int M) {  // of the least x beyond loc_core
+  return M <= 5 ? 40.f : M == 6 ? 50.f : M == 7 ? 80.f : 100.f;
 }
 
 // Binary tree over G groups of kGroup sorted records (the far field of the

@@ -103,7 +103,8 @@ __device__ __forceinline__ bool takes_m2p(const float4 tb, const float4 c) {
 //
 // loc_pair: do the target group (centre, radius) tc and the source group sc go
 // through local expansions (pair_local.cuh)?  Both must be compact, and their
-// centres at least sqrt(kLocMinX) core units apart: the rounding of an FP32
+// centres far enough apart: beyond loc_core for the truncation (common.cuh), and
+// at least sqrt(kLocMinX) core units because the rounding of an FP32
 // expansion is shared by the 1024 pairs of two groups, where pair by pair it
 // averages out (sqrt(32) times smaller), and the closest groups' terms are the
 // largest.  At n = 65536, M = 6 (two patches) the moment rates are off by
@@ -111,10 +112,13 @@ __device__ __forceinline__ bool takes_m2p(const float4 tb, const float4 c) {
 // x >= 8 an expansion's share is below 5e-8, and 1 of 8 near groups is closer.
 // The products are rounded one by one so that every kernel decides alike.
 constexpr float kLocMinX = 8.f;
+template <int M>
 __device__ __forceinline__ bool loc_pair(float rmax, const float4 tc, const float4 sc) {
   const float dx = tc.x - sc.x, dy = tc.y - sc.y;
-  return rmax > 0.f && tc.z <= rmax && sc.z <= rmax &&
-         __fadd_rn(__fmul_rn(dx, dx), __fmul_rn(dy, dy)) >= kLocMinX;
+  const float r = fmaxf(tc.z, sc.z);
+  const float xmin =
+      __fadd_rn(kLocMinX, __fmul_rn(loc_slope(M), fmaxf(__fsub_rn(r, loc_core(M)), 0.f)));
+  return rmax > 0.f && r <= rmax && __fadd_rn(__fmul_rn(dx, dx), __fmul_rn(dy, dy)) >= xmin;
 }
 template <int M>
 __global__ void near_list_kernel(const float* __restrict__ rec, int n, int G,
@@ -137,7 +141,7 @@ __global__ void near_list_kernel(const float* __restrict__ rec, int n, int G,
       }
       if (rmax > 0.f && tc.z <= rmax) {
         const bool loc =
-            nearg && loc_pair(rmax, tc, *reinterpret_cast<const float4*>(gdata + (size_t)g * GL + 4));
+            nearg && loc_pair<M>(rmax, tc, *reinterpret_cast<const float4*>(gdata + (size_t)g * GL + 4));
         const unsigned lb = __ballot_sync(0xffffffffu, loc);
         if (loc)
           ent[(size_t)tg * G + G - 1 - mc - __popc(lb & ((1u << lane) - 1u))] = make_int2(g, 0);

@@ -700,7 +700,7 @@ __global__ void __launch_bounds__(kLocWarps * 32)
       __syncwarp();
       continue;
     }
-    if (!far_box && loc_pair(rmax, tc, cen)) continue;  // a near group of loc_near_kernel
+    if (!far_box && loc_pair<M>(rmax, tc, cen)) continue;  // a near group of loc_near_kernel
     // source by source, as in far_tree_kernel
     const int nsrc = min(kGroup, n - i * kGroup);
     const float* r = rec + (size_t)(i * kGroup + min(lane, nsrc - 1)) * R;
