@@ -202,7 +202,10 @@ void list_shape(const mmvm_ctx* c, const mmvm::ListEntry& e, int64_t n, int* lse
   }
   const int64_t warp_slots = (int64_t)dev_sms * std::max(focc, 1) * 4;
   int64_t far = (8 * warp_slots + G - 1) / G;
-  far = std::min<int64_t>(far, std::max<int64_t>(1, G / 16));
+  // at least 16 source groups per warp, 2 in small problems (a warp's serial
+  // chain over its sources is what they wait for)
+  far = std::min<int64_t>(far, G < 512 ? std::min<int64_t>((G + 1) / 2, 32)
+                                       : std::max<int64_t>(1, G / 16));
   if (const char* f = std::getenv("MMVM_FAR_RANGES")) far = std::atoi(f);  // measurement override
   *lfar = (int)std::min<int64_t>(std::max<int64_t>(far, 1), 64);
 }
@@ -414,7 +417,7 @@ int enqueue_rhs(mmvm_ctx* c, int mode, const double* xin, const double* min_, do
     if (c->local) {  // groups with a local field have no far block
       A.gdata = c->gbox.p;
       A.gdata_len = mmvm::gdata_len(c->M);
-      A.rmax = c->le.far.loc_radius;
+      A.rmax = c->le.far.loc_field_radius;
     }
   }
   A.partial = n > 1 ? c->partial.p : nullptr;
@@ -491,7 +494,7 @@ static int ensure_list_buffers(mmvm_ctx* c, const mmvm::ListEntry& e, int n, boo
   if (local) {
     const size_t ge = (size_t)G * e.far.loc_len;
     const size_t fl = (size_t)*loc_seg * G * e.far.loc_rows * 32;
-    const size_t ff = (size_t)*lfar * G * 64;  // at most lfar nodes on the tree's start level
+    const size_t ff = (size_t)*lfar * G * 64;  // at most lfar far blocks
     if (ge > c->gexp.cap || !c->gexp.p || fl > c->fld.cap || !c->fld.p || ff > c->ffld.cap ||
         !c->ffld.p) {
       MMVM_CK(c->gexp.ensure(std::max(ge, c->gexp.cap)));
@@ -661,25 +664,28 @@ int tune_pair(mmvm_ctx* c) {
         tree_choice = 1;
       }
       MMVM_CK(e.far.loc_prepare());
-      rc = time_list_variant(c, e, n, true, true, e0, e1, &per_pair);
-      if (rc) return rc;
-      if (per_pair < best_list) {
-        best_list = per_pair;
-        tree_choice = local_choice = 1;
-        // short lists of close groups remain: the variants rank differently
-        for (int v = 0; v < nl; ++v) {
-          mmvm::ListEntry ev = mmvm::list_entry(c->M, v);
-          if (v == e.variant || ev.M != c->M) continue;
-          if (mmvm::list_prepare(ev) != cudaSuccess || mmvm::list_occupancy(ev) < 1) {
-            cudaGetLastError();
-            continue;
-          }
-          rc = time_list_variant(c, ev, n, true, true, e0, e1, &per_pair);
-          if (rc) return rc;
-          if (per_pair < best_list) {
-            best_list = per_pair;
-            best_v = v;
-          }
+      for (int tree = 0; tree < 2; ++tree) {
+        rc = time_list_variant(c, e, n, tree != 0, true, e0, e1, &per_pair);
+        if (rc) return rc;
+        if (per_pair < best_list) {
+          best_list = per_pair;
+          tree_choice = tree;
+          local_choice = 1;
+        }
+      }
+      // shorter lists of close groups remain: the variants rank differently
+      for (int v = 0; v < nl && local_choice; ++v) {
+        mmvm::ListEntry ev = mmvm::list_entry(c->M, v);
+        if (v == e.variant || ev.M != c->M) continue;
+        if (mmvm::list_prepare(ev) != cudaSuccess || mmvm::list_occupancy(ev) < 1) {
+          cudaGetLastError();
+          continue;
+        }
+        rc = time_list_variant(c, ev, n, tree_choice != 0, true, e0, e1, &per_pair);
+        if (rc) return rc;
+        if (per_pair < best_list) {
+          best_list = per_pair;
+          best_v = v;
         }
       }
       if (best_list < best_full) choice = nv + best_v;
@@ -703,7 +709,6 @@ int tune_pair(mmvm_ctx* c) {
   }
   if (const char* f = std::getenv("MMVM_FAR_TREE")) tree_choice = std::atoi(f) != 0;
   if (const char* f = std::getenv("MMVM_LOCAL")) local_choice = std::atoi(f) != 0;
-  if (!tree_choice) local_choice = 0;  // the far part of the local form walks the tree
   if (choice >= nv) {  // list form
     if (choice >= nv + nl) return fail(MMVM_E_INVALID_ARG, "MMVM_PAIR_VARIANT out of range");
     mmvm::ListEntry e = mmvm::list_entry(c->M, choice - nv);

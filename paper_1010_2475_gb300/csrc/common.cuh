@@ -137,6 +137,13 @@ __host__ __device__ constexpr int loc_extra(int M) {
 __host__ __device__ constexpr float loc_radius(int M) {
   return M <= 5 ? 2.0f : M == 6 ? 1.7f : M == 7 ? 1.1f : 0.85f;
 }
+// Widest target group whose far field is taken through its local field: at
+// most 0.3 of the distance to anything beyond x_far(M), so that the Taylor
+// series about its centre loses less than FP32 rounding.
+__host__ __device__ constexpr float loc_field_radius(int M) {
+  return M <= 0 ? 2.0f : M == 1 ? 2.3f : M == 2 ? 2.5f : M == 3 ? 2.8f : M == 4 ? 3.0f
+       : M == 5 ? 3.2f : M == 6 ? 3.4f : M == 7 ? 3.4f : 3.2f;
+}
 __host__ __device__ constexpr float loc_core(int M) {  // up to this radius kLocMinX is enough
   return M <= 6 ? 0.9f : M == 7 ? 0.8f : 0.7f;
 }

@@ -420,7 +420,8 @@ __device__ __forceinline__ void two_sum_into(float& hi, float& lo, float v) {
 template <int M>
 __global__ void __launch_bounds__(kFarWarps * 32)
     far_pair_kernel(const float* __restrict__ rec, int n, int G, const float* __restrict__ gdata,
-                    int S, double* __restrict__ fpart, unsigned long long* __restrict__ counts) {
+                    int S, float frad, double* __restrict__ fpart,
+                    unsigned long long* __restrict__ counts) {
   constexpr int R = rec_len<float>(M), K = n_moments(M), HDR = Rec<float>::HDR;
   constexpr int GL = gdata_len(M), NA = m2p_terms(M), BM = bmax_of(M), NE = n_edge(M);
   constexpr int NF = 2 * (M + 1);  // floats of a source's multipoles A'_n
@@ -439,6 +440,8 @@ __global__ void __launch_bounds__(kFarWarps * 32)
     tl2 = r[3];
   }
   const float4 tb = *reinterpret_cast<const float4*>(gdata + (size_t)tg * GL);
+  // a group with a local field is loc_far_kernel's; the finish leaves its block out
+  if (frad > 0.f && gdata[(size_t)tg * GL + 6] <= frad) return;
   float yhr[BM], yhi[BM], ylr[BM], yli[BM], tyr[BM], tyi[BM];
 #pragma unroll
   for (int b = 0; b < BM; ++b) {
@@ -640,7 +643,7 @@ constexpr int kTreeStack = 32;
 template <int M>
 __global__ void __launch_bounds__(kFarWarps * 32)
     far_tree_kernel(const float* __restrict__ rec, int n, int G, const float* __restrict__ gdata,
-                    const float* __restrict__ tree, int Lc, float rmax,
+                    const float* __restrict__ tree, int Lc, float frad,
                     double* __restrict__ fpart,
                     unsigned long long* __restrict__ counts) {
   constexpr int R = rec_len<float>(M), K = n_moments(M), HDR = Rec<float>::HDR;
@@ -661,8 +664,7 @@ __global__ void __launch_bounds__(kFarWarps * 32)
     tl2 = r[3];
   }
   const float4 tb = *reinterpret_cast<const float4*>(gdata + (size_t)tg * GL);
-  const float4 tc = *reinterpret_cast<const float4*>(gdata + (size_t)tg * GL + 4);
-  if (rmax > 0.f && tc.z <= rmax) return;  // loc_far_kernel's; the finish leaves its block out
+  if (frad > 0.f && gdata[(size_t)tg * GL + 6] <= frad) return;  // as in far_pair_kernel
   float yhr[BM], yhi[BM], ylr[BM], yli[BM], tyr[BM], tyi[BM];
 #pragma unroll
   for (int b = 0; b < BM; ++b) {

@@ -22,10 +22,10 @@ cudaError_t build_fn(const float* rec, int n, int G, const float* gdata, float r
   near_list_kernel<kM><<<blocks, 256, 0, st>>>(rec, n, G, gdata, rmax, ent, cnt, mcnt);
   return cudaGetLastError();
 }
-cudaError_t far_fn(const float* rec, int n, int G, const float* gdata, int S, double* fpart,
-                   unsigned long long* counts, cudaStream_t st) {
+cudaError_t far_fn(const float* rec, int n, int G, const float* gdata, int S, float frad,
+                   double* fpart, unsigned long long* counts, cudaStream_t st) {
   dim3 grid((G + kFarWarps - 1) / kFarWarps, S);
-  far_pair_kernel<kM><<<grid, kFarWarps * 32, 0, st>>>(rec, n, G, gdata, S, fpart, counts);
+  far_pair_kernel<kM><<<grid, kFarWarps * 32, 0, st>>>(rec, n, G, gdata, S, frad, fpart, counts);
   return cudaGetLastError();
 }
 cudaError_t far_occ_fn(int* blocks) {
@@ -46,10 +46,10 @@ cudaError_t tree_build_fn(const float* gdata, int n, int G, float* tree, cudaStr
   return cudaSuccess;
 }
 cudaError_t far_tree_fn(const float* rec, int n, int G, const float* gdata, const float* tree,
-                        int Lc, float rmax, double* fpart, unsigned long long* counts,
+                        int Lc, float frad, double* fpart, unsigned long long* counts,
                         cudaStream_t st) {
   dim3 grid((G + kFarWarps - 1) / kFarWarps, tree_level_nodes(G, Lc));
-  far_tree_kernel<kM><<<grid, kFarWarps * 32, 0, st>>>(rec, n, G, gdata, tree, Lc, rmax, fpart,
+  far_tree_kernel<kM><<<grid, kFarWarps * 32, 0, st>>>(rec, n, G, gdata, tree, Lc, frad, fpart,
                                                     counts);
   return cudaGetLastError();
 }
@@ -61,10 +61,11 @@ cudaError_t loc_prepare_fn() {
                               (int)LocFarSmem<kM>::bytes);
 }
 cudaError_t loc_far_fn(const float* rec, int n, int G, const float* gdata, const float* tree,
-                       int Lc, float2* ffld, unsigned long long* counts, cudaStream_t st) {
-  const dim3 grid((G + kLocWarps - 1) / kLocWarps, tree_level_nodes(G, Lc));
-  loc_far_kernel<kM><<<grid, kLocWarps * 32, LocFarSmem<kM>::bytes, st>>>(rec, n, G, gdata, tree,
-                                                                          Lc, ffld, counts);
+                       int Lc, int S, float2* ffld, unsigned long long* counts,
+                       cudaStream_t st) {
+  const dim3 grid((G + kLocWarps - 1) / kLocWarps, tree ? tree_level_nodes(G, Lc) : S);
+  loc_far_kernel<kM><<<grid, kLocWarps * 32, LocFarSmem<kM>::bytes, st>>>(
+      rec, n, G, gdata, tree, Lc, S, ffld, counts);
   return cudaGetLastError();
 }
 cudaError_t loc_near_fn(const float* rec, int n, int G, const float* gdata, float* gexp,
@@ -98,6 +99,7 @@ ListFarEntry MMVM_FAR(MMVM_INST_M)() {
   e.loc_len = Loc<kM>::LEN;
   e.loc_rows = Loc<kM>::FROWS;
   e.loc_radius = loc_radius(kM);
+  e.loc_field_radius = loc_field_radius(kM);
   return e;
 }
 

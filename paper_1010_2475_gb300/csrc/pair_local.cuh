@@ -555,7 +555,7 @@ __global__ void __launch_bounds__(kLocWarps * 32, 2)
 
 // ------------------------------------------------------------------ far field
 // The far field of the target groups that take local expansions, as in
-// far_tree_kernel (the same walk, the same criteria) but summed into the edge
+// far_tree_kernel and far_pair_kernel (the same walk, the same criteria) but summed into the edge
 // rows of the group's field instead of target by target: a node costs 4 (NA)
 // multiply-adds per lane instead of 2902 flops per target, a far source 4 (M +
 // 1) instead of 838 flops per target.  The lanes first form the point-vortex
@@ -577,13 +577,13 @@ struct LocFarSmem {
 template <int M>
 __global__ void __launch_bounds__(kLocWarps * 32)
     loc_far_kernel(const float* __restrict__ rec, int n, int G, const float* __restrict__ gdata,
-                   const float* __restrict__ tree, int Lc, float2* __restrict__ ffld,
+                   const float* __restrict__ tree, int Lc, int S, float2* __restrict__ ffld,
                    unsigned long long* __restrict__ counts) {
   using L = Loc<M>;
   using SM = LocFarSmem<M>;
   constexpr int R = rec_len<float>(M), K = n_moments(M), HDR = Rec<float>::HDR;
   constexpr int GL = gdata_len(M), NA = SM::NA, ST = SM::ST, NL = L::NL;
-  constexpr float rmax = loc_radius(M);
+  constexpr float rmax = loc_radius(M);  // near groups (loc_pair)
   extern __shared__ __align__(16) unsigned char smem_lf[];
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
   unsigned char* base = smem_lf + (size_t)w * SM::warp;
@@ -595,7 +595,7 @@ __global__ void __launch_bounds__(kLocWarps * 32)
   if (tg >= G) return;  // whole warps, no CTA barrier
   const float4 tb = *reinterpret_cast<const float4*>(gdata + (size_t)tg * GL);
   const float4 tc = *reinterpret_cast<const float4*>(gdata + (size_t)tg * GL + 4);
-  if (!(tc.z <= rmax)) return;  // far_tree_kernel's
+  if (!(tc.z <= loc_field_radius(M))) return;  // the target-by-target far kernels'
   for (int i = lane; i < 2 * SM::ROWS * ST; i += 32) te[i] = 0.f;
   __syncwarp();
   float h0 = 0.f, q0 = 0.f, h1 = 0.f, q1 = 0.f;  // edge rows E0, E1 of this lane's order
@@ -672,11 +672,19 @@ __global__ void __launch_bounds__(kLocWarps * 32)
     __syncwarp();
   };
   unsigned n_far = 0, n_m2p = 0, n_m2p_pairs = 0;
-  int sp = 1;
-  if (lane == 0) stack[0] = (Lc << kTreeShift) | blockIdx.y;
+  // the walk from node blockIdx.y of level Lc, or (no tree) the groups of
+  // source range blockIdx.y one after another
+  int sp = 0, gnext = 0, gend = 0;
+  if (tree != nullptr) {
+    if (lane == 0) stack[0] = (Lc << kTreeShift) | blockIdx.y;
+    sp = 1;
+  } else {
+    gnext = (int)((long long)blockIdx.y * G / S);
+    gend = (int)((long long)(blockIdx.y + 1) * G / S);
+  }
   __syncwarp();
-  while (sp > 0) {
-    const int top = stack[--sp];
+  while (sp > 0 || gnext < gend) {
+    const int top = sp > 0 ? stack[--sp] : gnext++;
     __syncwarp();
     const int Lv = top >> kTreeShift, i = top & ((1 << kTreeShift) - 1);
     const float* nd = node_rec(Lv, i);
@@ -761,7 +769,7 @@ __global__ void __launch_bounds__(128)
   if (tg >= G) return;  // whole warps
   const int j = tg * kGroup + lane;
   const float4 cen = *reinterpret_cast<const float4*>(gdata + (size_t)tg * GL + 4);
-  if (!(cen.z <= loc_radius(M))) {
+  if (!(cen.z <= loc_field_radius(M))) {
     if (j < n)
       for (int b = 0; b < NB; ++b) out[(size_t)b * n + j] = 0.0;
     return;

@@ -143,19 +143,20 @@ int tree_chunk_level(int G, int blocks, int* nodes) {
 cudaError_t list_launch(const ListEntry& e, const ListArgs& A, cudaStream_t st,
                         cudaEvent_t* marks) {
   const int n = A.n, G = (n + kGroup - 1) / kGroup;
-  const float rmax = A.local && A.tree ? e.far.loc_radius : 0.f;
+  const float rmax = A.local ? e.far.loc_radius : 0.f;
+  const float frad = A.local ? e.far.loc_field_radius : 0.f;
   cudaError_t r = e.far.build(A.rec, n, G, A.gdata, rmax, A.ent, A.cnt, A.cnt + G, st);
   if (A.tree && r == cudaSuccess) r = e.far.tree_build(A.gdata, n, G, A.tree, st);
   if (marks && r == cudaSuccess) r = cudaEventRecord(marks[0], st);
   if (r == cudaSuccess)
-    r = A.tree ? e.far.far_tree(A.rec, n, G, A.gdata, A.tree, A.Lc, rmax, A.fpart, A.counts, st)
-               : e.far.far(A.rec, n, G, A.gdata, A.far_ranges, A.fpart, A.counts, st);
-  if (rmax > 0.f && r == cudaSuccess)
-    r = e.far.loc_far(A.rec, n, G, A.gdata, A.tree, A.Lc, A.ffld, A.counts, st);
+    r = A.tree ? e.far.far_tree(A.rec, n, G, A.gdata, A.tree, A.Lc, frad, A.fpart, A.counts, st)
+               : e.far.far(A.rec, n, G, A.gdata, A.far_ranges, frad, A.fpart, A.counts, st);
+  if (A.local && r == cudaSuccess)
+    r = e.far.loc_far(A.rec, n, G, A.gdata, A.tree, A.Lc, A.far_ranges, A.ffld, A.counts, st);
   if (marks && r == cudaSuccess) r = cudaEventRecord(marks[1], st);
-  if (rmax > 0.f && r == cudaSuccess)
+  if (A.local && r == cudaSuccess)
     r = e.far.loc_near(A.rec, n, G, A.gdata, A.gexp, A.ent, A.cnt + G, A.loc_segments, A.fld,
-                       tree_level_nodes(G, A.Lc), A.ffld,
+                       A.tree ? tree_level_nodes(G, A.Lc) : A.far_ranges, A.ffld,
                        A.partial + (size_t)A.segments * n_beta(e.M) * n, A.counts, A.err, st);
   for (int s = 0; s < e.nslices && r == cudaSuccess; ++s) {
     r = e.slices[s].launch(A.rec, n, G, A.ent, A.cnt, A.segments, A.partial, A.counts, A.err, st);

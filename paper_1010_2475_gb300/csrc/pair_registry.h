@@ -81,13 +81,14 @@ struct ListSliceEntry {
 };
 // The list build and the far kernel of one order.
 struct ListFarEntry {
-  // rmax: widest group that takes local expansions (0: none); build() lists its
-  // near groups in mcnt, far_tree() leaves its far field to loc_far()
+  // rmax: widest group whose near groups build() lists for the local expansions
+  // in mcnt (0: none); frad: widest target group whose far field far() and
+  // far_tree() leave to loc_far() (0: none)
   cudaError_t (*build)(const float* rec, int n, int G, const float* gdata, float rmax, int2* ent,
                        int* cnt, int* mcnt, cudaStream_t st) = nullptr;
   // grid (target groups / 4, S source ranges); fpart: S blocks [n_edge][n]
-  cudaError_t (*far)(const float* rec, int n, int G, const float* gdata, int S, double* fpart,
-                     unsigned long long* counts, cudaStream_t st) = nullptr;
+  cudaError_t (*far)(const float* rec, int n, int G, const float* gdata, int S, float frad,
+                     double* fpart, unsigned long long* counts, cudaStream_t st) = nullptr;
   cudaError_t (*far_occupancy)(int* blocks_per_sm) = nullptr;
   // the tree over the groups (node storage: tree_nodes(G) records of
   // gdata_len(M) floats) and the far kernel walking it from the nodes of
@@ -95,24 +96,24 @@ struct ListFarEntry {
   cudaError_t (*tree_build)(const float* gdata, int n, int G, float* tree,
                             cudaStream_t st) = nullptr;
   cudaError_t (*far_tree)(const float* rec, int n, int G, const float* gdata, const float* tree,
-                          int Lc, float rmax, double* fpart, unsigned long long* counts,
+                          int Lc, float frad, double* fpart, unsigned long long* counts,
                           cudaStream_t st) = nullptr;
   int n_edge = 0;  // edge columns of a far block (2 BMAX)
   // local expansions (pair_local.cuh): expansions of the compact groups, the
   // fields of the target groups from C list segments, and the block `out`
   // [NB][n] of the partial sums.  gexp: G x loc_len floats, fld: C x G x
   // loc_rows x 32 float2, ffld: far blocks x G x 64 float2 (loc_far, one block
-  // per node of level Lc).
+  // per node of level Lc, or without a tree one per source range of S).
   cudaError_t (*loc_prepare)() = nullptr;
   cudaError_t (*loc_far)(const float* rec, int n, int G, const float* gdata, const float* tree,
-                         int Lc, float2* ffld, unsigned long long* counts,
+                         int Lc, int S, float2* ffld, unsigned long long* counts,
                          cudaStream_t st) = nullptr;
   cudaError_t (*loc_near)(const float* rec, int n, int G, const float* gdata, float* gexp,
                           const int2* ent, const int* mcnt, int C, float2* fld, int nfar,
                           const float2* ffld, double* out, unsigned long long* counts, int* err,
                           cudaStream_t st) = nullptr;
   int loc_len = 0, loc_rows = 0;
-  float loc_radius = 0.f;
+  float loc_radius = 0.f, loc_field_radius = 0.f;
 };
 struct ListEntry {
   int M = -1;  // -1: no such variant
@@ -141,7 +142,7 @@ struct ListArgs {
   double* fpart = nullptr;   // far blocks [n_edge][n]
   float* tree = nullptr;     // node records (null: the flat far kernel)
   int Lc = 0;                // level the tree is walked from (one far block per node)
-  bool local = false;        // compact groups through local expansions (with the tree)
+  bool local = false;        // compact groups through local expansions
   int loc_segments = 1;
   float* gexp = nullptr;
   float2 *fld = nullptr, *ffld = nullptr;

@@ -230,6 +230,7 @@ __device__ __forceinline__ void finish_block(const FinishArgs& A, int j0, int k0
     const int tt = idx % TG, b = idx / TG, j = j0 + tt;
     double v = 0.0;
     if (j < A.n && A.partial) {
+#pragma unroll 8
       for (int ch = 0; ch < A.nchunks; ++ch) v += A.partial[((size_t)ch * NB + b) * A.n + j];
       // far field of the list form: edge columns only
       if (A.fpart &&
@@ -239,6 +240,7 @@ __device__ __forceinline__ void finish_block(const FinishArgs& A, int j0, int k0
         const int b1 = bn - (b + 1 - tri(bn));
         if (b1 <= 1) {
           const int e = 2 * (bn - 1) + b1;
+#pragma unroll 8
           for (int ch = 0; ch < A.nfar; ++ch) v += A.fpart[((size_t)ch * A.n_edge + e) * A.n + j];
         }
       }
@@ -638,8 +640,7 @@ int finish_targets(int n, int sms) {
 cudaError_t launch_finish(const FinishArgs& A, int sms, cudaStream_t st) {
   const int TG = finish_targets(A.n, sms);
   const int rb = A.n == 1 ? A.tab.nrb : 1;
-  // row blocks hold a part of the pieces each; the bound covers any of them
-  const size_t smem = finish_smem_bytes(A.M, TG, A.tab.np);
+  const size_t smem = finish_smem_bytes(A.M, TG, rb > 1 ? A.tab.rb_pieces : A.tab.np);
   return with_targets(TG, [&](auto tg) {
     constexpr int T = decltype(tg)::value;
     if (smem > 48 * 1024) {

@@ -49,12 +49,24 @@ __device__ __forceinline__ int order_of_col(int col) {  // total order of column
   return s;
 }
 
+// c^{e/2} by repeated squaring (e may be negative): a few roundings, and a
+// fraction of the FP64 operations of pow().
+__device__ __forceinline__ double half_power(double c, int e) {
+  const double b = e < 0 ? 1.0 / c : c;
+  const int h = e < 0 ? -e : e;
+  double v = (h & 1) ? sqrt(b) : 1.0, q = b;
+  for (int i = h >> 1; i; i >>= 1) {
+    if (i & 1) v *= q;
+    q *= q;
+  }
+  return v;
+}
+
 // a_m = M_m c^{-|m|/2}
 __global__ void self_scale_kernel(SelfHighArgs A) {
   const int m = blockIdx.x * blockDim.x + threadIdx.x;
   if (m >= A.K) return;
-  const double c = stage_c_high(A);
-  A.at[m] = A.Min[m] * pow(c, -0.5 * order_of_col(m));
+  A.at[m] = A.Min[m] * half_power(stage_c_high(A), -order_of_col(m));
 }
 
 // Psi[beta] = sum_m a_m psi0[m + beta] for 1 <= |beta| <= 2M (psi0 vanishes at
@@ -67,6 +79,7 @@ __global__ void self_psi_kernel(SelfHighArgs A) {
   const int bn = order_of_col(b + 1);  // bcol(b1, b2) = tri(|beta|) + b2 - 1
   const int b2 = b + 1 - tri(bn), b1 = bn - b2;
   double acc = 0.0;
+#pragma unroll 4
   for (int m1 = b1 & 1; m1 <= A.M; m1 += 2)
     for (int m2 = (b2 & 1) + 2 * lane; m1 + m2 <= A.M; m2 += 64) {
       const int a1 = m1 + b1, a2 = m2 + b2;
@@ -90,12 +103,14 @@ __global__ void self_pass1_kernel(SelfHighArgs A) {
   // C(l2, q) g(k2 - q) and C(l2, q) g(k2 - 1 - q), q = 0, 1, ...
   const double* c1 = A.cg + ((size_t)l2 * (M + 1) + k2) * (M + 1);
   double u1 = 0.0, u2 = 0.0;
+#pragma unroll 4
   for (int q = 0; q <= min(l2, k2); ++q) {
     const int bb2 = k2 + l2 - 2 * q + 1;
     if (b1 + bb2 <= 2 * M) u1 = fma(c1[q], A.Psi[bcol(b1, bb2)], u1);
   }
   if (k2 >= 1) {
     const double* c2 = c1 - (M + 1);
+#pragma unroll 4
     for (int q = 0; q <= min(l2, k2 - 1); ++q) {
       const int bb2 = k2 + l2 - 2 * q - 1;
       if (b1 + bb2 <= 2 * M && b1 + bb2 >= 1) u2 = fma(c2[q], A.Psi[bcol(b1, bb2)], u2);
@@ -115,6 +130,7 @@ __global__ void self_pass2_kernel(SelfHighArgs A) {
   const double* u1 = A.U1 + (size_t)k2 * (M + 1) * W + b1;
   const double* u2 = A.U2 + (size_t)k2 * (M + 1) * W + b1;
   double v1 = 0.0, v2 = 0.0;
+#pragma unroll 4
   for (int l2 = 0; l1 + l2 <= M; ++l2) {
     const double a = (l2 & 1) ? -A.at[mcol(l1, l2)] : A.at[mcol(l1, l2)];
     v1 = fma(a, u1[(size_t)l2 * W], v1);
@@ -124,47 +140,56 @@ __global__ void self_pass2_kernel(SelfHighArgs A) {
   A.V2[idx] = v2;
 }
 
-// pass 3 and the finish: one warp per moment row k; lanes split l1, then a
-// warp sum.  R_k, dM_k = c^{|k|/2-1} R_k, the RK4 stage.
-__global__ void self_pass3_kernel(SelfHighArgs A) {
+// pass 3 and the finish: one CTA per moment row k, one thread per (l1, Gamma^I or
+// Gamma^II), then a sum over the CTA in a fixed order.  R_k, dM_k =
+// c^{|k|/2-1} R_k, the RK4 stage.  (A warp per row, the lanes splitting l1, took
+// 39 us at M = 60: its longest lane ran 240 dependent multiply-adds.)
+constexpr int kPass3Threads = 160;  // >= 2 (M + 1) up to order 64, whole warps
+__global__ void __launch_bounds__(kPass3Threads) self_pass3_kernel(SelfHighArgs A) {
   const int M = A.M, W = 2 * M + 1;
-  const int lane = threadIdx.x & 31;
-  const int k = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  if (blockIdx.x == 0 && threadIdx.x < 2) {  // the centre does not move
+  __shared__ double red[kPass3Threads / 32];
+  const int lane = threadIdx.x & 31, k = blockIdx.x;
+  if (k == 0 && threadIdx.x < 2) {  // the centre does not move
     const int c = threadIdx.x;
     if (A.mode == 0) A.out_dx[c] = 0.0;
     if (A.mode == 1) { A.ys_x[c] = A.y_x[c]; A.sum_x[c] = A.y_x[c]; }
     if (A.mode == 2 || A.mode == 3) A.ys_x[c] = A.y_x[c];
     if (A.mode == 4) A.y_x[c] = A.sum_x[c];
   }
-  if (k >= A.K) return;  // whole warps
   const int kn = order_of_col(k);
   const int k2 = k - tri(kn), k1 = kn - k2;
-  const double* v1 = A.V1 + (size_t)k2 * (M + 1) * W;
-  const double* v2 = A.V2 + (size_t)k2 * (M + 1) * W;
   double r = 0.0;
-  for (int l1 = lane; l1 <= M; l1 += 32) {
+  const int half = threadIdx.x > M, l1 = threadIdx.x - (half ? M + 1 : 0);
+  if (l1 <= M) {
     // C(l1, i) g(k1 - i) and C(l1, i) g(k1 - 1 - i), i = 0, 1, ...
     const double* cb = A.cg + ((size_t)l1 * (M + 1) + k1) * (M + 1);
     double s = 0.0;
-    if (k1 >= 1) {
+    if (!half && k1 >= 1) {
+      const double* v1 = A.V1 + ((size_t)k2 * (M + 1) + l1) * W;
       const double* ca = cb - (M + 1);
+#pragma unroll 4
       for (int i = 0; i <= min(l1, k1 - 1); ++i)
-        s = fma(-ca[i], v1[(size_t)l1 * W + k1 + l1 - 2 * i - 1], s);
+        s = fma(-ca[i], v1[k1 + l1 - 2 * i - 1], s);
     }
-    if (k2 >= 1)
+    if (half && k2 >= 1) {
+      const double* v2 = A.V2 + ((size_t)k2 * (M + 1) + l1) * W;
+#pragma unroll 4
       for (int i = 0; i <= min(l1, k1); ++i) {
         const int bb1 = k1 + l1 - 2 * i + 1;
-        if (bb1 < W) s = fma(cb[i], v2[(size_t)l1 * W + bb1], s);
+        if (bb1 < W) s = fma(cb[i], v2[bb1], s);
       }
-    r += (l1 & 1) ? -s : s;
+    }
+    r = (l1 & 1) ? -s : s;
   }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) r += __shfl_xor_sync(0xffffffffu, r, o);
-  if (lane != 0) return;
+  if (lane == 0) red[threadIdx.x >> 5] = r;
+  __syncthreads();
+  if (threadIdx.x != 0) return;
+  r = 0.0;
+  for (int w = 0; w < kPass3Threads / 32; ++w) r += red[w];
   if (kn & 1) r = -r;  // (-1)^{|k|}
-  const double c = stage_c_high(A);
-  const double dm = r * pow(c, 0.5 * kn - 1.0);
+  const double dm = r * half_power(stage_c_high(A), kn - 2);
   if (A.mode == 0) {
     A.out_dM[k] = dm;
     return;
@@ -198,7 +223,7 @@ cudaError_t launch_self_high(SelfHighArgs A, double* scratch, cudaStream_t st) {
   self_psi_kernel<<<(A.NB * 32 + T - 1) / T, T, 0, st>>>(A);
   self_pass1_kernel<<<(int)((P + T - 1) / T), T, 0, st>>>(A);
   self_pass2_kernel<<<(int)((P + T - 1) / T), T, 0, st>>>(A);
-  self_pass3_kernel<<<(A.K * 32 + T - 1) / T, T, 0, st>>>(A);
+  self_pass3_kernel<<<A.K, kPass3Threads, 0, st>>>(A);
   return cudaGetLastError();
 }
 

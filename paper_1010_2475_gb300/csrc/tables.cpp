@@ -37,9 +37,11 @@ long double pow4l(int e) {
 void cut_rows(FinishTables& t, const std::vector<std::vector<FinEntry>>& rows) {
   size_t total = 0;
   for (const auto& r : rows) total += r.size();
-  // ~128 pieces keep the threads of a CTA busy; longer rows of the high
-  // orders get more pieces instead of longer ones
-  const size_t piece = std::min<size_t>(std::max<size_t>(total / 128, 8), 96);
+  // ~128 pieces keep the threads of a CTA busy.  Orders above the pair limit
+  // serve one particle: short pieces, since a thread's dependent multiply-adds
+  // are what such an evaluation waits for (order 10: 96 entries per thread took
+  // 26 us per right-hand side).
+  const size_t piece = t.M > 8 ? 16 : std::min<size_t>(std::max<size_t>(total / 128, 8), 96);
   std::vector<std::vector<FinEntry>> ps;
   t.row_off.assign(1, 0);
   for (const auto& r : rows) {
@@ -62,8 +64,8 @@ void cut_rows(FinishTables& t, const std::vector<std::vector<FinEntry>>& rows) {
     t.piece_len.push_back((int)ps[p].size());
     for (size_t j = 0; j < ps[p].size(); ++j) t.tab[j * ps.size() + p] = ps[p][j];
   }
-  // row blocks of ~1500 entries: a CTA's threads then hold a few entries each
-  const int want = (int)std::min<size_t>(std::max<size_t>(total / 1500, 1), 64);
+  // row blocks of ~256 pieces, one per thread of a CTA
+  const int want = (int)std::min<size_t>(std::max<size_t>(ps.size() / 256, 1), 64);
   t.rb_off.assign(1, 0);
   size_t run = 0;
   for (int k = 0; k < t.K; ++k) {
@@ -73,6 +75,9 @@ void cut_rows(FinishTables& t, const std::vector<std::vector<FinEntry>>& rows) {
   }
   if (t.rb_off.back() != t.K) t.rb_off.push_back(t.K);
   t.nrb = (int)t.rb_off.size() - 1;
+  t.rb_pieces = 0;
+  for (int i = 0; i < t.nrb; ++i)
+    t.rb_pieces = std::max(t.rb_pieces, t.row_off[t.rb_off[i + 1]] - t.row_off[t.rb_off[i]]);
 }
 
 struct BlobOffsets {
@@ -122,6 +127,7 @@ FinishTab finish_tab(const FinishTables& t, const void* base) {
   f.psi0 = reinterpret_cast<const double*>(p + o.psi0);
   f.np = t.np;
   f.nrb = t.nrb;
+  f.rb_pieces = t.rb_pieces;
   return f;
 }
 

@@ -43,6 +43,7 @@ struct FinEntry {
 struct FinishTables {
   int M = 0, K = 0, NB = 0, NJ = 0;
   int np = 0, nrb = 1;
+  int rb_pieces = 0;           // most pieces of a row block
   std::vector<FinEntry> tab;
   std::vector<int> piece_len;  // np
   std::vector<int> row_off;    // K + 1
@@ -58,7 +59,7 @@ struct FinishTab {
   const int* row_off = nullptr;
   const int* rb_off = nullptr;
   const double* psi0 = nullptr;
-  int np = 0, nrb = 1;
+  int np = 0, nrb = 1, rb_pieces = 0;
 };
 FinishTab finish_tab(const FinishTables& t, const void* base);
 
