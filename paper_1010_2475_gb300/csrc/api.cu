@@ -186,13 +186,15 @@ int chunks_for(int64_t n, int tpc, int per_sm, int device, int S) {
 // Shape of the list form for n records: list segments per target group
 // (enough CTAs of the near kernels for ~20 waves) and source ranges of the
 // far kernel (~8 waves of warps, at least 16 source groups per warp).
-void list_shape(const mmvm_ctx* c, const mmvm::ListEntry& e, int64_t n, int* lseg, int* lfar) {
+// seg_hint > 0: that many segments (the tuner's choice).
+void list_shape(const mmvm_ctx* c, const mmvm::ListEntry& e, int64_t n, int seg_hint, int* lseg,
+                int* lfar) {
   int dev_sms = 0;
   cudaDeviceGetAttribute(&dev_sms, cudaDevAttrMultiProcessorCount, c->cfg.device);
   dev_sms = std::max(dev_sms, 1);
   const int64_t G = (n + mmvm::kGroup - 1) / mmvm::kGroup;
   const int occ = std::max(1, mmvm::list_occupancy(e));
-  int64_t seg = (20 * (int64_t)dev_sms * occ + G - 1) / G;
+  int64_t seg = seg_hint > 0 ? seg_hint : (20 * (int64_t)dev_sms * occ + G - 1) / G;
   if (const char* f = std::getenv("MMVM_LIST_SEGMENTS")) seg = std::atoi(f);  // measurement override
   *lseg = (int)std::min<int64_t>(std::max<int64_t>(seg, 1), 16);
   int focc = 0;
@@ -240,6 +242,7 @@ std::mutex g_tune_mu;
 std::map<std::tuple<int, int, int, int, int>, int> g_tuned;
 std::map<std::tuple<int, int, int, int, int>, int> g_tuned_tree;   // list form: tree far field
 std::map<std::tuple<int, int, int, int, int>, int> g_tuned_local;  // list form: local expansions
+std::map<std::tuple<int, int, int, int, int>, int> g_tuned_seg;    // list form: segments (0: rule)
 
 int ilog2(int64_t v) {
   int r = 0;
@@ -486,8 +489,8 @@ static cudaError_t time_pair_variant(mmvm_ctx* c, const mmvm::PairEntry& e, int 
 // Make the list buffers hold list variant e's shape for n records; the
 // shape goes to *lseg / *lfar.
 static int ensure_list_buffers(mmvm_ctx* c, const mmvm::ListEntry& e, int n, bool local,
-                               int* lseg, int* lfar, int* loc_seg) {
-  list_shape(c, e, n, lseg, lfar);
+                               int seg_hint, int* lseg, int* lfar, int* loc_seg) {
+  list_shape(c, e, n, seg_hint, lseg, lfar);
   const int64_t G = (n + mmvm::kGroup - 1) / mmvm::kGroup;
   // ~4 waves of warps (8 per SM) of the local kernel
   *loc_seg = (int)std::min<int64_t>(std::max<int64_t>((32 * (int64_t)c->sms + G - 1) / G, 1), 8);
@@ -522,9 +525,9 @@ static int ensure_list_buffers(mmvm_ctx* c, const mmvm::ListEntry& e, int n, boo
 // Time one launch of list variant e on the context's current records (after
 // one untimed launch); *per_pair = milliseconds per pair.
 static int time_list_variant(mmvm_ctx* c, const mmvm::ListEntry& e, int n, bool tree, bool local,
-                             cudaEvent_t e0, cudaEvent_t e1, double* per_pair) {
+                             int seg_hint, cudaEvent_t e0, cudaEvent_t e1, double* per_pair) {
   int lseg = 1, lfar = 1, loc_seg = 1;
-  int rc = ensure_list_buffers(c, e, n, local, &lseg, &lfar, &loc_seg);
+  int rc = ensure_list_buffers(c, e, n, local, seg_hint, &lseg, &lfar, &loc_seg);
   if (rc) return rc;
   int tfar = 1;
   const int lc = mmvm::tree_chunk_level((n + mmvm::kGroup - 1) / mmvm::kGroup, lfar, &tfar);
@@ -562,7 +565,7 @@ int tune_pair(mmvm_ctx* c) {
   if (n <= 1 || nv + nl <= 1) return MMVM_OK;
   const auto key = std::make_tuple(c->cfg.device, c->M, c->cfg.precision, c->far ? 1 : 0,
                                    ilog2(n));
-  int choice = -1, tree_choice = -1, local_choice = -1;
+  int choice = -1, tree_choice = -1, local_choice = -1, seg_choice = 0;
   if (const char* f = std::getenv("MMVM_PAIR_VARIANT")) choice = std::atoi(f);
   if (choice < 0) {
     if (const char* a = std::getenv("MMVM_AUTOTUNE"))
@@ -643,7 +646,7 @@ int tune_pair(mmvm_ctx* c) {
         continue;
       }
       double per_pair = 0.0;
-      int rc = time_list_variant(c, e, n, false, false, e0, e1, &per_pair);
+      int rc = time_list_variant(c, e, n, false, false, 0, e0, e1, &per_pair);
       if (rc) return rc;
       if (per_pair < best_list) {
         best_list = per_pair;
@@ -657,7 +660,7 @@ int tune_pair(mmvm_ctx* c) {
     if (best_v >= 0) {
       mmvm::ListEntry e = mmvm::list_entry(c->M, best_v);
       double per_pair = 0.0;
-      int rc = time_list_variant(c, e, n, true, false, e0, e1, &per_pair);
+      int rc = time_list_variant(c, e, n, true, false, 0, e0, e1, &per_pair);
       if (rc) return rc;
       if (per_pair < best_list) {
         best_list = per_pair;
@@ -665,7 +668,7 @@ int tune_pair(mmvm_ctx* c) {
       }
       MMVM_CK(e.far.loc_prepare());
       for (int tree = 0; tree < 2; ++tree) {
-        rc = time_list_variant(c, e, n, tree != 0, true, e0, e1, &per_pair);
+        rc = time_list_variant(c, e, n, tree != 0, true, 0, e0, e1, &per_pair);
         if (rc) return rc;
         if (per_pair < best_list) {
           best_list = per_pair;
@@ -681,11 +684,24 @@ int tune_pair(mmvm_ctx* c) {
           cudaGetLastError();
           continue;
         }
-        rc = time_list_variant(c, ev, n, tree_choice != 0, true, e0, e1, &per_pair);
+        rc = time_list_variant(c, ev, n, tree_choice != 0, true, 0, e0, e1, &per_pair);
         if (rc) return rc;
         if (per_pair < best_list) {
           best_list = per_pair;
           best_v = v;
+        }
+      }
+      // list segments: enough CTAs against short lists per CTA (n = 4096, M = 4:
+      // 16 segments left 5 rounds of work between a CTA's set-up and its sums)
+      e = mmvm::list_entry(c->M, best_v);
+      for (int seg : {1, 2, 3, 4, 6, 8, 12, 16}) {
+        if (seg > (n + mmvm::kGroup - 1) / mmvm::kGroup) break;
+        rc = time_list_variant(c, e, n, tree_choice != 0, local_choice != 0, seg, e0, e1,
+                               &per_pair);
+        if (rc) return rc;
+        if (per_pair < best_list) {
+          best_list = per_pair;
+          seg_choice = seg;
         }
       }
       if (best_list < best_full) choice = nv + best_v;
@@ -696,6 +712,7 @@ int tune_pair(mmvm_ctx* c) {
     g_tuned[key] = choice;
     g_tuned_tree[key] = tree_choice;
     g_tuned_local[key] = local_choice;
+    g_tuned_seg[key] = seg_choice;
   }
   if (tree_choice < 0) {
     std::lock_guard<std::mutex> lk(g_tune_mu);
@@ -706,6 +723,8 @@ int tune_pair(mmvm_ctx* c) {
     std::lock_guard<std::mutex> lk(g_tune_mu);
     auto it = g_tuned_local.find(key);
     local_choice = it != g_tuned_local.end() ? it->second : 1;
+    auto is = g_tuned_seg.find(key);
+    seg_choice = is != g_tuned_seg.end() && it != g_tuned_local.end() ? is->second : 0;
   }
   if (const char* f = std::getenv("MMVM_FAR_TREE")) tree_choice = std::atoi(f) != 0;
   if (const char* f = std::getenv("MMVM_LOCAL")) local_choice = std::atoi(f) != 0;
@@ -716,7 +735,7 @@ int tune_pair(mmvm_ctx* c) {
     MMVM_CK(mmvm::list_prepare(e));
     if (local_choice) MMVM_CK(e.far.loc_prepare());
     int lseg = 1, lfar = 1, loc_seg = 1;
-    int rc = ensure_list_buffers(c, e, n, local_choice != 0, &lseg, &lfar, &loc_seg);
+    int rc = ensure_list_buffers(c, e, n, local_choice != 0, seg_choice, &lseg, &lfar, &loc_seg);
     if (rc) return rc;
     int tfar = 1;
     const int lc = mmvm::tree_chunk_level((n + mmvm::kGroup - 1) / mmvm::kGroup, lfar, &tfar);

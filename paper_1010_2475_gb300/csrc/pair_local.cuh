@@ -563,6 +563,19 @@ __global__ void __launch_bounds__(kLocWarps * 32, 2)
 // them with one order of the field per lane.  A target group of radius
 // loc_radius sees everything here from sqrt(x_far) away or more, so the field's
 // Taylor series loses less than FP32 rounding.
+//
+// A node is taken at a radius of up to 0.2 of the distance, twice that of the
+// target-by-target kernels, which hold every order q <= 3M of the jet to 2e-9:
+// here the truncation sum_{k>P} C(q+k-1, k) 0.2^k is 1e-9 or less for the
+// velocities (q = 1) and below FP32 rounding for the orders whose far field
+// counts beside the near field (by q = 6, 5 / r^6 of the near field's size).
+constexpr float kLocTheta2 = 0.04f;
+__device__ __forceinline__ bool loc_takes(const float4 tb, const float4 c) {
+  const float dx = fmaxf(0.f, fmaxf(tb.x - c.x, c.x - tb.y));
+  const float dy = fmaxf(0.f, fmaxf(tb.z - c.y, c.y - tb.w));
+  return c.z * c.z <= kLocTheta2 * (dx * dx + dy * dy);
+}
+
 template <int M>
 struct LocFarSmem {
   using L = Loc<M>;
@@ -691,7 +704,7 @@ __global__ void __launch_bounds__(kLocWarps * 32)
     const float4 box = *reinterpret_cast<const float4*>(nd);
     const float4 cen = *reinterpret_cast<const float4*>(nd + 4);
     const bool far_box = box_dist2(tb, box) >= x_far(M);
-    if (far_box && takes_m2p(tb, cen)) {
+    if (far_box && loc_takes(tb, cen)) {
       if (lane == 0) node_s[nq] = top;
       n_m2p += 1;
       n_m2p_pairs += Lv == 0 ? min(kGroup, n - kGroup * i) : (unsigned)cen.w;

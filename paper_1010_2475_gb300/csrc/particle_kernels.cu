@@ -292,19 +292,32 @@ __device__ __forceinline__ void finish_block(const FinishArgs& A, int j0, int k0
     X[threadIdx.x] = 0.0;
   }
   // 3. add the self pair: Psi_self[beta] = sum_m a_m psi0[m + beta] (psi0
-  //    vanishes at odd indices: only m of the parity of beta contribute)
-  for (int idx = threadIdx.x; idx < TG * NB; idx += NT) {
-    const int tt = idx % TG, b = idx / TG;
-    int bn = 1;
-    while (tri(bn + 1) - 1 <= b) ++bn;
-    const int b2 = b + 1 - tri(bn), b1 = bn - b2;
+  //    vanishes at odd indices: only m of the parity of beta contribute).  One
+  //    row m1 after another; with few targets the rows of a beta are shared by
+  //    SP neighbouring lanes (a lone particle of order 10 waited 6 us for one
+  //    thread's 36 terms).
+  constexpr int SP = TG == 1 ? 4 : 1;
+  for (int i0 = 0; i0 < TG * NB * SP; i0 += NT) {  // whole warps take part in the sums
+    const int idx = i0 + threadIdx.x, part = idx % SP, bt = idx / SP;
+    const int tt = bt % TG, b = bt / TG;
     double acc = 0.0;
-    for (int m1 = b1 & 1; m1 <= M; m1 += 2)
-      for (int m2 = b2 & 1; m1 + m2 <= M; m2 += 2) {
-        const int a2 = m2 + b2;
-        acc = fma(at[mcol(m1, m2) * TG + tt], __ldg(A.tab.psi0 + tri(m1 + b1 + a2) + a2), acc);
+    if (b < NB) {
+      int bn = 1;
+      while (tri(bn + 1) - 1 <= b) ++bn;
+      const int b2 = b + 1 - tri(bn), b1 = bn - b2;
+      for (int m1 = (b1 & 1) + 2 * part; m1 <= M; m1 += 2 * SP) {
+#pragma unroll 4
+        for (int m2 = b2 & 1; m2 <= M - m1; m2 += 2) {
+          const int a2 = m2 + b2;
+          acc = fma(at[mcol(m1, m2) * TG + tt], __ldg(A.tab.psi0 + tri(m1 + b1 + a2) + a2), acc);
+        }
       }
-    psi[b * TG + tt] += acc;
+    }
+    if constexpr (SP > 1) {
+#pragma unroll
+      for (int o = SP >> 1; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+    }
+    if (b < NB && part == 0) psi[b * TG + tt] += acc;
   }
   __syncthreads();
   // 4. the table: sum_l a_l (sum_beta c Psi[beta]) over each piece
@@ -341,6 +354,7 @@ __device__ __forceinline__ void finish_block(const FinishArgs& A, int j0, int k0
     while (tri(kn + 1) <= k) ++kn;
     const int k2 = k - tri(kn), k1c = kn - k2;
     double R = 0.0;
+#pragma unroll 8
     for (int e = A.tab.row_off[k]; e < A.tab.row_off[k + 1]; ++e) R += pres[(e - p0) * TG + tt];
     double ctr = 0.0;
     if (k1c >= 1) ctr += X[2 * tt] * at[mcol(k1c - 1, k2) * TG + tt];

@@ -40,8 +40,8 @@ void cut_rows(FinishTables& t, const std::vector<std::vector<FinEntry>>& rows) {
   // ~128 pieces keep the threads of a CTA busy.  Orders above the pair limit
   // serve one particle: short pieces, since a thread's dependent multiply-adds
   // are what such an evaluation waits for (order 10: 96 entries per thread took
-  // 26 us per right-hand side).
-  const size_t piece = t.M > 8 ? 16 : std::min<size_t>(std::max<size_t>(total / 128, 8), 96);
+  // 26 us per right-hand side, 16 took 20 us).
+  const size_t piece = t.M > 8 ? 8 : std::min<size_t>(std::max<size_t>(total / 128, 8), 96);
   std::vector<std::vector<FinEntry>> ps;
   t.row_off.assign(1, 0);
   for (const auto& r : rows) {
