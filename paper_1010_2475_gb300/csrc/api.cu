@@ -204,9 +204,9 @@ void list_shape(const mmvm_ctx* c, const mmvm::ListEntry& e, int64_t n, int seg_
   }
   const int64_t warp_slots = (int64_t)dev_sms * std::max(focc, 1) * 4;
   int64_t far = (8 * warp_slots + G - 1) / G;
-  // at least 16 source groups per warp, 2 in small problems (a warp's serial
-  // chain over its sources is what they wait for)
-  far = std::min<int64_t>(far, G < 512 ? std::min<int64_t>((G + 1) / 2, 32)
+  // at least 16 source groups per warp, up to 64 ranges in small problems (a
+  // warp's serial chain over its sources is what they wait for)
+  far = std::min<int64_t>(far, G < 512 ? std::min<int64_t>(G, 64)
                                        : std::max<int64_t>(1, G / 16));
   if (const char* f = std::getenv("MMVM_FAR_RANGES")) far = std::atoi(f);  // measurement override
   *lfar = (int)std::min<int64_t>(std::max<int64_t>(far, 1), 64);

@@ -87,6 +87,15 @@ __device__ __forceinline__ float box_dist2(const float4 a, const float4 b) {
   const float dy = fmaxf(0.f, fmaxf(a.z - b.w, b.z - a.w));
   return dx * dx + dy * dy;
 }
+// Is every point of the box sb within x_far(M) of the box tb (point_is_far at
+// none of them)?
+template <int M>
+__device__ __forceinline__ bool box_inside(const float4 tb, const float4 sb) {
+  const float dx = fmaxf(0.f, fmaxf(fmaxf(tb.x - sb.x, sb.x - tb.y), fmaxf(tb.x - sb.y, sb.y - tb.y)));
+  const float dy = fmaxf(0.f, fmaxf(fmaxf(tb.z - sb.z, sb.z - tb.w), fmaxf(tb.z - sb.w, sb.w - tb.w)));
+  // a margin above the rounding differences of the two expressions
+  return dx * dx + dy * dy < x_far(M) * 0.999f;
+}
 // tile_takes_m2p for a target box tb and a source group's (centre, radius) c.
 __device__ __forceinline__ bool takes_m2p(const float4 tb, const float4 c) {
   const float dx = fmaxf(0.f, fmaxf(tb.x - c.x, c.x - tb.y));
@@ -148,21 +157,36 @@ __global__ void near_list_kernel(const float* __restrict__ rec, int n, int G,
         mc += __popc(lb);
         nearg = nearg && !loc;
       }
+      // a group whose box lies wholly within x_far(M) needs no look at its
+      // sources (the distance is largest at a corner, in FP32 too)
+      const bool part = nearg && g < G && !box_inside<M>(tb, *reinterpret_cast<const float4*>(
+                                                                 gdata + (size_t)g * GL));
       unsigned bal = __ballot_sync(0xffffffffu, nearg);
-      while (bal) {
-        const int gg = gb + __ffs(bal) - 1;
-        bal &= bal - 1;
-        const int s = gg * kGroup + lane;
-        bool ns = false;
-        if (s < n) {
-          const float* r = rec + (size_t)s * R;
-          ns = !point_is_far<M>(tb, r[0], r[1]);
+      const unsigned pbal = __ballot_sync(0xffffffffu, part);
+      while (bal) {  // four groups at a time: their loads overlap
+        int gg[4];
+        unsigned m[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          gg[q] = bal ? gb + __ffs(bal) - 1 : -1;
+          m[q] = 0;
+          if (gg[q] < 0) continue;
+          bal &= bal - 1;
+          const int s = gg[q] * kGroup + lane;
+          bool ns = s < n;
+          if ((pbal >> (gg[q] - gb)) & 1u) {
+            const float2 z = s < n ? *reinterpret_cast<const float2*>(rec + (size_t)s * R)
+                                   : make_float2(0.f, 0.f);
+            ns = ns && !point_is_far<M>(tb, z.x, z.y);
+          }
+          m[q] = __ballot_sync(0xffffffffu, ns);
         }
-        const unsigned m = __ballot_sync(0xffffffffu, ns);
-        if (m) {
-          if (lane == 0) ent[(size_t)tg * G + c] = make_int2(gg, (int)m);
-          ++c;
-        }
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+          if (m[q]) {
+            if (lane == 0) ent[(size_t)tg * G + c] = make_int2(gg[q], (int)m[q]);
+            ++c;
+          }
       }
     }
     if (lane == 0) {
@@ -575,36 +599,30 @@ __global__ void __launch_bounds__(kFarWarps * 32)
 // every node; the traversal replaces the per-group expansions of far groups
 // by as few node expansions as the criterion allows.
 
-// Node i of a level from its children in the level below (nchild records;
-// counts of level-0 children: min(kGroup, n - kGroup g)).
+// One warp: node i of a level from its children in the level below (nchild records;
+// counts of level-0 children: min(kGroup, n - kGroup g)), lane j its order j.
 template <int M>
-__global__ void tree_level_kernel(const float* __restrict__ child, int nchild, int child_is_group,
-                                  int n, float* __restrict__ node, int nnode) {
+__device__ __forceinline__ void tree_node(const float* child, int nchild, bool child_is_group,
+                                          int n, float* node, int i) {
   constexpr int GL = gdata_len(M), NA = m2p_terms(M);
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= nnode) return;
+  static_assert(NA <= 32, "one lane per order");
+  const int lane = threadIdx.x & 31;
   const int c0 = 2 * i, c1 = min(2 * i + 1, nchild - 1);
   const float* a = child + (size_t)c0 * GL;
   const float* b = child + (size_t)c1 * GL;
   float4 box = *reinterpret_cast<const float4*>(a);
-  if (c1 != c0) {
-    const float4 bb = *reinterpret_cast<const float4*>(b);
-    box = make_float4(fminf(box.x, bb.x), fmaxf(box.y, bb.y), fminf(box.z, bb.z),
-                      fmaxf(box.w, bb.w));
-  }
+  const float4 bb = *reinterpret_cast<const float4*>(b);  // c1 == c0: the same box
+  box = make_float4(fminf(box.x, bb.x), fmaxf(box.y, bb.y), fminf(box.z, bb.z), fmaxf(box.w, bb.w));
   const float cx = 0.5f * (box.x + box.y), cy = 0.5f * (box.z + box.w);
-  float br[NA], bi[NA];
-#pragma unroll
-  for (int j = 0; j < NA; ++j) {
-    br[j] = 0.f;
-    bi[j] = 0.f;
-  }
-  float rad = 0.f, count = 0.f;
+  float br = 0.f, bi = 0.f, rad = 0.f, count = 0.f;
   for (int c = c0; c <= c1; ++c) {
     const float* r = child + (size_t)c * GL;
-    const float dx = r[4] - cx, dy = r[5] - cy;
-    rad = fmaxf(rad, sqrtf(dx * dx + dy * dy) + r[6]);
-    count += child_is_group ? (float)min(kGroup, n - kGroup * c) : r[7];
+    const float4 h = *reinterpret_cast<const float4*>(r + 4);
+    const float2 v = lane < NA ? *reinterpret_cast<const float2*>(r + 8 + 2 * lane)
+                               : make_float2(0.f, 0.f);
+    const float dx = h.x - cx, dy = h.y - cy;
+    rad = fmaxf(rad, sqrtf(dx * dx + dy * dy) + h.z);
+    count += child_is_group ? (float)min(kGroup, n - kGroup * c) : h.w;
     // B_j += sum_k B^child_{j-k} Delta^k / k!
     float er = 1.f, ei = 0.f;  // Delta^k / k!
 #pragma unroll
@@ -614,21 +632,40 @@ __global__ void tree_level_kernel(const float* __restrict__ child, int nchild, i
         ei = (er * dy + ei * dx) * (1.f / k);
         er = tr;
       }
-#pragma unroll
-      for (int j = k; j < NA; ++j) {
-        const float cr = r[8 + 2 * (j - k)], ci = r[9 + 2 * (j - k)];
-        br[j] = fmaf(cr, er, fmaf(-ci, ei, br[j]));
-        bi[j] = fmaf(cr, ei, fmaf(ci, er, bi[j]));
+      const float cr = __shfl_up_sync(0xffffffffu, v.x, k), ci = __shfl_up_sync(0xffffffffu, v.y, k);
+      if (lane >= k) {
+        br = fmaf(cr, er, fmaf(-ci, ei, br));
+        bi = fmaf(cr, ei, fmaf(ci, er, bi));
       }
     }
   }
   float* o = node + (size_t)i * GL;
-  *reinterpret_cast<float4*>(o) = box;
-  *reinterpret_cast<float4*>(o + 4) = make_float4(cx, cy, rad, count);
-#pragma unroll
-  for (int j = 0; j < NA; ++j) {
-    o[8 + 2 * j] = br[j];
-    o[9 + 2 * j] = bi[j];
+  if (lane == 0) {
+    *reinterpret_cast<float4*>(o) = box;
+    *reinterpret_cast<float4*>(o + 4) = make_float4(cx, cy, rad, count);
+  }
+  if (lane < NA) *reinterpret_cast<float2*>(o + 8 + 2 * lane) = make_float2(br, bi);
+}
+
+// Levels L0 .. L1 of the tree.  A grid of several CTAs takes one level (L0 ==
+// L1); the narrow upper levels, at most kTreeTop nodes each, go to one CTA
+// level after level (a launch each, one thread per node, took 8 us apiece: 72
+// of 1100 us per right-hand side at n = 2011, M = 8).
+constexpr int kTreeTop = 64;  // two nodes per warp of the one CTA
+template <int M>
+__global__ void __launch_bounds__(1024)
+    tree_level_kernel(const float* gdata, int n, int G, int L0, int L1, float* tree) {
+  constexpr int GL = gdata_len(M);
+  const int w0 = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  const int nw = (gridDim.x * blockDim.x) >> 5;
+  for (int L = L0; L <= L1; ++L) {
+    // plain loads: the children may be this CTA's own stores
+    const float* child = L == 1 ? gdata : tree + (size_t)tree_level_offset(G, L - 1) * GL;
+    float* node = tree + (size_t)tree_level_offset(G, L) * GL;
+    const int nnode = tree_level_nodes(G, L);
+    for (int i = w0; i < nnode; i += nw)
+      tree_node<M>(child, tree_level_nodes(G, L - 1), L == 1, n, node, i);
+    if (L < L1) __syncthreads();  // one CTA
   }
 }
 

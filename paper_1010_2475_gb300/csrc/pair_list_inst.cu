@@ -3,6 +3,8 @@
 // -DMMVM_INST_S so the kernels compile in parallel; with -DMMVM_INST_FAR
 // instead of -DMMVM_INST_V / -DMMVM_INST_S, the list build and the far
 // kernel of order MMVM_INST_M.
+#include <algorithm>
+
 #include "pair_local.cuh"
 #include "pair_registry.h"
 
@@ -18,8 +20,9 @@ namespace {
 constexpr int kM = MMVM_INST_M;
 cudaError_t build_fn(const float* rec, int n, int G, const float* gdata, float rmax, int2* ent,
                      int* cnt, int* mcnt, cudaStream_t st) {
-  const int blocks = (G + 7) / 8;  // 8 warps (target groups) per block
-  near_list_kernel<kM><<<blocks, 256, 0, st>>>(rec, n, G, gdata, rmax, ent, cnt, mcnt);
+  // a warp per target group; one warp per CTA while that spreads them over the SMs
+  const int wpc = G <= 1024 ? 1 : 8;
+  near_list_kernel<kM><<<(G + wpc - 1) / wpc, 32 * wpc, 0, st>>>(rec, n, G, gdata, rmax, ent, cnt, mcnt);
   return cudaGetLastError();
 }
 cudaError_t far_fn(const float* rec, int n, int G, const float* gdata, int S, float frad,
@@ -34,16 +37,14 @@ cudaError_t far_occ_fn(int* blocks) {
 }
 cudaError_t tree_build_fn(const float* gdata, int n, int G, float* tree, cudaStream_t st) {
   const int top = tree_levels(G);
-  for (int L = 1; L <= top; ++L) {
-    const float* child = L == 1 ? gdata : tree + (size_t)tree_level_offset(G, L - 1) * gdata_len(kM);
-    const int nchild = tree_level_nodes(G, L - 1), nnode = tree_level_nodes(G, L);
-    tree_level_kernel<kM><<<(nnode + 127) / 128, 128, 0, st>>>(
-        child, nchild, L == 1 ? 1 : 0, n, tree + (size_t)tree_level_offset(G, L) * gdata_len(kM),
-        nnode);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
+  int L = 1;
+  for (; L <= top && tree_level_nodes(G, L) > kTreeTop; ++L)
+    tree_level_kernel<kM><<<(tree_level_nodes(G, L) + 3) / 4, 128, 0, st>>>(gdata, n, G, L, L, tree);
+  if (L <= top) {
+    const int warps = std::min(tree_level_nodes(G, L), 32);
+    tree_level_kernel<kM><<<1, 32 * warps, 0, st>>>(gdata, n, G, L, top, tree);
   }
-  return cudaSuccess;
+  return cudaGetLastError();
 }
 cudaError_t far_tree_fn(const float* rec, int n, int G, const float* gdata, const float* tree,
                         int Lc, float frad, double* fpart, unsigned long long* counts,
@@ -73,10 +74,10 @@ cudaError_t loc_near_fn(const float* rec, int n, int G, const float* gdata, floa
                         const float2* ffld, double* out, unsigned long long* counts, int* err,
                         cudaStream_t st) {
   const int blocks = (G + kLocWarps - 1) / kLocWarps;
-  loc_expand_kernel<kM><<<(G + 3) / 4, 128, 0, st>>>(rec, n, G, gdata, gexp);
+  loc_expand_kernel<kM><<<G, 32, 0, st>>>(rec, n, G, gdata, gexp);
   loc_near_kernel<kM><<<dim3(blocks, C), kLocWarps * 32, LocSmem<kM>::bytes, st>>>(
       n, G, gdata, gexp, ent, mcnt, C, fld, counts, err);
-  loc_eval_kernel<kM><<<(G + 3) / 4, 128, 0, st>>>(rec, n, G, gdata, C, fld, nfar, ffld, out);
+  loc_eval_kernel<kM><<<G, kEvalWarps * 32, 0, st>>>(rec, n, G, gdata, C, fld, nfar, ffld, out);
   return cudaGetLastError();
 }
 }  // namespace

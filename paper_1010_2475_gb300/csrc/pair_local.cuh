@@ -78,22 +78,18 @@ struct Loc {
 // One warp per eligible group: lane k2 sums its column of A over the sources,
 // then the division by D1^2 + D2^2, one lane per order.
 template <int M>
-__global__ void __launch_bounds__(128)
+__global__ void __launch_bounds__(32)
     loc_expand_kernel(const float* __restrict__ rec, int n, int G,
                       const float* __restrict__ gdata, float* __restrict__ gexp) {
   using L = Loc<M>;
   constexpr int R = rec_len<float>(M), K = n_moments(M), GL = gdata_len(M), Q = L::Q;
   constexpr int ST = 33;
-  __shared__ float pw_s[4][2][(Q + 1) * ST];
-  __shared__ float a_s[4][(Q + 1) * (Q + 2)];
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  const int g = blockIdx.x * 4 + w;
-  if (g >= G) return;  // whole warps, no CTA barrier
+  __shared__ float px[(Q + 1) * ST], py[(Q + 1) * ST];
+  __shared__ float as[(Q + 1) * (Q + 2)];
+  const int lane = threadIdx.x, g = blockIdx.x;  // one warp per CTA: groups spread over the SMs
   const float4 cen = *reinterpret_cast<const float4*>(gdata + (size_t)g * GL + 4);
   if (!(cen.z <= loc_radius(M))) return;
   const int cnt = min(kGroup, n - g * kGroup);
-  float* px = pw_s[w][0];
-  float* py = pw_s[w][1];
   {  // lane = source: (-delta / scale)^j / j!
     const float* r = rec + (size_t)(g * kGroup + min(lane, cnt - 1)) * R;
     const float tx = -((r[0] - cen.x) + r[2]) * (1.f / kLocScale);
@@ -154,7 +150,6 @@ __global__ void __launch_bounds__(128)
 #pragma unroll
   for (int k = 0; k < KC; ++k) A[k] += Al[k];
   float* o = gexp + (size_t)g * L::LEN;
-  float* as = a_s[w];
   if (lane <= Q) {
     static_for<0, Q + 1>([&](auto kc) {
       constexpr int k1 = decltype(kc)::value;
@@ -759,12 +754,16 @@ __global__ void __launch_bounds__(kLocWarps * 32)
 }
 
 // ------------------------------------------------------------------ targets
-// One warp per target group: the sum of the C segments' fields, then
-// Psi (edge columns) and R (columns beta1 >= 2) at its 32 targets into partial
-// block `out` ([NB][n] FP64).  The value at the centre is added in FP64, the
-// rest of the Taylor sum in FP32.  Groups without a local field get zeros.
+// One CTA per target group: the sum of the C segments' fields, then Psi (edge
+// columns) and R (columns beta1 >= 2) at its 32 targets into partial block
+// `out` ([NB][n] FP64).  The value at the centre is added in FP64, the rest of
+// the Taylor sum in FP32.  Groups without a local field get zeros.  A warp
+// takes every kEvalWarps-th row of the field and of the results: one warp alone
+// is a chain of ~150 us of dependent shared loads and multiply-adds at M = 8
+// (97 us at n = 24000, M = 6, with 5 warps on an SM).
+constexpr int kEvalWarps = 4;
 template <int M>
-__global__ void __launch_bounds__(128)
+__global__ void __launch_bounds__(kEvalWarps * 32)
     loc_eval_kernel(const float* __restrict__ rec, int n, int G, const float* __restrict__ gdata,
                     int C, const float2* __restrict__ fld, int nfar,
                     const float2* __restrict__ ffld, double* __restrict__ out) {
@@ -773,33 +772,29 @@ __global__ void __launch_bounds__(128)
   constexpr int BM = bmax_of(M), NB = n_beta(M);
   constexpr int GS = (NG + 1 + 3) / 4 * 4;  // row strides, whole float4s
   constexpr int FS = 36;
-  __shared__ __align__(16) float g_s[4][(NG + 1) * GS];
-  __shared__ __align__(16) float f_s[4][(P + 2) * FS];  // F rows n1 = 0 .. P + 1
-  __shared__ double gd_s[4][n_moments(BM >= 2 ? BM - 2 : 0)];
-  __shared__ double fd_s[4][2 * 32];
-  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int tg = blockIdx.x * 4 + w;
-  if (tg >= G) return;  // whole warps
+  __shared__ __align__(16) float gs[(NG + 1) * GS];
+  __shared__ __align__(16) float fs[(P + 2) * FS];  // F rows n1 = 0 .. P + 1
+  __shared__ double gd[n_moments(BM >= 2 ? BM - 2 : 0)];
+  __shared__ double fd[2 * 32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, tg = blockIdx.x;
   const int j = tg * kGroup + lane;
   const float4 cen = *reinterpret_cast<const float4*>(gdata + (size_t)tg * GL + 4);
-  if (!(cen.z <= loc_field_radius(M))) {
+  if (!(cen.z <= loc_field_radius(M))) {  // the whole CTA
     if (j < n)
-      for (int b = 0; b < NB; ++b) out[(size_t)b * n + j] = 0.0;
+      for (int b = warp; b < NB; b += kEvalWarps) out[(size_t)b * n + j] = 0.0;
     return;
   }
-  float* gs = g_s[w];
-  float* fs = f_s[w];
-  double* gd = gd_s[w];
-  double* fd = fd_s[w];
   // sum of the segments; G rows as FP32, the low orders and the edges in FP64
-  for (int r = 0; r < L::FROWS; ++r) {
+  for (int r = L::FROWS - 1 - warp; r >= 0; r -= kEvalWarps) {  // the long edge rows first
     float h = 0.f, l = 0.f;
+#pragma unroll 4
     for (int c = 0; c < C; ++c) {
       const float2 v = fld[(((size_t)c * G + tg) * L::FROWS + r) * 32 + lane];
       two_sum_into(h, l, v.x);
       l += v.y;
     }
     if (r > NG)
+#pragma unroll 8
       for (int c = 0; c < nfar; ++c) {
         const float2 v = ffld[(((size_t)c * G + tg) * 2 + r - NG - 1) * 32 + lane];
         two_sum_into(h, l, v.x);
@@ -814,16 +809,20 @@ __global__ void __launch_bounds__(128)
       fs[(r - NG - 1) * FS + lane] = r - NG - 1 + lane <= NL ? h + l : 0.f;
     }
   }
-  __syncwarp();
-  // F_(n1, n2) = scale^2 G_(n1-2, n2) - F_(n1-2, n2+2), rows n1 >= 2
-  for (int n1 = 2; n1 <= P + 1; ++n1) {
-    float v = 0.f;
-    if (n1 + lane <= NL)
-      v = kLocScale * kLocScale * gs[(n1 - 2) * GS + lane] - fs[(n1 - 2) * FS + lane + 2];
-    fs[n1 * FS + lane] = v;
-    __syncwarp();
+  __syncthreads();
+  // F_(n1, n2) = scale^2 G_(n1-2, n2) - F_(n1-2, n2+2), rows n1 >= 2: the even
+  // rows by warp 0, the odd ones by warp 1 (orders n1 + n2 > NL are zero, so the
+  // top lanes need no neighbour)
+  if (warp < 2) {
+    float v = fs[warp * FS + lane];
+    for (int n1 = 2 + warp; n1 <= P + 1; n1 += 2) {
+      const float up = __shfl_down_sync(0xffffffffu, v, 2);
+      v = n1 + lane <= NL ? kLocScale * kLocScale * gs[(n1 - 2) * GS + lane] - up : 0.f;
+      fs[n1 * FS + lane] = v;
+    }
   }
-  if (j >= n) return;  // no further warp-wide step
+  __syncthreads();
+  if (j >= n) return;  // no further CTA-wide step
   const float* r = rec + (size_t)j * R;
   const float t1 = ((r[0] - cen.x) + r[2]) * (1.f / kLocScale);
   const float t2 = ((r[1] - cen.y) + r[3]) * (1.f / kLocScale);
@@ -874,7 +873,7 @@ __global__ void __launch_bounds__(128)
   static_assert(kLocScale == 0.25f, "inv_scale");
   if constexpr (BM >= 2) {
 #pragma unroll 1
-    for (int q1 = 0; q1 <= BM - 2; ++q1)
+    for (int q1 = warp; q1 <= BM - 2; q1 += kEvalWarps)
       row(q1, std::integral_constant<int, NG + 1>{}, std::integral_constant<int, GS>{}, gs,
           std::integral_constant<int, BM - 2>{}, [&](int q2, float v) {
             if (q1 + q2 <= BM - 2)
@@ -882,8 +881,9 @@ __global__ void __launch_bounds__(128)
                   (gd[tri(q1 + q2) + q2] + (double)v) * inv_scale(q1 + q2);
           });
   }
-#pragma unroll 1
-  for (int q1 = 0; q1 < 2; ++q1)
+  // the edge rows to the warps with the fewest rows so far
+  const int q1 = ((BM >= 2 ? BM - 1 : 0) + kEvalWarps - 1 - warp) % kEvalWarps;
+  if (q1 < 2)
     row(q1, std::integral_constant<int, NL + 1>{}, std::integral_constant<int, FS>{}, fs,
         std::integral_constant<int, BM>{}, [&](int q2, float v) {
           if (q1 + q2 >= 1 && q1 + q2 <= BM)

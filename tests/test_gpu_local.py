@@ -71,6 +71,31 @@ def test_group_expansions(mm, order, n, monkeypatch):
         assert any(not np.array_equal(res[nd, "0"][i], res[nd, "1"][i]) for i in range(2))
 
 
+@pytest.mark.parametrize("groups", [1, 2, 3, 64, 65, 127, 128, 129, 130, 258])
+def test_tree_levels(mm, groups, monkeypatch):
+    """The levels built by one CTA (at most 64 nodes) and those below it, full
+    and ragged; every group range against the same groups without a tree."""
+    n, order = 32 * groups - 5, 3
+    wl = mmvm_inputs.two_patches(n=n, order=order, sigma=0.1, seed=groups)
+    wl.moments[:, 3:] = np.random.default_rng(groups).normal(size=wl.moments[:, 3:].shape) \
+        * 1e-2 * wl.moments[:, :1] * wl.lam0 ** 2
+    nd, nl = mm.pair_variant_counts(order)
+    monkeypatch.setenv("MMVM_PAIR_VARIANT", str(nd + nl - 1))
+    rows = np.array(sorted({0, n // 2, n - 1, *range(max(0, n - 40), n, 8)}))
+    ox, oM = rhs_regrouped(wl.x, wl.moments, 0.0, order, wl.lam0, wl.nu, rows=rows)
+    sx, sM = abs_scale_rows(wl.x, wl.moments, 0.0, order, wl.lam0, wl.nu, rows)
+    for tree, local in (("1", "1"), ("1", "0"), ("0", "1")):
+        monkeypatch.setenv("MMVM_FAR_TREE", tree)
+        monkeypatch.setenv("MMVM_LOCAL", local)
+        with mm.Context(order, wl.lam0, wl.nu, mm.MMVM_MIXED_FP32) as ctx:
+            ctx.set_state(wl.x, wl.moments, 0.0)
+            gx, gM = ctx.rhs()
+            near, far_pp, n_m2p, m2p_pairs = mm.mmvm_pair_work(ctx.handle)
+        assert near + far_pp + m2p_pairs == n * n
+        assert vel_error_cond(gx[rows], ox, sx) <= 5e-6
+        assert rhs_error_cond(gM[rows], oM, sM, order, wl.lam0) <= 5e-6
+
+
 @pytest.mark.parametrize("n", [1, 2, 2431, 2433, 4865, 9729, 19457])
 def test_finish_shapes(mm, n):
     """Targets per finish CTA (1, 4, 8, 16, 32) on both sides of each switch."""
