@@ -106,6 +106,7 @@ struct mmvm_ctx {
   int order_launches = 0;  // kernels launched by one spatial ordering
   DevBuf<unsigned char> ftab;  // finish tables (blob of tables.h)
   mmvm::FinishTab ft;
+  DevBuf<double> fscal;        // powers of c and weights of the stage
   int sms = 1;                 // multiprocessors of the device
   mmvm::PairEntry pe;
   // interaction-list form of the all-pairs kernels (FP32 with the far field):
@@ -360,7 +361,7 @@ int enqueue_rhs(mmvm_ctx* c, int mode, const double* xin, const double* min_, do
     }
     MMVM_CK(mmvm::launch_prep(c->cfg.precision, n, c->M, perm, xin, min_, c->t_dev(), dt_dev,
                               cs, lam0sq, four_nu, c->rec.p, c->far ? c->gbox.p : nullptr,
-                              c->st));
+                              c->fscal.p, c->st));
     const int slot = mode == 0 ? 4 : mode - 1;
     if (c->timing) MMVM_CK(cudaEventRecord(c->ev[slot][0], c->st));
     if (c->list) {
@@ -427,6 +428,7 @@ int enqueue_rhs(mmvm_ctx* c, int mode, const double* xin, const double* min_, do
   A.perm = perm;
   A.Min = min_;
   A.tab = c->ft;
+  A.scal = n > 1 ? c->fscal.p : nullptr;  // written by launch_prep
   A.lam0sq = lam0sq;
   A.four_nu = four_nu;
   A.t_dev = c->t_dev();
@@ -585,7 +587,7 @@ int tune_pair(mmvm_ctx* c) {
                                          c->st));
     MMVM_CK(mmvm::launch_prep(c->cfg.precision, n, c->M, perm, c->x.p, c->m.p, c->t_dev(),
                               nullptr, 0.0, lam0sq, four_nu, c->rec.p,
-                              c->far ? c->gbox.p : nullptr, c->st));
+                              c->far ? c->gbox.p : nullptr, c->fscal.p, c->st));
     cudaEvent_t e0, e1;
     MMVM_CK(cudaEventCreate(&e0));
     MMVM_CK(cudaEventCreate(&e1));
@@ -882,7 +884,9 @@ int mmvm_create(const mmvm_config* cfg, mmvm_ctx** out) {
   }
   const std::vector<unsigned char> tb = T.blob();
   if ((e = c->ftab.ensure(tb.size())) != cudaSuccess || (e = c->scal.ensure(2)) != cudaSuccess ||
-      (e = c->flags.ensure(2)) != cudaSuccess || (e = c->counts.ensure(4)) != cudaSuccess)
+      (e = c->flags.ensure(2)) != cudaSuccess ||
+      (e = c->fscal.ensure(mmvm::finish_scalars(c->M))) != cudaSuccess ||
+      (e = c->counts.ensure(4)) != cudaSuccess)
     return bail(cuda_fail(e, "cudaMalloc(tables)"));
   if ((e = cudaMemcpy(c->ftab.p, tb.data(), tb.size(), cudaMemcpyHostToDevice)) != cudaSuccess ||
       (e = cudaMemset(c->scal.p, 0, 2 * sizeof(double))) != cudaSuccess ||
@@ -907,7 +911,8 @@ void mmvm_destroy(mmvm_ctx* c) {
     for (auto& e : pr)
       if (e) cudaEventDestroy(e);
   for (auto* b : {&c->x, &c->m, &c->xs, &c->ms, &c->xsum, &c->msum, &c->rdx, &c->rdm, &c->scal,
-                  &c->partial, &c->sbinom, &c->sg, &c->scg, &c->sscr, &c->dpts, &c->dval, &c->dring, &c->dk,
+                  &c->partial, &c->fscal, &c->sbinom, &c->sg, &c->scg, &c->sscr, &c->dpts, &c->dval, &c->dring,
+                  &c->dk,
                   &c->fpart})
     b->release();
   c->tnodes.release();

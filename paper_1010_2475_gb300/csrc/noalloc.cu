@@ -141,7 +141,7 @@ extern "C" int mmvm_rhs_noalloc(const mmvm_config* cfg, int64_t n, double t, con
       return set_err(MMVM_E_UNSUPPORTED, "records exceed the fixed scratch");
     if ((e = pair_prepare(pe, kGroup)) != cudaSuccess ||
         (e = launch_prep(prec, (int)n, M, nullptr, d_x, d_moments, t_dev, nullptr, 0.0, lam0sq,
-                         four_nu, rec, nullptr, st)) != cudaSuccess ||
+                         four_nu, rec, nullptr, nullptr, st)) != cudaSuccess ||
         (e = pair_launch(pe, rec, (int)n, chunks, kGroup, nullptr, partial, 0, st)) != cudaSuccess)
       return set_err(MMVM_E_DEVICE, std::string("launch: ") + cudaGetErrorString(e));
   }

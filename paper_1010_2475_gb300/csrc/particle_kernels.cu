@@ -24,6 +24,34 @@ __device__ __forceinline__ double stage_c(const double* t_dev, const double* dt_
   return 2.0 * (lam0sq + four_nu * t);
 }
 
+// c^{e/2} by repeated squaring (e may be negative): a few roundings, and a
+// fraction of the FP64 operations of pow().
+__device__ __forceinline__ double half_power(double c, int e) {
+  const double b = e < 0 ? 1.0 / c : c;
+  const int h = e < 0 ? -e : e;
+  double v = (h & 1) ? sqrt(b) : 1.0, q = b;
+  for (int i = h >> 1; i; i >>= 1) {
+    if (i & 1) v *= q;
+    q *= q;
+  }
+  return v;
+}
+
+// Powers of the core scale and the step's weights (FinishArgs::scal): c^{-s/2},
+// s = 0..M, then c^{s/2-1}, s = 0..M, then h, h/2, h/3, h/6.  One thread per
+// value (thread i of at least 2 (M + 1) + 4).
+__host__ __device__ constexpr int scal_len(int M) { return 2 * (M + 1) + 4; }
+__device__ __forceinline__ void write_scalars(double* o, int i, int M, double c, double h) {
+  if (i <= M)
+    o[i] = half_power(c, -i);
+  else if (i < 2 * (M + 1))
+    o[i] = half_power(c, i - (M + 1) - 2);
+  else if (i < scal_len(M)) {
+    const int w = i - 2 * (M + 1);
+    o[i] = w == 0 ? h : w == 1 ? 0.5 * h : w == 2 ? h / 3.0 : h / 6.0;
+  }
+}
+
 // The source record of one particle (centre xj, moments mj): zeta = x / sqrt(c)
 // (FP32: exact (hi, lo) pair), a_m = M_m c^{-|m|/2} and, for FP32 records,
 // the far-field multipoles A'_n = sum_{|m|=n} a_m (-i)^{m1+n}.
@@ -69,40 +97,106 @@ __device__ __forceinline__ void make_record(T* __restrict__ r, const double* __r
   for (int q = h + K + rec_far<T>(M); q < R; ++q) r[q] = T(0);
 }
 
-// Sorted position p holds particle perm[p] (perm == null: identity).  Every
-// warp (kGroup consecutive positions) writes the bounding box of its hi-part
-// centres at the head of its group record in gdata (if given; records of GL
-// floats, see gdata_len).
+// The records of kGroup consecutive sorted positions by one CTA (position p
+// holds particle perm[p]; perm == null: identity), values as in make_record.
+// With gdata, the bounding box of the group's hi-part centres goes to the head
+// of its group record (records of GL floats, see gdata_len).  Bound: latency;
+// moments and records move as coalesced rows through shared memory (a thread
+// per particle waited for K strided loads in turn: 31 us at n = 2011, M = 8).
+constexpr int kPrepThreads = 128;
+constexpr int kMaxPairM = 8;  // highest order with pair kernels
 template <typename T>
-__global__ void prep_kernel(int n, int M, int K, int R, const int* __restrict__ perm,
-                            const double* __restrict__ x, const double* __restrict__ mom,
-                            const double* t_dev, const double* dt_dev, double cs, double lam0sq,
-                            double four_nu, T* __restrict__ rec, float* __restrict__ gdata,
-                            int GL) {
-  const int p = blockIdx.x * blockDim.x + threadIdx.x;
-  const bool valid = p < n;
-  float lo1 = 3.4e38f, hi1 = -3.4e38f, lo2 = 3.4e38f, hi2 = -3.4e38f;
-  if (valid) {
-    const int j = perm ? perm[p] : p;
-    const double c = stage_c(t_dev, dt_dev, cs, lam0sq, four_nu);
-    T* r = rec + (size_t)p * R;
-    make_record<T>(r, x + 2 * j, mom + (size_t)j * K, M, K, R, 1.0 / sqrt(c));
-    if constexpr (sizeof(T) == 4) {
-      lo1 = hi1 = r[0];
-      lo2 = hi2 = r[1];
+__global__ void __launch_bounds__(kPrepThreads)
+    prep_kernel(int n, int M, int K, int R, const int* __restrict__ perm,
+                const double* __restrict__ x, const double* __restrict__ mom,
+                const double* t_dev, const double* dt_dev, double cs, double lam0sq,
+                double four_nu, T* __restrict__ rec, float* __restrict__ gdata, int GL,
+                double* __restrict__ scal) {
+  if (scal != nullptr && blockIdx.x == gridDim.x - 1) {  // the extra CTA: scalars of the finish
+    for (int i = threadIdx.x; i < scal_len(M); i += blockDim.x)
+      write_scalars(scal, i, M, stage_c(t_dev, dt_dev, cs, lam0sq, four_nu),
+                    dt_dev ? *dt_dev : 0.0);
+    return;
+  }
+  constexpr int H = Rec<T>::HDR;
+  __shared__ double a_s[kGroup * (n_moments(kMaxPairM) | 1)];  // odd stride
+  __shared__ double pw[kMaxPairM + 1];                         // c^{-s/2}
+  __shared__ int j_s[kGroup];
+  const int p0 = blockIdx.x * kGroup, np = min(kGroup, n - p0), KS = K | 1;
+  if (threadIdx.x < kGroup) {
+    const int p = p0 + threadIdx.x;
+    const bool valid = p < n;
+    const int j = valid ? (perm ? perm[p] : p) : 0;
+    j_s[threadIdx.x] = j;
+    const double irc = 1.0 / sqrt(stage_c(t_dev, dt_dev, cs, lam0sq, four_nu));
+    double sc = 1.0;
+    for (int s = 0; s <= M; ++s) {
+      if (threadIdx.x == 0) pw[s] = sc;
+      sc *= irc;
+    }
+    float lo1 = 3.4e38f, hi1 = -3.4e38f, lo2 = 3.4e38f, hi2 = -3.4e38f;
+    if (valid) {
+      const double z1 = x[2 * j] * irc, z2 = x[2 * j + 1] * irc;
+      T* r = rec + (size_t)p * R;
+      r[0] = (T)z1;
+      r[1] = (T)z2;
+      if constexpr (sizeof(T) == 4) {
+        lo1 = hi1 = (float)z1;
+        lo2 = hi2 = (float)z2;
+        r[2] = (float)(z1 - (double)lo1);
+        r[3] = (float)(z2 - (double)lo2);
+      }
+    }
+    if (gdata) {
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) {
+        lo1 = fminf(lo1, __shfl_xor_sync(0xffffffffu, lo1, o));
+        hi1 = fmaxf(hi1, __shfl_xor_sync(0xffffffffu, hi1, o));
+        lo2 = fminf(lo2, __shfl_xor_sync(0xffffffffu, lo2, o));
+        hi2 = fmaxf(hi2, __shfl_xor_sync(0xffffffffu, hi2, o));
+      }
+      if (threadIdx.x == 0)
+        *reinterpret_cast<float4*>(gdata + (size_t)blockIdx.x * GL) =
+            make_float4(lo1, hi1, lo2, hi2);
     }
   }
-  if (gdata) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      lo1 = fminf(lo1, __shfl_xor_sync(0xffffffffu, lo1, o));
-      hi1 = fmaxf(hi1, __shfl_xor_sync(0xffffffffu, hi1, o));
-      lo2 = fminf(lo2, __shfl_xor_sync(0xffffffffu, lo2, o));
-      hi2 = fmaxf(hi2, __shfl_xor_sync(0xffffffffu, hi2, o));
+  __syncthreads();
+  for (int i = threadIdx.x; i < np * K; i += kPrepThreads) {
+    const int q = i / K, col = i - q * K;
+    int s = 0;
+    while (tri(s + 1) <= col) ++s;
+    const double a = mom[(size_t)j_s[q] * K + col] * pw[s];
+    if constexpr (sizeof(T) == 4) a_s[q * KS + col] = a;
+    rec[(size_t)(p0 + q) * R + H + col] = (T)a;
+  }
+  // A'_s = sum_k2 (-i)^{m1 + s} a, m1 = s - k2
+  if constexpr (sizeof(T) == 4) {
+    __syncthreads();
+    const int tail = R - H - K;  // far multipoles and the padding
+    for (int i = threadIdx.x; i < np * (M + 1); i += kPrepThreads) {
+      const int q = i / (M + 1), s = i - q * (M + 1);
+      const double* a = a_s + q * KS + tri(s);
+      double fr = 0.0, fi = 0.0;
+      for (int k2 = 0; k2 <= s; ++k2) switch ((s - k2 + s) & 3) {
+          case 0: fr += a[k2]; break;
+          case 1: fi -= a[k2]; break;
+          case 2: fr -= a[k2]; break;
+          default: fi += a[k2]; break;
+        }
+      float* r = rec + (size_t)(p0 + q) * R + H + K + 2 * s;
+      r[0] = (float)fr;
+      r[1] = (float)fi;
     }
-    if ((threadIdx.x & 31) == 0 && valid)
-      *reinterpret_cast<float4*>(gdata + (size_t)(p / kGroup) * GL) =
-          make_float4(lo1, hi1, lo2, hi2);
+    for (int i = threadIdx.x; i < np * (tail - rec_far<T>(M)); i += kPrepThreads) {
+      const int w = tail - rec_far<T>(M), q = i / w;
+      rec[(size_t)(p0 + q) * R + H + K + rec_far<T>(M) + i - q * w] = T(0);
+    }
+  } else {
+    const int w = R - H - K;
+    for (int i = threadIdx.x; i < np * w; i += kPrepThreads) {
+      const int q = i / w;
+      rec[(size_t)(p0 + q) * R + H + K + i - q * w] = T(0);
+    }
   }
 }
 
@@ -189,74 +283,93 @@ __global__ void group_multipole_kernel(int n, const float* __restrict__ rec,
   }
 }
 
+// v[0] + v[stride] + ... (n values) as four interleaved sums: fixed order, a
+// quarter of the dependent additions, several loads in flight.
+__device__ __forceinline__ double block_sum(const double* __restrict__ v, int n, size_t stride) {
+  double s[4] = {0.0, 0.0, 0.0, 0.0};
+  int i = 0;
+#pragma unroll 2
+  for (; i + 4 <= n; i += 4) {
+#pragma unroll
+    for (int q = 0; q < 4; ++q) s[q] += v[(size_t)(i + q) * stride];
+  }
+#pragma unroll
+  for (int q = 0; q < 3; ++q)
+    if (i + q < n) s[q] += v[(size_t)(i + q) * stride];
+  return (s[0] + s[1]) + (s[2] + s[3]);
+}
+
 // The finish of TG targets (sorted positions j0 .. j0 + TG - 1, those below
-// A.n) by one CTA, moment rows [k0, k1) with the table pieces [p0, p1).
+// A.n) by one CTA, row blocks [rb0, rb1) of the table.
 //
-// Bound: FP64 arithmetic (2 FMA per cycle and SM here, 1/64 of FP32).  Per
-// target: the sums over the partial blocks, NB K / 4 multiply-adds of the
-// self pair and one multiply-add per table entry and (k, l) group (4214 at
-// M = 6; the form c a_l Psi took 6916).  A thread takes whole pieces of the
-// table for one target, so that rows of very different length (0 to 260
-// entries at M = 6) do not leave lanes idle, and the entries are read by
-// neighbouring threads side by side.  TG = 32 makes the entry stream of a warp
-// uniform; small n takes smaller TG so that every SM has work
-// (finish_targets).  Shared memory holds [column][target] arrays: Psi (NB), a
-// (K), X (2), M_00, the powers c^{-s/2} and the pieces' sums.  Every global
-// read of the stage input precedes the first write behind a barrier.  All
-// threads of the CTA call this; a caller that loops must add a barrier.
+// Bound: FP64 arithmetic.  An FP64 instruction keeps this SM's pipe busy for 16
+// cycles however few of its lanes are active, so what counts is lanes in use:
+//  * per target NB K / 4 multiply-adds of the self pair, one addition per
+//    partial block and column, one multiply-add per table entry and one per
+//    (k, l) group (4214 at M = 6);
+//  * a thread takes whole groups for one target; groups are sorted by length,
+//    so a warp's lanes run loops of (nearly) one length.  (A thread per row, 0
+//    to 260 entries, kept 2/3 of the lanes idle; closing groups of mixed
+//    lengths inside one loop executed a second multiply-add per entry.)
+//  * scalars (powers of c, weights of the step) come from the record kernel;
+//    without one (a single particle, batches) two warps form them.
+// Shared memory holds [column][target] arrays: Psi (NB), a (K), X (2), 1 / M_00,
+// the scalars and the groups' sums.  Every global read of the stage input
+// precedes the first write behind a barrier.  All threads of the CTA call this;
+// a caller that loops must add a barrier.
 template <int TG>
-__device__ __forceinline__ void finish_block(const FinishArgs& A, int j0, int k0, int k1,
+__device__ __forceinline__ void finish_block(const FinishArgs& A, int j0, int rb0, int rb1,
                                              double* sm) {
   const int NB = A.NB, K = A.K, M = A.M, NT = blockDim.x;
-  const int p0 = A.tab.row_off[k0], p1 = A.tab.row_off[k1];
   double* psi = sm;                 // NB * TG
   double* at = psi + NB * TG;       // K * TG
   double* X = at + K * TG;          // 2 * TG
-  double* m00s = X + 2 * TG;        // TG
-  double* cpow = m00s + TG;         // c^{-s/2}, s = 0..M
-  double* pres = cpow + M + 1;      // (p1 - p0) * TG
-  const double c = stage_c(A.t_dev, A.dt_dev, A.cs, A.lam0sq, A.four_nu);
-  if (threadIdx.x <= M) {  // c^{-s/2} by repeated squaring of 1/c: a few roundings
-    double base = 1.0 / c, v = (threadIdx.x & 1) ? 1.0 / sqrt(c) : 1.0;
-    for (int e = threadIdx.x >> 1; e; e >>= 1) {
-      if (e & 1) v *= base;
-      base *= base;
-    }
-    cpow[threadIdx.x] = v;
+  double* m00s = X + 2 * TG;        // TG: 1 / M_00
+  double* cpow = m00s + TG;         // the scalars
+  double* cinv = cpow + M + 1;
+  double* hs = cinv + M + 1;
+  double* gsum = hs + 4;            // max_groups * TG
+  // 1. the scalars, the stage moments, Psi_excl = sum over the partial blocks
+  //    (fixed order)
+  if (A.scal) {
+    for (int i = threadIdx.x; i < scal_len(M); i += NT) cpow[i] = A.scal[i];
+  } else if (threadIdx.x >= NT - 64) {
+    write_scalars(cpow, threadIdx.x - (NT - 64), M,
+                  stage_c(A.t_dev, A.dt_dev, A.cs, A.lam0sq, A.four_nu),
+                  A.dt_dev ? *A.dt_dev : 0.0);
   }
-  __syncthreads();
-  // 1. Psi_excl = sum over the partial blocks (fixed order), scaled moments
+  for (int idx = threadIdx.x; idx < TG * K; idx += NT) {
+    const int tt = idx / K, m = idx % K, p = j0 + tt;
+    const int j = p < A.n ? (A.perm ? A.perm[p] : p) : 0;
+    const double mv = (p < A.n) ? A.Min[(size_t)j * K + m] : 0.0;
+    at[m * TG + tt] = p < A.n || m ? mv : 1.0;
+  }
   for (int idx = threadIdx.x; idx < TG * NB; idx += NT) {
     const int tt = idx % TG, b = idx / TG, j = j0 + tt;
     double v = 0.0;
     if (j < A.n && A.partial) {
-#pragma unroll 8
-      for (int ch = 0; ch < A.nchunks; ++ch) v += A.partial[((size_t)ch * NB + b) * A.n + j];
+      v = block_sum(A.partial + (size_t)b * A.n + j, A.nchunks, (size_t)NB * A.n);
       // far field of the list form: edge columns only
       if (A.fpart &&
           !(A.rmax > 0.f && A.gdata[(size_t)(j / kGroup) * A.gdata_len + 6] <= A.rmax)) {
         int bn = 1;
         while (tri(bn + 1) - 1 <= b) ++bn;
         const int b1 = bn - (b + 1 - tri(bn));
-        if (b1 <= 1) {
-          const int e = 2 * (bn - 1) + b1;
-#pragma unroll 8
-          for (int ch = 0; ch < A.nfar; ++ch) v += A.fpart[((size_t)ch * A.n_edge + e) * A.n + j];
-        }
+        if (b1 <= 1)
+          v += block_sum(A.fpart + (size_t)(2 * (bn - 1) + b1) * A.n + j, A.nfar,
+                         (size_t)A.n_edge * A.n);
       }
     }
     psi[b * TG + tt] = v;
   }
-  for (int idx = threadIdx.x; idx < TG * K; idx += NT) {
-    const int tt = idx / K, m = idx % K, p = j0 + tt;
-    int s = 0;
-    while (tri(s + 1) <= m) ++s;  // total order of column m
-    const int j = p < A.n ? (A.perm ? A.perm[p] : p) : 0;
-    const double mv = (p < A.n) ? A.Min[(size_t)j * K + m] : 0.0;
-    at[m * TG + tt] = mv * cpow[s];
-    if (m == 0) m00s[tt] = (p < A.n) ? mv : 1.0;
-  }
   __syncthreads();
+  if (threadIdx.x < TG) m00s[threadIdx.x] = 1.0 / at[threadIdx.x];
+  for (int idx = TG + threadIdx.x; idx < TG * K; idx += NT) {
+    int s = 0;
+    while (tri(s + 1) <= idx / TG) ++s;  // total order of the column
+    at[idx] *= cpow[s];
+  }
+  if (!A.partial) __syncthreads();
   if (A.partial) {
     // 1b. the pair kernels leave Psi itself only in the edge columns beta1 <= 1;
     //     a column beta1 >= 2 holds R[beta] = sum_m a_m D^{m + beta - 2 e1} Lap psi.
@@ -269,7 +382,7 @@ __device__ __forceinline__ void finish_block(const FinishArgs& A, int j0, int k0
       for (int b1 = 2; b1 <= k; ++b1)
         ps[bcol(b1, k - b1) * TG] -= ps[bcol(b1 - 2, k - b1 + 2) * TG];
     }
-    __syncthreads();
+    __syncthreads();  // Psi and the scaled moments
     // 2. centroid sums X_c = sum_m (-1)^{|m|} a_m What_c[m], What_1[m] = -Psi[m+e2],
     //    What_2[m] = Psi[m+e1]  (eq:xjdot_Final in c = 1 units, self pair excluded);
     //    the columns m of one (target, component) are split over q lanes
@@ -320,75 +433,95 @@ __device__ __forceinline__ void finish_block(const FinishArgs& A, int j0, int k0
     if (b < NB && part == 0) psi[b * TG + tt] += acc;
   }
   __syncthreads();
-  // 4. the table: sum_l a_l (sum_beta c Psi[beta]) over each piece
+  for (int rb = rb0; rb < rb1; ++rb) {
+  const RowBlock B = A.tab.blocks[rb];
+  // 4. the groups of the table: g = sum_beta c Psi[beta]; with one target the
+  //    entries of a group are shared by GL neighbouring lanes (a lone particle
+  //    of order 10 otherwise waits for up to 110 dependent loads and additions)
   {
-    const int tt = threadIdx.x % TG, np = A.tab.np;
+    constexpr int GL = TG == 1 ? 4 : 1;
+    const int tt = threadIdx.x % TG, part = threadIdx.x % GL;
     const double* ps = psi + tt;
-    const double* a = at + tt;
-    for (int p = p0 + threadIdx.x / TG; p < p1; p += NT / TG) {
-      const int len = __ldg(A.tab.piece_len + p);
-      const double2* e = reinterpret_cast<const double2*>(A.tab.tab) + p;
-      double R = 0.0, g = 0.0;
+    const int* off = A.tab.offs + B.off_at;
+    for (int q0 = 0; q0 < B.groups; q0 += NT / (TG * GL)) {  // whole warps stay together
+      const int q = q0 + threadIdx.x / (TG * GL);
+      const int len = q < B.groups ? __ldg(A.tab.glen + B.len_at + q) : 0;
+      const double2* e = reinterpret_cast<const double2*>(A.tab.tab) + q;
+      double g = 0.0;
 #pragma unroll 4
-      for (int j = 0; j < len; ++j) {
-        const double2 v = __ldg(e + (size_t)j * np);  // (c, packed b and l)
-        const long long bl = __double_as_longlong(v.y);
-        const int b = (int)(bl & 0xffffffffll), l = (int)(bl >> 32);
-        g = fma(v.x, ps[b * TG], g);
-        if (l >= 0) {
-          R = fma(a[l * TG], g, R);
-          g = 0.0;
-        }
+      for (int j = part; j < len; j += GL) {
+        const double2 v = __ldg(e + __ldg(off + j));  // (c, packed b)
+        g = fma(v.x, ps[(int)(__double_as_longlong(v.y) & 0xffffffffll) * TG], g);
       }
-      pres[(p - p0) * TG + tt] = R;
+      if constexpr (GL > 1) {
+#pragma unroll
+        for (int o = GL >> 1; o > 0; o >>= 1) g += __shfl_xor_sync(0xffffffffu, g, o);
+      }
+      if (q < B.groups && part == 0) gsum[q * TG + tt] = g;
     }
   }
   __syncthreads();
-  // 5. moment equation and stage update per (target, k)
-  const int nk = k1 - k0;
-  for (int idx = threadIdx.x; idx < TG * nk; idx += NT) {
-    const int tt = idx / nk, k = k0 + idx % nk, p = j0 + tt;
-    if (p >= A.n) continue;
+  // 5. moment equation and stage update per (target, k): R_k = sum_l a_l g_kl,
+  //    the l shared by RL neighbouring lanes
+  const int k0 = B.k0, nk = B.k1 - B.k0;
+  constexpr int RL = TG == 1 ? 16 : 1;
+  for (int i0 = 0; i0 < TG * nk * RL; i0 += NT) {  // whole warps take part in the sums
+    const int it = i0 + threadIdx.x, part = it % RL, idx = it / RL;
+    const bool on = idx < TG * nk;
+    const int tt = on ? idx % TG : 0, k = on ? k0 + idx / TG : k0, p = j0 + tt;
+    double R = 0.0;
+    if (on) {
+      const int e1 = A.tab.rows_off[k + 1];
+#pragma unroll 4
+      for (int e = A.tab.rows_off[k] + part; e < e1; e += RL) {
+        const int2 w = __ldg(reinterpret_cast<const int2*>(A.tab.rows) + e);  // (q, l)
+        R = fma(at[w.y * TG + tt], gsum[w.x * TG + tt], R);
+      }
+    }
+    if constexpr (RL > 1) {
+#pragma unroll
+      for (int o = RL >> 1; o > 0; o >>= 1) R += __shfl_xor_sync(0xffffffffu, R, o);
+    }
+    if (!on || part != 0 || p >= A.n) continue;
     const int j = A.perm ? A.perm[p] : p;
     int kn = 0;
     while (tri(kn + 1) <= k) ++kn;
     const int k2 = k - tri(kn), k1c = kn - k2;
-    double R = 0.0;
-#pragma unroll 8
-    for (int e = A.tab.row_off[k]; e < A.tab.row_off[k + 1]; ++e) R += pres[(e - p0) * TG + tt];
     double ctr = 0.0;
     if (k1c >= 1) ctr += X[2 * tt] * at[mcol(k1c - 1, k2) * TG + tt];
     if (k2 >= 1) ctr += X[2 * tt + 1] * at[mcol(k1c, k2 - 1) * TG + tt];
-    const double dm = (R + ctr / m00s[tt]) / (cpow[kn] * c);  // c^{|k|/2 - 1}
+    const double dm = fma(ctr, m00s[tt], R) * cinv[kn];  // c^{|k|/2 - 1}
     const size_t o = (size_t)j * K + k;
     if (A.mode == 0) {
       A.out_dM[o] = dm;
     } else {
-      const double h = *A.dt_dev;
       const double base = A.y_M[o];
-      if (A.mode == 1) { A.ys_M[o] = base + 0.5 * h * dm; A.sum_M[o] = base + h / 6.0 * dm; }
-      if (A.mode == 2) { A.ys_M[o] = base + 0.5 * h * dm; A.sum_M[o] += h / 3.0 * dm; }
-      if (A.mode == 3) { A.ys_M[o] = base + h * dm;       A.sum_M[o] += h / 3.0 * dm; }
-      if (A.mode == 4) { A.y_M[o] = A.sum_M[o] + h / 6.0 * dm; }
+      if (A.mode == 1) { A.ys_M[o] = base + hs[1] * dm; A.sum_M[o] = base + hs[3] * dm; }
+      if (A.mode == 2) { A.ys_M[o] = base + hs[1] * dm; A.sum_M[o] += hs[2] * dm; }
+      if (A.mode == 3) { A.ys_M[o] = base + hs[0] * dm; A.sum_M[o] += hs[2] * dm; }
+      if (A.mode == 4) { A.y_M[o] = A.sum_M[o] + hs[3] * dm; }
     }
   }
+  if (rb + 1 < rb1) __syncthreads();  // the group sums are reused
+  }
   // 6. centroid velocity xdot_c = c^{-1/2} X_c / M_00 and its stage update
-  if (k0 != 0) return;
+  if (rb0 != 0) return;
+  // c^{-1/2} (order 0 has only c^0 in its powers, and c^{-1})
+  const double cpow1 = M >= 1 ? cpow[1] : sqrt(cinv[0]);
   for (int idx = threadIdx.x; idx < TG * 2; idx += NT) {
     const int tt = idx >> 1, comp = idx & 1, p = j0 + tt;
     if (p >= A.n) continue;
     const int j = A.perm ? A.perm[p] : p;
-    const double dx = X[idx] / (sqrt(c) * m00s[tt]);
+    const double dx = X[idx] * cpow1 * m00s[tt];
     const size_t ox = (size_t)j * 2 + comp;
     if (A.mode == 0) {
       A.out_dx[ox] = dx;
     } else {
-      const double h = *A.dt_dev;
       const double base = A.y_x[ox];
-      if (A.mode == 1) { A.ys_x[ox] = base + 0.5 * h * dx; A.sum_x[ox] = base + h / 6.0 * dx; }
-      if (A.mode == 2) { A.ys_x[ox] = base + 0.5 * h * dx; A.sum_x[ox] += h / 3.0 * dx; }
-      if (A.mode == 3) { A.ys_x[ox] = base + h * dx;       A.sum_x[ox] += h / 3.0 * dx; }
-      if (A.mode == 4) { A.y_x[ox] = A.sum_x[ox] + h / 6.0 * dx; }
+      if (A.mode == 1) { A.ys_x[ox] = base + hs[1] * dx; A.sum_x[ox] = base + hs[3] * dx; }
+      if (A.mode == 2) { A.ys_x[ox] = base + hs[1] * dx; A.sum_x[ox] += hs[2] * dx; }
+      if (A.mode == 3) { A.ys_x[ox] = base + hs[0] * dx; A.sum_x[ox] += hs[2] * dx; }
+      if (A.mode == 4) { A.y_x[ox] = A.sum_x[ox] + hs[3] * dx; }
     }
   }
 }
@@ -400,8 +533,8 @@ template <int TG>
 __global__ void __launch_bounds__(kFinishThreads) finish_kernel(FinishArgs A) {
   extern __shared__ double sm[];
   const bool split = gridDim.y > 1;
-  finish_block<TG>(A, blockIdx.x * TG, split ? A.tab.rb_off[blockIdx.y] : 0,
-                   split ? A.tab.rb_off[blockIdx.y + 1] : A.K, sm);
+  finish_block<TG>(A, blockIdx.x * TG, split ? blockIdx.y : 0, split ? blockIdx.y + 1 : A.tab.nrb,
+                   sm);
 }
 
 __global__ void advance_time_kernel(double* t_dev, const double* dt_dev) {
@@ -508,7 +641,7 @@ __global__ void __launch_bounds__(kFinishThreads) finish_batch_kernel(BatchFinis
     A.ys_M = I.state + blk + 2 * (size_t)I.n;
     A.sum_x = I.state + 2 * blk;
     A.sum_M = I.state + 2 * blk + 2 * (size_t)I.n;
-    finish_block<TG>(A, w.y, 0, B.K, sm);
+    finish_block<TG>(A, w.y, 0, B.tab.nrb, sm);
     __syncthreads();  // shared memory is reused by the next item
   }
 }
@@ -561,30 +694,30 @@ cudaError_t launch_prep_batch(int precision, int M, const BatchInst* inst, const
   return cudaGetLastError();
 }
 
-// Shared memory of a finish CTA of TG targets and np pieces.
-size_t finish_smem_bytes(int M, int TG, int np) {
-  return sizeof(double) * ((size_t)TG * (n_beta(M) + n_moments(M) + 3 + np) + M + 1);
+// Shared memory of a finish CTA of TG targets.
+size_t finish_smem_bytes(int M, int TG, const FinishTab& tab) {
+  return sizeof(double) *
+         ((size_t)TG * (n_beta(M) + n_moments(M) + 3 + tab.max_groups) + scal_len(M));
 }
 
-// Call f(kernel of TG targets) for the run-time TG in {1, 4, 8, 16, 32}.
+// Call f(kernel of TG targets) for the run-time TG in {1, 2, 4, 8}.
 template <typename F>
 cudaError_t with_targets(int TG, F&& f) {
   switch (TG) {
     case 1: return f(std::integral_constant<int, 1>{});
+    case 2: return f(std::integral_constant<int, 2>{});
     case 4: return f(std::integral_constant<int, 4>{});
-    case 8: return f(std::integral_constant<int, 8>{});
-    case 16: return f(std::integral_constant<int, 16>{});
-    default: return f(std::integral_constant<int, 32>{});
+    default: return f(std::integral_constant<int, 8>{});
   }
 }
 
 // Targets per batch item: instances of 64 to 8192 particles give 8-target
 // items enough CTAs; orders above the pair limit hold one particle.
-int finish_batch_targets(int M) { return M > 8 ? 1 : 8; }
+int finish_batch_targets(int M) { return M > 8 ? 1 : M > 6 ? 4 : 8; }
 
 cudaError_t launch_finish_batch(const BatchFinishArgs& B, int grid, cudaStream_t st) {
   const int TG = finish_batch_targets(B.M);
-  const size_t smem = finish_smem_bytes(B.M, TG, B.tab.np);
+  const size_t smem = finish_smem_bytes(B.M, TG, B.tab);
   return with_targets(TG, [&](auto tg) {
     constexpr int T = decltype(tg)::value;
     if (smem > 48 * 1024) {
@@ -626,35 +759,39 @@ cudaError_t launch_group_multipole(int M, int n, const void* rec, void* gdata,
 
 cudaError_t launch_prep(int precision, int n, int M, const int* perm, const double* x,
                         const double* mom, const double* t_dev, const double* dt_dev, double cs,
-                        double lam0sq, double four_nu, void* rec, void* gbox, cudaStream_t st) {
+                        double lam0sq, double four_nu, void* rec, void* gbox, double* scal,
+                        cudaStream_t st) {
   const int K = n_moments(M);
-  const int threads = 128, blocks = (n + threads - 1) / threads;
+  const int threads = kPrepThreads, blocks = (n + kGroup - 1) / kGroup + (scal ? 1 : 0);
   if (precision == 1) {
     prep_kernel<float><<<blocks, threads, 0, st>>>(n, M, K, rec_len<float>(M), perm, x, mom,
                                                    t_dev, dt_dev, cs, lam0sq, four_nu,
-                                                   (float*)rec, (float*)gbox, gdata_len(M));
+                                                   (float*)rec, (float*)gbox, gdata_len(M), scal);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess || !gbox) return e;
     return launch_group_multipole(M, n, rec, gbox, nullptr, nullptr, nullptr, n, st);
   }
   prep_kernel<double><<<blocks, threads, 0, st>>>(n, M, K, rec_len<double>(M), perm, x, mom,
                                                   t_dev, dt_dev, cs, lam0sq, four_nu,
-                                                  (double*)rec, nullptr, 0);
+                                                  (double*)rec, nullptr, 0, scal);
   return cudaGetLastError();
 }
 
-// Targets per finish CTA: the largest of 32, 16, 8, 4, 1 that still gives 4
-// CTAs per SM (the FP64 pipe of every SM then has work to the end).
-int finish_targets(int n, int sms) {
-  for (int TG : {32, 16, 8, 4})
-    if ((n + TG - 1) / TG >= 4 * sms) return TG;
+int finish_scalars(int M) { return scal_len(M); }
+
+// Targets per finish CTA: 8 keep every lane of the FP64 instructions in use (the
+// group sums of 8 targets at M = 6 take 48 KB; orders 7 and 8, with up to 127
+// KB, take 4), fewer while there are not 3 CTAs per SM.
+int finish_targets(int n, int M, int sms) {
+  for (int TG : {8, 4, 2})
+    if (!(TG == 8 && M > 6) && (n + TG - 1) / TG >= 3 * sms) return TG;
   return 1;
 }
 
 cudaError_t launch_finish(const FinishArgs& A, int sms, cudaStream_t st) {
-  const int TG = finish_targets(A.n, sms);
+  const int TG = finish_targets(A.n, A.M, sms);
   const int rb = A.n == 1 ? A.tab.nrb : 1;
-  const size_t smem = finish_smem_bytes(A.M, TG, rb > 1 ? A.tab.rb_pieces : A.tab.np);
+  const size_t smem = finish_smem_bytes(A.M, TG, A.tab);
   return with_targets(TG, [&](auto tg) {
     constexpr int T = decltype(tg)::value;
     if (smem > 48 * 1024) {

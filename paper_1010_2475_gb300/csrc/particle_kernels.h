@@ -22,6 +22,7 @@ struct FinishArgs {
   const int* perm = nullptr;        // sorted position -> particle (null: identity)
   const double* Min = nullptr;      // stage moments (n x K)
   FinishTab tab;                    // finish tables (tables.h)
+  const double* scal = nullptr;     // powers of c and weights of the step (null: formed here)
   double lam0sq = 0, four_nu = 0;   // lambda^2 = lam0sq + four_nu * t
   const double* t_dev = nullptr;    // step start time
   const double* dt_dev = nullptr;   // step size (null: 0)
@@ -131,7 +132,9 @@ cudaError_t launch_dp_error(int n, int K, const double* y_x, const double* y_M,
 
 cudaError_t launch_prep(int precision, int n, int M, const int* perm, const double* x,
                         const double* mom, const double* t_dev, const double* dt_dev, double cs,
-                        double lam0sq, double four_nu, void* rec, void* gbox, cudaStream_t st);
+                        double lam0sq, double four_nu, void* rec, void* gbox, double* scal,
+                        cudaStream_t st);
+int finish_scalars(int M);  // doubles launch_prep writes to scal (nullable)
 // Centre, radius and expansion of every group (after the boxes are written);
 // in a batch (inst non-null) n_slots and slot_inst give the slots, else n.
 cudaError_t launch_group_multipole(int M, int n, const void* rec, void* gdata,

@@ -32,70 +32,79 @@ long double pow4l(int e) {
   return r;
 }
 
-// Pieces, their interleaved layout and the row blocks of t from the rows'
-// entries (FinEntry::l holds the group on entry).
-void cut_rows(FinishTables& t, const std::vector<std::vector<FinEntry>>& rows) {
-  size_t total = 0;
-  for (const auto& r : rows) total += r.size();
-  // ~128 pieces keep the threads of a CTA busy.  Orders above the pair limit
-  // serve one particle: short pieces, since a thread's dependent multiply-adds
-  // are what such an evaluation waits for (order 10: 96 entries per thread took
-  // 26 us per right-hand side, 16 took 20 us).
-  const size_t piece = t.M > 8 ? 8 : std::min<size_t>(std::max<size_t>(total / 128, 8), 96);
-  std::vector<std::vector<FinEntry>> ps;
-  t.row_off.assign(1, 0);
-  for (const auto& r : rows) {
-    const size_t cnt = (r.size() + piece - 1) / piece;
-    for (size_t i = 0; i < cnt; ++i) {
-      const size_t e0 = i * r.size() / cnt, e1 = (i + 1) * r.size() / cnt;
-      std::vector<FinEntry> p(r.begin() + e0, r.begin() + e1);
-      for (size_t e = 0; e + 1 < p.size(); ++e)
-        if (p[e].l == p[e + 1].l) p[e].l = -1;  // only the last entry of a group closes it
-      ps.push_back(std::move(p));
+// One row's entries by group l.
+struct Group {
+  int k, l;
+  std::vector<FinEntry> e;
+};
+
+// The row blocks and the interleaved entries of t from the groups (by row).
+void lay_out(FinishTables& t, const std::vector<std::vector<Group>>& rows) {
+  size_t total = 0, groups = 0;
+  for (const auto& r : rows)
+    for (const Group& g : r) {
+      total += g.e.size();
+      ++groups;
     }
-    t.row_off.push_back((int)ps.size());
-  }
-  t.np = (int)ps.size();
-  size_t plen = 0;
-  for (const auto& p : ps) plen = std::max(plen, p.size());
-  t.tab.assign(plen * ps.size(), FinEntry{0.0, 0, -1});
-  t.piece_len.clear();
-  for (size_t p = 0; p < ps.size(); ++p) {
-    t.piece_len.push_back((int)ps[p].size());
-    for (size_t j = 0; j < ps[p].size(); ++j) t.tab[j * ps.size() + p] = ps[p][j];
-  }
-  // row blocks of ~256 pieces, one per thread of a CTA
-  const int want = (int)std::min<size_t>(std::max<size_t>(ps.size() / 256, 1), 64);
-  t.rb_off.assign(1, 0);
+  // orders above the pair limit serve one particle: a CTA per ~64 groups, four
+  // threads each
+  const int want = t.M > 8 ? (int)std::min<size_t>(std::max<size_t>(groups / 64, 1), 128) : 1;
+  std::vector<int> cut(1, 0);
   size_t run = 0;
   for (int k = 0; k < t.K; ++k) {
-    run += rows.size() ? rows[k].size() : 0;
-    if (run * want >= total * t.rb_off.size() && (int)t.rb_off.size() < want)
-      t.rb_off.push_back(k + 1);
+    for (const Group& g : rows[k]) run += g.e.size();
+    if (run * want >= total * cut.size() && (int)cut.size() < want) cut.push_back(k + 1);
   }
-  if (t.rb_off.back() != t.K) t.rb_off.push_back(t.K);
-  t.nrb = (int)t.rb_off.size() - 1;
-  t.rb_pieces = 0;
-  for (int i = 0; i < t.nrb; ++i)
-    t.rb_pieces = std::max(t.rb_pieces, t.row_off[t.rb_off[i + 1]] - t.row_off[t.rb_off[i]]);
+  if (cut.back() != t.K) cut.push_back(t.K);
+  t.nrb = (int)cut.size() - 1;
+  t.max_groups = 0;
+  t.rows_off.assign(1, 0);
+  for (int i = 0; i < t.nrb; ++i) {
+    RowBlock rb{};
+    rb.k0 = cut[i];
+    rb.k1 = cut[i + 1];
+    rb.len_at = (int)t.glen.size();
+    rb.off_at = (int)t.offs.size();
+    std::vector<const Group*> gs;
+    for (int k = rb.k0; k < rb.k1; ++k)
+      for (const Group& g : rows[k]) gs.push_back(&g);
+    std::stable_sort(gs.begin(), gs.end(),
+                     [](const Group* a, const Group* b) { return a->e.size() > b->e.size(); });
+    rb.groups = (int)gs.size();
+    t.max_groups = std::max(t.max_groups, rb.groups);
+    for (const Group* g : gs) t.glen.push_back((int)g->e.size());
+    const size_t longest = gs.empty() ? 0 : gs[0]->e.size();
+    for (size_t j = 0; j < longest; ++j) {
+      t.offs.push_back((int)t.tab.size());
+      for (size_t q = 0; q < gs.size() && gs[q]->e.size() > j; ++q) t.tab.push_back(gs[q]->e[j]);
+    }
+    for (int k = rb.k0; k < rb.k1; ++k) {
+      for (size_t q = 0; q < gs.size(); ++q)
+        if (gs[q]->k == k) t.rows.push_back({(int)q, gs[q]->l});
+      t.rows_off.push_back((int)t.rows.size());
+    }
+    t.blocks.push_back(rb);
+  }
 }
 
 struct BlobOffsets {
-  size_t tab, piece_len, row_off, rb_off, psi0, bytes;
+  size_t tab, blocks, glen, offs, rows, rows_off, psi0, bytes;
 };
 BlobOffsets blob_offsets(const FinishTables& t) {
   BlobOffsets o;
   size_t off = 0;
-  auto take = [&](size_t bytes) {
+  auto take = [&](const auto& v) {
     const size_t at = off;
-    off = (off + bytes + 255) & ~(size_t)255;
+    off = (off + v.size() * sizeof(v[0]) + 255) & ~(size_t)255;
     return at;
   };
-  o.tab = take(t.tab.size() * sizeof(FinEntry));
-  o.piece_len = take(t.piece_len.size() * sizeof(int));
-  o.row_off = take(t.row_off.size() * sizeof(int));
-  o.rb_off = take(t.rb_off.size() * sizeof(int));
-  o.psi0 = take(t.psi0.size() * sizeof(double));
+  o.tab = take(t.tab);
+  o.blocks = take(t.blocks);
+  o.glen = take(t.glen);
+  o.offs = take(t.offs);
+  o.rows = take(t.rows);
+  o.rows_off = take(t.rows_off);
+  o.psi0 = take(t.psi0);
   o.bytes = off;
   return o;
 }
@@ -105,14 +114,16 @@ BlobOffsets blob_offsets(const FinishTables& t) {
 std::vector<unsigned char> FinishTables::blob() const {
   const BlobOffsets o = blob_offsets(*this);
   std::vector<unsigned char> b(o.bytes, 0);
-  auto put = [&](size_t at, const void* src, size_t bytes) {
-    if (bytes) std::memcpy(b.data() + at, src, bytes);
+  auto put = [&](size_t at, const auto& v) {
+    if (!v.empty()) std::memcpy(b.data() + at, v.data(), v.size() * sizeof(v[0]));
   };
-  put(o.tab, tab.data(), tab.size() * sizeof(FinEntry));
-  put(o.piece_len, piece_len.data(), piece_len.size() * sizeof(int));
-  put(o.row_off, row_off.data(), row_off.size() * sizeof(int));
-  put(o.rb_off, rb_off.data(), rb_off.size() * sizeof(int));
-  put(o.psi0, psi0.data(), psi0.size() * sizeof(double));
+  put(o.tab, tab);
+  put(o.blocks, blocks);
+  put(o.glen, glen);
+  put(o.offs, offs);
+  put(o.rows, rows);
+  put(o.rows_off, rows_off);
+  put(o.psi0, psi0);
   return b;
 }
 
@@ -121,13 +132,14 @@ FinishTab finish_tab(const FinishTables& t, const void* base) {
   const unsigned char* p = static_cast<const unsigned char*>(base);
   FinishTab f;
   f.tab = reinterpret_cast<const FinEntry*>(p + o.tab);
-  f.piece_len = reinterpret_cast<const int*>(p + o.piece_len);
-  f.row_off = reinterpret_cast<const int*>(p + o.row_off);
-  f.rb_off = reinterpret_cast<const int*>(p + o.rb_off);
+  f.blocks = reinterpret_cast<const RowBlock*>(p + o.blocks);
+  f.glen = reinterpret_cast<const int*>(p + o.glen);
+  f.offs = reinterpret_cast<const int*>(p + o.offs);
+  f.rows = reinterpret_cast<const RowGroup*>(p + o.rows);
+  f.rows_off = reinterpret_cast<const int*>(p + o.rows_off);
   f.psi0 = reinterpret_cast<const double*>(p + o.psi0);
-  f.np = t.np;
   f.nrb = t.nrb;
-  f.rb_pieces = t.rb_pieces;
+  f.max_groups = t.max_groups;
   return f;
 }
 
@@ -137,7 +149,7 @@ FinishTables build_finish_tables(int M, bool entries) {
   t.K = n_moments(M);
   t.NB = n_beta(M);
   t.NJ = jet_order(M);
-  std::vector<std::vector<FinEntry>> rows(t.K);  // entries by row, grouped by l
+  std::vector<std::vector<Group>> rows(t.K);  // groups by row
   for (int kn = 0, kcol = 0; entries && kn <= M; ++kn) {
     for (int k2 = 0; k2 <= kn; ++k2, ++kcol) {
       const int k1 = kn - k2;
@@ -171,11 +183,13 @@ FinishTables build_finish_tables(int M, bool entries) {
       }
       for (auto& kv : acc) {
         if (kv.second == 0.0L) continue;
-        rows[kcol].push_back({(double)kv.second, kv.first.second, kv.first.first});
+        std::vector<Group>& r = rows[kcol];
+        if (r.empty() || r.back().l != kv.first.first) r.push_back({kcol, kv.first.first, {}});
+        r.back().e.push_back({(double)kv.second, kv.first.second, 0});
       }
     }
   }
-  cut_rows(t, rows);
+  lay_out(t, rows);
   // psi0 (jet of the Gaussian-vortex stream function at the origin, c = 1)
   t.psi0.assign(tri(t.NJ + 1), 0.0);
   const long double inv4pi = 0.0795774715459476678844418816862571810L;

@@ -26,40 +26,52 @@
 
 namespace mmvm {
 
-// One (k, l, beta) entry.  The entries of a row k are grouped by l, so that a
-// row is sum_l a_l (sum_beta c Psi[beta]): one multiply-add per entry and one
-// per (k, l) group.
+// One (k, l, beta) entry.
 struct FinEntry {
   double c;  // coefficient
   int b;     // Psi column beta (bcol)
-  int l;     // moment column l on the last entry of a group, else -1
+  int pad;
 };
 
-// The rows are cut into pieces of similar length (whole groups or parts of
-// one), one thread sums a piece.  Entry j of piece p sits at tab[j * np + p],
-// so threads on neighbouring pieces read neighbouring entries; row k owns the
-// pieces [row_off[k], row_off[k + 1]).  Row blocks [rb_off[i], rb_off[i + 1])
-// split the rows of a single particle over several CTAs (similar entry counts).
+// The moment equation as R_k = sum_l a_l g_kl, g_kl = sum_beta c Psi[beta]: the
+// entries form one group per (k, l).  The rows are split into row blocks (one,
+// or several CTAs' worth for the single particles of high order); the groups
+// of a block are sorted by length, longest first, and entry j of its group q
+// sits at tab[off[j] + q], so that threads on neighbouring groups run equally
+// long loops over neighbouring entries.
+struct RowBlock {
+  int k0, k1;    // rows
+  int groups;    // groups of the block
+  int len_at;    // group lengths: glen[len_at + q]
+  int off_at;    // off[j] = offs[off_at + j], j below the longest group's length
+  int row_at;    // row k's groups: rows[rows_off[k] .. rows_off[k + 1]) hold (q, l)
+};
+struct RowGroup {
+  int q, l;
+};
 struct FinishTables {
   int M = 0, K = 0, NB = 0, NJ = 0;
-  int np = 0, nrb = 1;
-  int rb_pieces = 0;           // most pieces of a row block
+  int nrb = 1;
+  int max_groups = 0;              // most groups of a row block
   std::vector<FinEntry> tab;
-  std::vector<int> piece_len;  // np
-  std::vector<int> row_off;    // K + 1
-  std::vector<int> rb_off;     // nrb + 1
-  std::vector<double> psi0;    // psi0 for |alpha| <= NJ, column q(|alpha|) + alpha_2
+  std::vector<RowBlock> blocks;    // nrb
+  std::vector<int> glen, offs;
+  std::vector<RowGroup> rows;
+  std::vector<int> rows_off;       // K + 1
+  std::vector<double> psi0;        // psi0 for |alpha| <= NJ, column q(|alpha|) + alpha_2
   std::vector<unsigned char> blob() const;  // all of them, 256-byte aligned parts
 };
 
 // Device view of a blob() copied to `base`.
 struct FinishTab {
   const FinEntry* tab = nullptr;
-  const int* piece_len = nullptr;
-  const int* row_off = nullptr;
-  const int* rb_off = nullptr;
+  const RowBlock* blocks = nullptr;
+  const int* glen = nullptr;
+  const int* offs = nullptr;
+  const RowGroup* rows = nullptr;
+  const int* rows_off = nullptr;
   const double* psi0 = nullptr;
-  int np = 0, nrb = 1, rb_pieces = 0;
+  int nrb = 1, max_groups = 0;
 };
 FinishTab finish_tab(const FinishTables& t, const void* base);
 

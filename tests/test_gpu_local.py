@@ -98,7 +98,7 @@ def test_tree_levels(mm, groups, monkeypatch):
 
 @pytest.mark.parametrize("n", [1, 2, 2431, 2433, 4865, 9729, 19457])
 def test_finish_shapes(mm, n):
-    """Targets per finish CTA (1, 4, 8, 16, 32) on both sides of each switch."""
+    """One and many targets per finish CTA, full and ragged."""
     wl = mmvm_inputs.random_disk(n=n, order=3, radius=4.0, seed=n) if n > 1 else \
         mmvm_inputs.single_quadrupole(order=3)
     with mm.Context(3, wl.lam0, wl.nu, mm.MMVM_FP64) as ctx:
@@ -110,6 +110,26 @@ def test_finish_shapes(mm, n):
     if n > 1:
         assert vel_error_rows(gx[rows], ox) <= 1e-12
     assert rhs_error_rows(gM[rows], oM, 3, lam) <= 1e-12
+
+
+# the group-sorted moment table at 1, 2, 4 and 8 targets per CTA, ragged tails
+@pytest.mark.parametrize("order,n", [(0, 1826), (1, 3655), (2, 1), (5, 911), (6, 3651), (6, 913),
+                                     (7, 1825), (7, 3650), (8, 2), (8, 1827)])
+def test_finish_groups(mm, order, n):
+    wl = mmvm_inputs.random_disk(n=n, order=order, radius=4.0, seed=n) if n > 1 else \
+        mmvm_inputs.single_quadrupole(order=order)
+    with mm.Context(order, wl.lam0, wl.nu, mm.MMVM_FP64) as ctx:
+        ctx.set_state(wl.x, wl.moments, 0.3)
+        gx, gM = ctx.rhs()
+    rows = np.array(sorted({0, n - 1, n // 2, *range(max(0, n - 3), n)}))
+    ox, oM = rhs_regrouped(wl.x, wl.moments, 0.3, order, wl.lam0, wl.nu, rows=rows)
+    sx, sM = abs_scale_rows(wl.x, wl.moments, 0.3, order, wl.lam0, wl.nu, rows)
+    if n > 1:
+        assert vel_error_cond(gx[rows], ox, sx) <= 1e-12
+    if order >= 1 and n > 1:
+        assert rhs_error_cond(gM[rows], oM, sM, order, lam_at(0.3, wl.lam0, wl.nu)) <= 1e-12
+    elif order >= 1:
+        assert rhs_error_rows(gM[rows], oM, order, lam_at(0.3, wl.lam0, wl.nu)) <= 1e-12
 
 
 @pytest.mark.parametrize("order", range(9))
