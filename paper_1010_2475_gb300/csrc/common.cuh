@@ -127,15 +127,21 @@ __host__ __device__ constexpr int gdata_len(int M) { return round_up(8 + 2 * m2p
 // a target group's field (2M + extra <= 31: one lane per order), the widest
 // group they serve, and the least separation x = |t0 - s0|^2 of two groups, the
 // wider of radius r: the further apart, the faster the expansions converge.
-// Measured against FP64 on two patches and disks (2-norm of the moment rates,
-// with / without expansions): M = 6, n = 65536: 1.8e-7 / 1.9e-7, n = 40000:
-// 2.1e-7 / 2.1e-7, M = 4 disk, n = 8192: 2.7e-7 / 3.3e-7.  A limit of 2.0 at
-// M = 6 lets single particles reach 7e-6 (n = 8192), 1.4 at M = 8 1e-4.
+// Up to loc_core kLocMinX is enough; beyond, x grows by loc_slope per unit of the
+// radius.  What they keep small is the remainder of the Taylor series of the
+// Gaussian part, e^{-x} at orders up to 2M + 1 + P; with 0.9 and 40 .. 80 at
+// M >= 4 single particles of groups of radius 0.7 .. 1.1 were off by up to 100
+// times the error without expansions (M = 6, disk of 16000).  Errors against
+// FP64 with / without expansions, two patches of 8192, 20000, 36000 and disks of
+// 6000, 16000, 30011, 44000, M = 6: velocities 0.91 .. 1.01 (2-norm), 0.77 .. 1.28
+// (largest), moment rates 0.98 .. 1.03 and 0.94 .. 1.19; a radius of 2.0 with
+// slope 40 at M = 4 and 5 adds 10 to 20 % to the moment rates' error (two patches
+// of 8192).
 __host__ __device__ constexpr int loc_extra(int M) {
   return M <= 1 ? 13 : M == 2 ? 14 : M == 3 ? 15 : M == 4 ? 16 : M <= 7 ? 17 : 15;
 }
 __host__ __device__ constexpr float loc_radius(int M) {
-  return M <= 5 ? 2.0f : M == 6 ? 1.7f : M == 7 ? 1.1f : 0.85f;
+  return M <= 2 ? 2.0f : M <= 4 ? 1.8f : M == 5 ? 1.6f : M == 6 ? 1.7f : M == 7 ? 1.1f : 0.85f;
 }
 // Widest target group whose far field is taken through its local field: at
 // most 0.3 of the distance to anything beyond x_far(M), so that the Taylor
@@ -145,10 +151,10 @@ __host__ __device__ constexpr float loc_field_radius(int M) {
        : M == 5 ? 3.2f : M == 6 ? 3.4f : M == 7 ? 3.4f : 3.2f;
 }
 __host__ __device__ constexpr float loc_core(int M) {  // up to this radius kLocMinX is enough
-  return M <= 6 ? 0.9f : M == 7 ? 0.8f : 0.7f;
+  return M <= 2 ? 0.9f : M == 3 ? 0.8f : M == 4 ? 0.6875f : M <= 7 ? 0.5625f : 0.4375f;
 }
 __host__ __device__ constexpr float loc_slope(int M) {  // of the least x beyond loc_core
-  return M <= 5 ? 40.f : M == 6 ? 50.f : M == 7 ? 80.f : 100.f;
+  return M == 3 ? 50.f : M == 4 ? 55.f : M <= 6 ? 40.f : 60.f;
 }
 
 // Binary tree over G groups of kGroup sorted records (the far field of the

@@ -14,8 +14,8 @@ import pytest
 import mmvm_inputs
 from oracle.diagnostics import vorticity
 from oracle.rhs import lam_at, rhs_regrouped
-from tests.parity_util import (abs_scale_rows, rhs_error_cond, rhs_error_rows, vel_error_cond,
-                               vel_error_rows)
+from tests.parity_util import (abs_scale_rows, rhs_error_cond, rhs_error_rows, vel_error,
+                               vel_error_cond, vel_error_rows)
 
 pytestmark = pytest.mark.gpu
 
@@ -69,6 +69,33 @@ def test_group_expansions(mm, order, n, monkeypatch):
             assert rhs_error_cond(gM[rows], oM, sM, order, wl.lam0) <= tol, key
     if n > 1000:  # the expansions were really used: other roundings
         assert any(not np.array_equal(res[nd, "0"][i], res[nd, "1"][i]) for i in range(2))
+
+
+# groups of radius 0.6 to 1.2 core sizes, where the remainder of the Gaussian
+# part's Taylor series sets the least separation
+@pytest.mark.parametrize("order,kind,n", [(4, "patches", 20000), (5, "patches", 20000),
+                                          (6, "disk", 16000), (6, "patches", 20000),
+                                          (7, "disk", 16000), (8, "disk", 30011)])
+def test_expansions_of_moderate_groups(mm, order, kind, n, monkeypatch):
+    """No particle's velocity further off than the far field's bound (2e-6 of
+    the largest velocity) against the FP64 form."""
+    if kind == "patches":
+        wl = mmvm_inputs.two_patches(n=n, order=order, sigma=0.1, seed=600 + order)
+    else:
+        wl = mmvm_inputs.random_disk(n=n, order=order, radius=10.0, sigma=0.5, seed=n)
+    wl.moments[:, 3:] = np.random.default_rng(order).normal(size=wl.moments[:, 3:].shape) \
+        * 1e-3 * wl.moments[:, :1] * wl.lam0 ** 2
+    monkeypatch.setenv("MMVM_PAIR_VARIANT", str(mm.pair_variant_counts(order)[0]))
+    monkeypatch.setenv("MMVM_FAR_TREE", "1")
+    monkeypatch.setenv("MMVM_LOCAL", "1")
+    with mm.Context(order, wl.lam0, wl.nu, mm.MMVM_MIXED_FP32) as ctx:
+        ctx.set_state(wl.x, wl.moments, 0.0)
+        gx = ctx.rhs()[0]
+    monkeypatch.delenv("MMVM_PAIR_VARIANT")
+    with mm.Context(order, wl.lam0, wl.nu, mm.MMVM_FP64) as ctx:
+        ctx.set_state(wl.x, wl.moments, 0.0)
+        rx = ctx.rhs()[0]
+    assert vel_error(gx, rx) <= 2e-6
 
 
 @pytest.mark.parametrize("groups", [1, 2, 3, 64, 65, 127, 128, 129, 130, 258])
