@@ -206,6 +206,10 @@ int mmvm_pair_counts(mmvm_ctx* ctx, int64_t* near_pairs, int64_t* far_pairs);
  * about the tile centre), pairs those expansions covered.                   */
 int mmvm_pair_work(mmvm_ctx* ctx, int64_t* out);
 
+/* Of the near pairs of mmvm_pair_work, those that went through the expansions
+ * of compact source groups instead of one full jet each.                     */
+int mmvm_pair_expanded(mmvm_ctx* ctx, int64_t* near_expanded);
+
 /* Right-hand side without any device allocation.  The paper has no
  * counterpart: this is a variant of mmvm_rhs_device for callers that cannot
  * call cudaMalloc (an application that owns all device memory through its own

@@ -56,7 +56,7 @@ EXPORTS = (
     "mmvm_enable_timing",
     "mmvm_pair_time", "mmvm_pair_time_parts", "mmvm_pair_config", "mmvm_pair_variant_counts",
     "mmvm_pair_counts",
-    "mmvm_pair_work", "mmvm_alu_peak",
+    "mmvm_pair_work", "mmvm_pair_expanded", "mmvm_alu_peak",
     "mmvm_rhs_noalloc", "mmvm_integrate", "mmvm_vorticity", "mmvm_nonaxi_enstrophy", "mmvm_server_create", "mmvm_server_destroy", "mmvm_submit",
     "mmvm_poll", "mmvm_server_stats", "mmvm_request_footprint",
 )
@@ -170,6 +170,8 @@ def load_library(path: str = LIB_PATH):
     lib.mmvm_alu_peak.restype = ctypes.c_int
     lib.mmvm_pair_work.argtypes = [P, ctypes.POINTER(ctypes.c_int64)]
     lib.mmvm_pair_work.restype = ctypes.c_int
+    lib.mmvm_pair_expanded.argtypes = [P, ctypes.POINTER(ctypes.c_int64)]
+    lib.mmvm_pair_expanded.restype = ctypes.c_int
     lib.mmvm_pair_counts.argtypes = [P, ctypes.POINTER(ctypes.c_int64),
                                      ctypes.POINTER(ctypes.c_int64)]
     lib.mmvm_pair_counts.restype = ctypes.c_int
@@ -356,6 +358,13 @@ def mmvm_pair_work(h):
     out = (ctypes.c_int64 * 4)()
     _check(load_library().mmvm_pair_work(h, out))
     return tuple(int(v) for v in out)
+
+
+def mmvm_pair_expanded(h) -> int:
+    """Near pairs that went through group expansions so far."""
+    a = ctypes.c_int64()
+    _check(load_library().mmvm_pair_expanded(h, ctypes.byref(a)))
+    return a.value
 
 
 def mmvm_pair_counts(h):

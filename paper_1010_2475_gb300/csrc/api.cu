@@ -111,12 +111,14 @@ struct mmvm_ctx {
   mmvm::PairEntry pe;
   // interaction-list form of the all-pairs kernels (FP32 with the far field):
   // near lists (G x G entries, G counts), far-field partials (lfar blocks of
-  // the edge columns), list segments of the near partials, device error flag
+  // the edge columns), shares of the near pairs (lcut, lpre) and blocks of their
+  // partials, device error flag
   bool list = false;
   mmvm::ListEntry le;
-  int lseg = 1, lfar = 1;
+  int shares = 1, lseg = 2, lfar = 1;
   DevBuf<int2> lent;
-  DevBuf<int> lcnt, errf;
+  DevBuf<int> lcnt, lcut, errf;
+  DevBuf<unsigned long long> lpre;
   DevBuf<double> fpart;
   // far field of the list form through the tree over the groups (walked from
   // the lc-th level, tfar nodes there = far blocks), else the flat far kernel
@@ -184,20 +186,24 @@ int chunks_for(int64_t n, int tpc, int per_sm, int device, int S) {
   return (int)ch;
 }
 
-// Shape of the list form for n records: list segments per target group
-// (enough CTAs of the near kernels for ~20 waves) and source ranges of the
-// far kernel (~8 waves of warps, at least 16 source groups per warp).
-// seg_hint > 0: that many segments (the tuner's choice).
-void list_shape(const mmvm_ctx* c, const mmvm::ListEntry& e, int64_t n, int seg_hint, int* lseg,
-                int* lfar) {
+// Shape of the list form for n records: shares of the near pairs (CTAs of a near
+// kernel: `per` per CTA the device holds), the most shares a group may fall
+// into (2.5 times the average), and source ranges of the far kernel (~8 waves
+// of warps, at least 16 source groups per warp).  seg_hint > 0: `per` (the
+// tuner's choice); else 2, so that a CTA that starts late, behind other work on
+// the device, holds back half as much.
+void list_shape(const mmvm_ctx* c, const mmvm::ListEntry& e, int64_t n, int seg_hint, int* shares,
+                int* lseg, int* lfar) {
   int dev_sms = 0;
   cudaDeviceGetAttribute(&dev_sms, cudaDevAttrMultiProcessorCount, c->cfg.device);
   dev_sms = std::max(dev_sms, 1);
   const int64_t G = (n + mmvm::kGroup - 1) / mmvm::kGroup;
   const int occ = std::max(1, mmvm::list_occupancy(e));
-  int64_t seg = seg_hint > 0 ? seg_hint : (20 * (int64_t)dev_sms * occ + G - 1) / G;
-  if (const char* f = std::getenv("MMVM_LIST_SEGMENTS")) seg = std::atoi(f);  // measurement override
-  *lseg = (int)std::min<int64_t>(std::max<int64_t>(seg, 1), 16);
+  int64_t per = seg_hint > 0 ? seg_hint : 2;
+  if (const char* f = std::getenv("MMVM_LIST_SEGMENTS")) per = std::atoi(f);  // measurement override
+  per = std::min<int64_t>(std::max<int64_t>(per, 1), 16);
+  *shares = (int)(per * dev_sms * occ);
+  *lseg = (int)std::min<int64_t>(2 + (5 * *shares) / (2 * G), 32);
   int focc = 0;
   if (e.far.far_occupancy(&focc) != cudaSuccess) {
     cudaGetLastError();
@@ -217,7 +223,7 @@ void list_shape(const mmvm_ctx* c, const mmvm::ListEntry& e, int64_t n, int seg_
 int pair_launches(const mmvm_ctx* c) {
   if (!c->list) return c->pe.nslices;
   const int G = (int)((c->n + mmvm::kGroup - 1) / mmvm::kGroup);
-  return 1 + (c->tree ? mmvm::tree_levels(G) + 1 : 1) + (c->local ? 4 : 0) + c->le.nslices;
+  return 2 + (c->tree ? mmvm::tree_build_launches(G) + 1 : 1) + (c->local ? 4 : 0) + c->le.nslices;
 }
 
 int choose_chunks(const mmvm_ctx* c, int64_t n) {
@@ -243,7 +249,7 @@ std::mutex g_tune_mu;
 std::map<std::tuple<int, int, int, int, int>, int> g_tuned;
 std::map<std::tuple<int, int, int, int, int>, int> g_tuned_tree;   // list form: tree far field
 std::map<std::tuple<int, int, int, int, int>, int> g_tuned_local;  // list form: local expansions
-std::map<std::tuple<int, int, int, int, int>, int> g_tuned_seg;    // list form: segments (0: rule)
+std::map<std::tuple<int, int, int, int, int>, int> g_tuned_seg;    // list form: shares per CTA slot (0: rule)
 
 int ilog2(int64_t v) {
   int r = 0;
@@ -318,7 +324,7 @@ int ensure_buffers(mmvm_ctx* c, int64_t n) {
 }
 
 // The context's buffers for a list-form evaluation of the given shape.
-mmvm::ListArgs list_args(mmvm_ctx* c, int n, int lseg, int lfar, bool tree, int lc, bool local,
+mmvm::ListArgs list_args(mmvm_ctx* c, int n, int shares, int lseg, int lfar, bool tree, int lc, bool local,
                          int loc_seg, unsigned long long* counts) {
   mmvm::ListArgs A;
   A.rec = reinterpret_cast<const float*>(c->rec.p);
@@ -326,7 +332,10 @@ mmvm::ListArgs list_args(mmvm_ctx* c, int n, int lseg, int lfar, bool tree, int 
   A.gdata = c->gbox.p;
   A.ent = c->lent.p;
   A.cnt = c->lcnt.p;
+  A.shares = shares;
   A.segments = lseg;
+  A.cut = c->lcut.p;
+  A.pre = c->lpre.p;
   A.partial = c->partial.p;
   A.far_ranges = lfar;
   A.fpart = c->fpart.p;
@@ -367,7 +376,7 @@ int enqueue_rhs(mmvm_ctx* c, int mode, const double* xin, const double* min_, do
     if (c->list) {
       MMVM_CK(mmvm::list_launch(
           c->le,
-          list_args(c, n, c->lseg, c->lfar, c->tree, c->lc, c->local, c->loc_seg, c->counts.p),
+          list_args(c, n, c->shares, c->lseg, c->lfar, c->tree, c->lc, c->local, c->loc_seg, c->counts.p),
           c->st, c->timing ? c->evm[slot] : nullptr));
       if (c->timing) c->evm_pending[slot] = true;
     } else {
@@ -413,8 +422,10 @@ int enqueue_rhs(mmvm_ctx* c, int mode, const double* xin, const double* min_, do
   A.M = c->M;
   A.K = c->K;
   A.NB = c->NB;
-  A.nchunks = n > 1 ? (c->list ? c->lseg + (c->local ? 1 : 0) : c->chunks) : 0;
+  A.nchunks = n > 1 ? (c->list ? c->lseg : c->chunks) : 0;
   if (n > 1 && c->list) {
+    A.gshares = c->lcut.p + (n + mmvm::kGroup - 1) / mmvm::kGroup;
+    A.local_block = c->local ? c->lseg : -1;
     A.fpart = c->fpart.p;
     A.nfar = c->tree ? c->tfar : c->lfar;
     A.n_edge = c->le.far.n_edge;
@@ -489,10 +500,10 @@ static cudaError_t time_pair_variant(mmvm_ctx* c, const mmvm::PairEntry& e, int 
 }
 
 // Make the list buffers hold list variant e's shape for n records; the
-// shape goes to *lseg / *lfar.
+// shape goes to *shares, *lseg, *lfar and *loc_seg.
 static int ensure_list_buffers(mmvm_ctx* c, const mmvm::ListEntry& e, int n, bool local,
-                               int seg_hint, int* lseg, int* lfar, int* loc_seg) {
-  list_shape(c, e, n, seg_hint, lseg, lfar);
+                               int seg_hint, int* shares, int* lseg, int* lfar, int* loc_seg) {
+  list_shape(c, e, n, seg_hint, shares, lseg, lfar);
   const int64_t G = (n + mmvm::kGroup - 1) / mmvm::kGroup;
   // ~4 waves of warps (8 per SM) of the local kernel
   *loc_seg = (int)std::min<int64_t>(std::max<int64_t>((32 * (int64_t)c->sms + G - 1) / G, 1), 8);
@@ -507,6 +518,12 @@ static int ensure_list_buffers(mmvm_ctx* c, const mmvm::ListEntry& e, int n, boo
       MMVM_CK(c->ffld.ensure(std::max(ff, c->ffld.cap)));
       c->drop_graph();
     }
+  }
+  const size_t cut = 2 * (size_t)G + *shares;
+  if (cut > c->lcut.cap || (size_t)G + 2 > c->lpre.cap || !c->lcut.p || !c->lpre.p) {
+    MMVM_CK(c->lcut.ensure(std::max(cut, c->lcut.cap)));
+    MMVM_CK(c->lpre.ensure(std::max((size_t)G + 2, c->lpre.cap)));
+    c->drop_graph();
   }
   const size_t tn = (size_t)mmvm::tree_nodes((n + mmvm::kGroup - 1) / mmvm::kGroup) *
                     mmvm::gdata_len(c->M);
@@ -528,12 +545,13 @@ static int ensure_list_buffers(mmvm_ctx* c, const mmvm::ListEntry& e, int n, boo
 // one untimed launch); *per_pair = milliseconds per pair.
 static int time_list_variant(mmvm_ctx* c, const mmvm::ListEntry& e, int n, bool tree, bool local,
                              int seg_hint, cudaEvent_t e0, cudaEvent_t e1, double* per_pair) {
-  int lseg = 1, lfar = 1, loc_seg = 1;
-  int rc = ensure_list_buffers(c, e, n, local, seg_hint, &lseg, &lfar, &loc_seg);
+  int shares = 1, lseg = 2, lfar = 1, loc_seg = 1;
+  int rc = ensure_list_buffers(c, e, n, local, seg_hint, &shares, &lseg, &lfar,
+                                &loc_seg);
   if (rc) return rc;
   int tfar = 1;
   const int lc = mmvm::tree_chunk_level((n + mmvm::kGroup - 1) / mmvm::kGroup, lfar, &tfar);
-  const mmvm::ListArgs A = list_args(c, n, lseg, lfar, tree, lc, local, loc_seg, nullptr);
+  const mmvm::ListArgs A = list_args(c, n, shares, lseg, lfar, tree, lc, local, loc_seg, nullptr);
   MMVM_CK(mmvm::list_launch(e, A, c->st));
   MMVM_CK(cudaEventRecord(e0, c->st));
   MMVM_CK(mmvm::list_launch(e, A, c->st));
@@ -544,9 +562,9 @@ static int time_list_variant(mmvm_ctx* c, const mmvm::ListEntry& e, int n, bool 
   *per_pair = ms / ((double)n * n);
   if (const char* vb = std::getenv("MMVM_TUNE_VERBOSE"))
     if (std::atoi(vb))
-      std::fprintf(stderr, "[mmvm tune] M=%d n=%d list variant %d (near kernels=%d, segments=%d, "
+      std::fprintf(stderr, "[mmvm tune] M=%d n=%d list variant %d (near kernels=%d, shares=%d, "
                    "far %s, far blocks=%d, local %d): %.3f ms, %.3e pairs/s\n", c->M, n, e.variant,
-                   e.nslices, lseg, tree ? "tree" : "flat", tree ? tfar : lfar, local ? 1 : 0, ms,
+                   e.nslices, shares, tree ? "tree" : "flat", tree ? tfar : lfar, local ? 1 : 0, ms,
                    (double)n * n / (ms * 1e-3));
   return MMVM_OK;
 }
@@ -693,11 +711,9 @@ int tune_pair(mmvm_ctx* c) {
           best_v = v;
         }
       }
-      // list segments: enough CTAs against short lists per CTA (n = 4096, M = 4:
-      // 16 segments left 5 rounds of work between a CTA's set-up and its sums)
+      // shares of the near pairs: few set-ups of groups against an even load
       e = mmvm::list_entry(c->M, best_v);
-      for (int seg : {1, 2, 3, 4, 6, 8, 12, 16}) {
-        if (seg > (n + mmvm::kGroup - 1) / mmvm::kGroup) break;
+      for (int seg : {1, 3, 4, 8}) {
         rc = time_list_variant(c, e, n, tree_choice != 0, local_choice != 0, seg, e0, e1,
                                &per_pair);
         if (rc) return rc;
@@ -736,17 +752,20 @@ int tune_pair(mmvm_ctx* c) {
     if (e.M != c->M) return fail(MMVM_E_INVALID_ARG, "MMVM_PAIR_VARIANT out of range");
     MMVM_CK(mmvm::list_prepare(e));
     if (local_choice) MMVM_CK(e.far.loc_prepare());
-    int lseg = 1, lfar = 1, loc_seg = 1;
-    int rc = ensure_list_buffers(c, e, n, local_choice != 0, seg_choice, &lseg, &lfar, &loc_seg);
+    int shares = 1, lseg = 2, lfar = 1, loc_seg = 1;
+    int rc = ensure_list_buffers(c, e, n, local_choice != 0, seg_choice, &shares, &lseg,
+                                  &lfar, &loc_seg);
     if (rc) return rc;
     int tfar = 1;
     const int lc = mmvm::tree_chunk_level((n + mmvm::kGroup - 1) / mmvm::kGroup, lfar, &tfar);
-    if (!c->list || e.variant != c->le.variant || lseg != c->lseg || lfar != c->lfar ||
+    if (!c->list || e.variant != c->le.variant || shares != c->shares ||
+        lseg != c->lseg || lfar != c->lfar ||
         c->tree != (tree_choice != 0) || lc != c->lc || c->local != (local_choice != 0) ||
         loc_seg != c->loc_seg)
       c->drop_graph();
     c->le = e;
     c->list = true;
+    c->shares = shares;
     c->lseg = lseg;
     c->lfar = lfar;
     c->tree = tree_choice != 0;
@@ -886,11 +905,11 @@ int mmvm_create(const mmvm_config* cfg, mmvm_ctx** out) {
   if ((e = c->ftab.ensure(tb.size())) != cudaSuccess || (e = c->scal.ensure(2)) != cudaSuccess ||
       (e = c->flags.ensure(2)) != cudaSuccess ||
       (e = c->fscal.ensure(mmvm::finish_scalars(c->M))) != cudaSuccess ||
-      (e = c->counts.ensure(4)) != cudaSuccess)
+      (e = c->counts.ensure(5)) != cudaSuccess)
     return bail(cuda_fail(e, "cudaMalloc(tables)"));
   if ((e = cudaMemcpy(c->ftab.p, tb.data(), tb.size(), cudaMemcpyHostToDevice)) != cudaSuccess ||
       (e = cudaMemset(c->scal.p, 0, 2 * sizeof(double))) != cudaSuccess ||
-      (e = cudaMemset(c->counts.p, 0, 4 * sizeof(unsigned long long))) != cudaSuccess)
+      (e = cudaMemset(c->counts.p, 0, 5 * sizeof(unsigned long long))) != cudaSuccess)
     return bail(cuda_fail(e, "cudaMemcpy(tables)"));
   c->ft = mmvm::finish_tab(T, c->ftab.p);
   if (c->pe.nslices && (e = mmvm::pair_prepare(c->pe, c->S)) != cudaSuccess)
@@ -921,6 +940,8 @@ void mmvm_destroy(mmvm_ctx* c) {
   c->ffld.release();
   c->lent.release();
   c->lcnt.release();
+  c->lcut.release();
+  c->lpre.release();
   c->errf.release();
   c->rec.release();
   c->counts.release();
@@ -1277,6 +1298,16 @@ int mmvm_pair_work(mmvm_ctx* c, int64_t* out) {
   MMVM_CK(cudaMemcpyAsync(h, c->counts.p, sizeof(h), cudaMemcpyDeviceToHost, c->st));
   MMVM_CK(cudaStreamSynchronize(c->st));
   for (int i = 0; i < 4; ++i) out[i] = (int64_t)h[i];
+  return MMVM_OK;
+}
+
+int mmvm_pair_expanded(mmvm_ctx* c, int64_t* near_expanded) {
+  if (!c || !near_expanded) return fail(MMVM_E_INVALID_ARG, "null argument");
+  MMVM_CK(cudaSetDevice(c->cfg.device));
+  unsigned long long h = 0;
+  MMVM_CK(cudaMemcpyAsync(&h, c->counts.p + 4, sizeof(h), cudaMemcpyDeviceToHost, c->st));
+  MMVM_CK(cudaStreamSynchronize(c->st));
+  *near_expanded = (int64_t)h;
   return MMVM_OK;
 }
 

@@ -174,6 +174,14 @@ __host__ __device__ inline long long tree_level_offset(int G, int L) {
   return off;
 }
 
+// Levels of at most this many nodes are built by one CTA in one launch.
+constexpr int kTreeTop = 64;  // two nodes per warp
+__host__ __device__ inline int tree_build_launches(int G) {
+  int L = 1, top = tree_levels(G), k = 0;
+  for (; L <= top && tree_level_nodes(G, L) > kTreeTop; ++L) ++k;
+  return k + (L <= top ? 1 : 0);
+}
+
 // Compile-time loop: f(std::integral_constant<int, i>) for i in [B, E).
 template <int B, int E, typename F>
 __device__ __forceinline__ void static_for(F&& f) {

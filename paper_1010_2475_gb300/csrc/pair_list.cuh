@@ -9,9 +9,10 @@
 //     consecutive sorted targets, one warp), the source groups whose box
 //     comes within x_far(M) of tg's box, each with the 32-bit mask of its
 //     sources that lie within x_far(M) of tg's box;
-//  2. near pairs (near_pair_kernel): one CTA per (target group, list
-//     segment).  Its W warps serve the same 32 targets and take the
-//     segment's near sources in turn: in round r warp w evaluates the
+//  2. near pairs (near_pair_kernel): the (target group, near source) items of
+//     all groups in one row, cut into equal shares (near_cut_kernel), one CTA
+//     per share.  Its W warps serve the same 32 targets and take the
+//     group's near sources in turn: in round r warp w evaluates the
 //     (r W + w)-th near source, then the CTA meets at one barrier, so all
 //     warps run the same code in step.  Each warp brings its sources into
 //     shared-memory slots of its own by 1-D bulk copies (cp.async.bulk,
@@ -107,6 +108,7 @@ __device__ __forceinline__ bool takes_m2p(const float4 tb, const float4 c) {
 // ent[tg * G + e] = (source group, near mask), e < cnt[tg], in increasing
 // source-group order; only groups with a non-empty mask are listed.  One warp
 // per target group; groups of kGroup sorted records, the last one partial.
+// nsrc[tg] = sources in the listed masks.
 // With rmax > 0 (local expansions), a near group that loc_pair takes goes to
 // the other end of the row instead, ent[tg * G + G - 1 - e], e < mcnt[tg].
 //
@@ -133,14 +135,14 @@ template <int M>
 __global__ void near_list_kernel(const float* __restrict__ rec, int n, int G,
                                  const float* __restrict__ gdata, float rmax,
                                  int2* __restrict__ ent, int* __restrict__ cnt,
-                                 int* __restrict__ mcnt) {
+                                 int* __restrict__ mcnt, int* __restrict__ nsrc) {
   constexpr int R = rec_len<float>(M), GL = gdata_len(M);
   const int lane = threadIdx.x & 31;
   const int nwarps = (gridDim.x * blockDim.x) >> 5;
   for (int tg = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; tg < G; tg += nwarps) {
     const float4 tb = *reinterpret_cast<const float4*>(gdata + (size_t)tg * GL);
     const float4 tc = *reinterpret_cast<const float4*>(gdata + (size_t)tg * GL + 4);
-    int c = 0, mc = 0;
+    int c = 0, mc = 0, ns_all = 0;
     for (int gb = 0; gb < G; gb += 32) {
       const int g = gb + lane;
       bool nearg = false;
@@ -186,12 +188,14 @@ __global__ void near_list_kernel(const float* __restrict__ rec, int n, int G,
           if (m[q]) {
             if (lane == 0) ent[(size_t)tg * G + c] = make_int2(gg[q], (int)m[q]);
             ++c;
+            ns_all += __popc(m[q]);
           }
       }
     }
     if (lane == 0) {
       cnt[tg] = c;
       mcnt[tg] = mc;
+      nsrc[tg] = ns_all;
     }
   }
 }
@@ -225,14 +229,22 @@ struct NearListSmem {
 // pair: one source per round, so 32 sources per flush as in the direct form.
 constexpr int kNearFlush = 32;
 
-// One CTA: the near pairs of target group blockIdx.x against list segment
-// blockIdx.y of C (the entries [y cnt / C, (y+1) cnt / C) of its list); writes
-// this part's columns of partial block blockIdx.y ([NB][n] FP64).
+// One CTA: share blockIdx.x of the near pairs.  pre[g] = near sources of the
+// target groups before g (pre[G] all), pre[G + 1] = sources per share; share t
+// starts in group start[t].  The CTA takes its part of one group after another
+// and writes this part's columns of partial block c ([NB][n] FP64), c = how many
+// shares have had a part of the group before (near_cut_kernel bounds it).
 //
-// The segment is taken in windows of WIN list entries: warp 0 forms the
+// Equal shares: setting up a group (its list, empty sums) and adding the W
+// warps' sums cost as much as ~10 rounds of sources, so a CTA should see few
+// groups, and an SM gets one CTA's worth of rounds whatever the lists' lengths.
+// (A CTA per group and segment of its list, 8 segments per group at n = 5003,
+// M = 6, spent 2/3 of its time outside the sources.)
+//
+// The part is taken in windows of WIN list entries: warp 0 forms the
 // exclusive prefix sums of the entries' near counts, the CTA lists the
 // window's near sources in order (16-bit entry and lane), then round k gives
-// warp w the (k W + w)-th near source of the window.  Each warp brings its own
+// warp w the (k W + w)-th near source of the part in the window.  Each warp brings its own
 // sources into NST record slots of its own, one bulk copy per source issued
 // by its lane 0 NST rounds ahead (completion on the slot's mbarrier), so a
 // warp only ever waits for copies it issued itself.  SYNC > 0: a CTA barrier
@@ -243,7 +255,8 @@ constexpr int kNearFlush = 32;
 template <int M, int LO, int HI, int PART, int W, int MINB, int NST, int SYNC>
 __global__ void __launch_bounds__(W * 32, MINB)
     near_pair_kernel(const float* __restrict__ rec, int n, int G, const int2* __restrict__ ent,
-                     const int* __restrict__ cnt, int C, double* __restrict__ partial,
+                     const int* __restrict__ cnt, const unsigned long long* __restrict__ pre,
+                     const int* __restrict__ start, double* __restrict__ partial,
                      unsigned long long* __restrict__ counts, int* __restrict__ err) {
   using PN = PairNear<M, float, LO, HI, PART>;
   using PC = PartCols<LO, HI, PART>;
@@ -260,11 +273,27 @@ __global__ void __launch_bounds__(W * 32, MINB)
   unsigned long long* bar =
       reinterpret_cast<unsigned long long*>(smem_list + L::bar_off) + (size_t)warp * NST;
 
-  const int tg = blockIdx.x;
+  const unsigned long long share = pre[G + 1], all = pre[G];
+  const unsigned long long lo = blockIdx.x * share, hi = min(lo + share, all);
+  if (lo >= hi) return;  // the whole CTA: nothing left for it
+  if (lane == 0) {
+    for (int s = 0; s < NST; ++s) mbar_init(bar + s, 1);
+    fence_mbar_init();
+  }
+  float* my_hi = acc_hi + warp * NS * 32;
+  float* my_lo = acc_lo + warp * NS * 32;
+  unsigned n_near = 0;
+  bool timeout = false;
+  int tbase = 0;  // sources this warp took in earlier windows (slot t % NST, phase t / NST)
+  for (int tg = start[blockIdx.x]; tg < G; ++tg) {
+  const unsigned long long g0 = pre[tg], g1 = pre[tg + 1];
+  if (g0 >= hi) break;
+  // this group's near sources [sa, sb)
+  const int sa = (int)((lo > g0 ? lo : g0) - g0), sb = (int)((hi < g1 ? hi : g1) - g0);
+  if (sa >= sb) continue;
+  const int block = sa > 0 ? (int)(blockIdx.x - g0 / share) : 0;
   const int j = tg * kGroup + lane;
   const int ne = cnt[tg];
-  const int e0 = (int)((long long)blockIdx.y * ne / C);
-  const int e1 = (int)((long long)(blockIdx.y + 1) * ne / C);
   const int2* tent = ent + (size_t)tg * G;
 
   float tz1 = 3e15f, tz2 = 3e15f, tl1 = 0.f, tl2 = 0.f;
@@ -278,24 +307,16 @@ __global__ void __launch_bounds__(W * 32, MINB)
   float acc[NBL];
 #pragma unroll
   for (int b = 0; b < NBL; ++b) acc[b] = 0.f;
-  float* my_hi = acc_hi + warp * NS * 32;
-  float* my_lo = acc_lo + warp * NS * 32;
   for (int i = lane; i < NS * 32; i += 32) {
     my_hi[i] = 0.f;
     my_lo[i] = 0.f;
   }
-  if (lane == 0) {
-    for (int s = 0; s < NST; ++s) mbar_init(bar + s, 1);
-    fence_mbar_init();
-  }
   __syncthreads();
 
-  unsigned n_near = 0;
-  bool timeout = false;
   int since_flush = 0;
-  int tbase = 0;  // sources this warp took in earlier windows (slot t % NST, phase t / NST)
-  for (int wb = e0; wb < e1; wb += WIN) {
-    const int nw = min(e1 - wb, WIN);
+  int seen = 0;  // near sources of the windows before this one
+  for (int wb = 0; wb < ne && seen < sb; wb += WIN) {
+    const int nw = min(ne - wb, WIN);
     // the window's entries and the exclusive prefix sum of their near counts
     // (warp 0: each lane scans WIN/32 consecutive entries; past nw they count 0)
     if (warp == 0) {
@@ -329,21 +350,28 @@ __global__ void __launch_bounds__(W * 32, MINB)
       if (lane == 31) pref_s[WIN] = incl;
     }
     __syncthreads();
+    const int Lall = pref_s[WIN];
+    const int w0 = max(sa - seen, 0), Lw = min(sb - seen, Lall) - w0;  // this part: w0 + [0, Lw)
+    seen += Lall;
+    if (Lw <= 0) {        // before the part
+      __syncthreads();    // the next window overwrites ent_s / pref_s
+      continue;
+    }
     // every thread lists the near sources of one entry at the entry's offset
     for (int e = threadIdx.x; e < nw; e += W * 32) {
-      unsigned m = (unsigned)ent_s[e].y;
       int q = pref_s[e];
+      if (pref_s[e + 1] <= w0 || q >= w0 + Lw) continue;
+      unsigned m = (unsigned)ent_s[e].y;
       while (m) {
         src_s[q++] = (unsigned short)((e << 5) | (__ffs(m) - 1));
         m &= m - 1;
       }
     }
     __syncthreads();
-    const int Lw = pref_s[WIN];
     const int mine = Lw > warp ? (Lw - 1 - warp) / W + 1 : 0;  // this warp's sources
     // lane 0: bulk copy of the k-th source of this warp into slot (tbase + k) % NST
     auto issue = [&](int k) {
-      const unsigned sv = src_s[warp + k * W];
+      const unsigned sv = src_s[w0 + warp + k * W];
       const int ls = (int)(sv & 31u);
       const int2 en = ent_s[sv >> 5];
       const int t = tbase + k;
@@ -352,12 +380,14 @@ __global__ void __launch_bounds__(W * 32, MINB)
       bulk_copy_g2s(slots + (size_t)(t % NST) * R, rec + ((size_t)en.x * kGroup + ls) * R,
                     (unsigned)(R * 4), b);
     };
-    if (lane == 0)
+    if (lane == 0) {
+      fence_proxy_async_smem();  // the slots' last readers are behind a barrier
       for (int k = 0; k < min(NST, mine); ++k) issue(k);
+    }
     for (int k = 0; k * W < Lw; ++k) {
       const int p = warp + k * W;
       if (p < Lw) {
-        const unsigned sv = src_s[p];
+        const unsigned sv = src_s[w0 + p];
         const int ls = (int)(sv & 31u);
         const int2 en = ent_s[sv >> 5];
         const int t = tbase + k;
@@ -383,28 +413,14 @@ __global__ void __launch_bounds__(W * 32, MINB)
     __syncthreads();  // the next window overwrites ent_s / pref_s
   }
   flush_sums<LO, HI, PART, 32>(acc, my_hi, my_lo, lane);
-  if (timeout) {
-    // a copy may still be in flight: wait (bounded) for this warp's last
-    // NST copies before the CTA's shared memory is released
-    if (lane == 0) {
-      for (int t = max(0, tbase - NST); t < tbase; ++t)
-        mbar_wait_bounded(bar + t % NST, (unsigned)((t / NST) & 1));
-      atomicExch(err, 1);
-    }
-  }
-  if (LO == 1 && PART != 2 && counts != nullptr) {
-    const unsigned wn = __reduce_add_sync(0xffffffffu, n_near);
-    if (lane == 0 && wn) atomicAdd(counts, (unsigned long long)wn);
-  }
   __syncthreads();  // every warp's (hi, lo) sums are in shared memory
-  // (hi, lo) sums of the W warps -> FP64, this part's columns of block y:
+  // (hi, lo) sums of the W warps -> FP64, this part's columns of the block:
   // column c (slot q) is summed by warp q mod W, one target per lane (the
   // column of each slot is a compile-time constant).  The W pairs are added
   // in FP32 with the rounding of every hi addition carried into lo, and only
   // the final pair is widened: FP64 arithmetic is a small fraction of the
   // FP32 rate here, and the CTA's tail runs alone on its SM.
-  double* out = partial + (size_t)blockIdx.y * NB * n + (size_t)PN::B0 * n;
-  const int jj = tg * kGroup + lane;
+  double* out = partial + (size_t)block * NB * n + (size_t)PN::B0 * n;
   static_for<0, NBL>([&](auto cc) {
     constexpr int c = decltype(cc)::value;
     if constexpr (PC::in(c)) {
@@ -419,10 +435,25 @@ __global__ void __launch_bounds__(W * 32, MINB)
           l += ((h - (sum - bp)) + (v - bp)) + acc_lo[(w * NS + q) * 32 + lane];
           h = sum;
         }
-        if (jj < n) out[(size_t)c * n + jj] = (double)h + (double)l;
+        if (j < n) out[(size_t)c * n + j] = (double)h + (double)l;
       }
     }
   });
+  __syncthreads();  // the next group's sums overwrite acc_hi / acc_lo
+  }
+  if (timeout) {
+    // a copy may still be in flight: wait (bounded) for this warp's last
+    // NST copies before the CTA's shared memory is released
+    if (lane == 0) {
+      for (int t = max(0, tbase - NST); t < tbase; ++t)
+        mbar_wait_bounded(bar + t % NST, (unsigned)((t / NST) & 1));
+      atomicExch(err, 1);
+    }
+  }
+  if (LO == 1 && PART != 2 && counts != nullptr) {
+    const unsigned wn = __reduce_add_sync(0xffffffffu, n_near);
+    if (lane == 0 && wn) atomicAdd(counts, (unsigned long long)wn);
+  }
 }
 
 // ------------------------------------------------------------------ 3. far field
@@ -649,9 +680,8 @@ __device__ __forceinline__ void tree_node(const float* child, int nchild, bool c
 
 // Levels L0 .. L1 of the tree.  A grid of several CTAs takes one level (L0 ==
 // L1); the narrow upper levels, at most kTreeTop nodes each, go to one CTA
-// level after level (a launch each, one thread per node, took 8 us apiece: 72
-// of 1100 us per right-hand side at n = 2011, M = 8).
-constexpr int kTreeTop = 64;  // two nodes per warp of the one CTA
+// level after level (a launch each with one thread per node took 54 us per
+// right-hand side at n = 2011, M = 8; now 20 us).
 template <int M>
 __global__ void __launch_bounds__(1024)
     tree_level_kernel(const float* gdata, int n, int G, int L0, int L1, float* tree) {

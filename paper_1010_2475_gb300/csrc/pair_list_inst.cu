@@ -19,10 +19,11 @@ namespace mmvm {
 namespace {
 constexpr int kM = MMVM_INST_M;
 cudaError_t build_fn(const float* rec, int n, int G, const float* gdata, float rmax, int2* ent,
-                     int* cnt, int* mcnt, cudaStream_t st) {
+                     int* cnt, int* mcnt, int* nsrc, cudaStream_t st) {
   // a warp per target group; one warp per CTA while that spreads them over the SMs
   const int wpc = G <= 1024 ? 1 : 8;
-  near_list_kernel<kM><<<(G + wpc - 1) / wpc, 32 * wpc, 0, st>>>(rec, n, G, gdata, rmax, ent, cnt, mcnt);
+  near_list_kernel<kM><<<(G + wpc - 1) / wpc, 32 * wpc, 0, st>>>(rec, n, G, gdata, rmax, ent,
+                                                                    cnt, mcnt, nsrc);
   return cudaGetLastError();
 }
 cudaError_t far_fn(const float* rec, int n, int G, const float* gdata, int S, float frad,
@@ -123,10 +124,10 @@ cudaError_t prepare_fn() {
   return cudaFuncSetAttribute(MMVM_NEAR_KERNEL, cudaFuncAttributeMaxDynamicSharedMemorySize,
                               (int)kSmem);
 }
-cudaError_t launch_fn(const float* rec, int n, int G, const int2* ent, const int* cnt, int C,
-                      double* partial, unsigned long long* counts, int* err, cudaStream_t st) {
-  dim3 grid(G, C);
-  MMVM_NEAR_KERNEL<<<grid, kS.w * 32, kSmem, st>>>(rec, n, G, ent, cnt, C, partial, counts, err);
+cudaError_t launch_fn(const float* rec, int n, int G, const int2* ent, const int* cnt, int T,
+                      const unsigned long long* pre, const int* start, double* partial, unsigned long long* counts, int* err, cudaStream_t st) {
+  MMVM_NEAR_KERNEL<<<T, kS.w * 32, kSmem, st>>>(rec, n, G, ent, cnt, pre, start, partial, counts,
+                                                err);
   return cudaGetLastError();
 }
 cudaError_t occ_fn(int* blocks) {

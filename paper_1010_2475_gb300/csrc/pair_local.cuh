@@ -543,8 +543,11 @@ __global__ void __launch_bounds__(kLocWarps * 32, 2)
   }
   if (counts != nullptr) {  // near pairs covered
     const unsigned tot = __reduce_add_sync(0xffffffffu, nsrc);
-    if (lane == 0)
-      atomicAdd(counts, (unsigned long long)tot * (unsigned)min(kGroup, n - tg * kGroup));
+    const unsigned long long p = (unsigned long long)tot * (unsigned)min(kGroup, n - tg * kGroup);
+    if (lane == 0 && p) {
+      atomicAdd(counts, p);
+      atomicAdd(counts + 4, p);
+    }
   }
 }
 
@@ -758,9 +761,9 @@ __global__ void __launch_bounds__(kLocWarps * 32)
 // columns) and R (columns beta1 >= 2) at its 32 targets into partial block
 // `out` ([NB][n] FP64).  The value at the centre is added in FP64, the rest of
 // the Taylor sum in FP32.  Groups without a local field get zeros.  A warp
-// takes every kEvalWarps-th row of the field and of the results: one warp alone
-// is a chain of ~150 us of dependent shared loads and multiply-adds at M = 8
-// (97 us at n = 24000, M = 6, with 5 warps on an SM).
+// takes every kEvalWarps-th row of the field and of the results: with one warp per
+// group the chain of dependent shared loads and multiply-adds took 77 us at n =
+// 2011, M = 8 (now 33 us) and 97 us at n = 24000, M = 6, with 5 warps on an SM.
 constexpr int kEvalWarps = 4;
 template <int M>
 __global__ void __launch_bounds__(kEvalWarps * 32)

@@ -140,12 +140,94 @@ int tree_chunk_level(int G, int blocks, int* nodes) {
   return L;
 }
 
+namespace {
+
+constexpr int kCutThreads = 1024;
+constexpr int kMinShare = 32;  // sources: about 3 rounds of a CTA's warps
+
+// One CTA: the near sources nsrc[g] of the G target groups, put one group after
+// another, in at most T equal shares, so that no group falls into more than C
+// of them: pre[g] = sources before group g, pre[G] = all, pre[G + 1] = sources
+// per share, gshares[g] = shares that group g falls into, start[t] = group in
+// which share t starts (only set for shares that exist).
+__global__ void __launch_bounds__(kCutThreads)
+    near_cut_kernel(int G, int T, int C, const int* nsrc, unsigned long long* pre, int* gshares,
+                    int* start) {
+  __shared__ unsigned long long wsum[32], total;
+  __shared__ int wmax[32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  unsigned long long run = 0;
+  int most = 0;
+  for (int g0 = 0; g0 < G; g0 += kCutThreads) {
+    const int g = g0 + threadIdx.x;
+    const int w = g < G ? nsrc[g] : 0;
+    most = max(most, w);
+    unsigned long long incl = w;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const unsigned long long v = __shfl_up_sync(0xffffffffu, incl, o);
+      if (lane >= o) incl += v;
+    }
+    if (lane == 31) wsum[warp] = incl;
+    __syncthreads();
+    if (warp == 0) {
+      unsigned long long s = wsum[lane];
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const unsigned long long v = __shfl_up_sync(0xffffffffu, s, o);
+        if (lane >= o) s += v;
+      }
+      wsum[lane] = s;
+      if (lane == 31) total = s;
+    }
+    __syncthreads();
+    if (g < G) pre[g] = run + (warp ? wsum[warp - 1] : 0) + incl - w;
+    run += total;
+    __syncthreads();  // wsum and total are rewritten
+  }
+  most = __reduce_max_sync(0xffffffffu, most);
+  if (lane == 0) wmax[warp] = most;
+  __syncthreads();
+  most = __reduce_max_sync(0xffffffffu, wmax[lane]);
+  // a group of w sources falls into at most ceil(w / share) + 1 shares
+  unsigned long long share = (run + T - 1) / T;
+  share = max(share, (unsigned long long)((most + C - 2) / (C - 1)));
+  share = max(share, (unsigned long long)kMinShare);
+  if (threadIdx.x == 0) {
+    pre[G] = run;
+    pre[G + 1] = share;
+  }
+  __syncthreads();
+  for (int g = threadIdx.x; g < G; g += kCutThreads) {
+    const unsigned long long a = pre[g], b = pre[g + 1];
+    gshares[g] = b > a ? (int)((b - 1) / share - a / share) + 1 : 0;
+  }
+  for (int t = threadIdx.x; t < T; t += kCutThreads) {
+    const unsigned long long at = t * share;
+    if (at >= run) break;
+    int l = 0, h = G - 1;  // the last group with pre <= at: it has sources
+    while (l < h) {
+      const int m = (l + h + 1) >> 1;
+      if (pre[m] <= at) l = m;
+      else h = m - 1;
+    }
+    start[t] = l;
+  }
+}
+
+}  // namespace
+
 cudaError_t list_launch(const ListEntry& e, const ListArgs& A, cudaStream_t st,
                         cudaEvent_t* marks) {
   const int n = A.n, G = (n + kGroup - 1) / kGroup;
   const float rmax = A.local ? e.far.loc_radius : 0.f;
   const float frad = A.local ? e.far.loc_field_radius : 0.f;
-  cudaError_t r = e.far.build(A.rec, n, G, A.gdata, rmax, A.ent, A.cnt, A.cnt + G, st);
+  cudaError_t r = e.far.build(A.rec, n, G, A.gdata, rmax, A.ent, A.cnt, A.cnt + G, A.cut, st);
+  if (r == cudaSuccess) {
+    near_cut_kernel<<<1, kCutThreads, 0, st>>>(G, A.shares, A.segments, A.cut, A.pre, A.cut + G,
+                                               A.cut + 2 * (size_t)G);
+    r = cudaGetLastError();
+  }
   if (A.tree && r == cudaSuccess) r = e.far.tree_build(A.gdata, n, G, A.tree, st);
   if (marks && r == cudaSuccess) r = cudaEventRecord(marks[0], st);
   if (r == cudaSuccess)
@@ -159,7 +241,8 @@ cudaError_t list_launch(const ListEntry& e, const ListArgs& A, cudaStream_t st,
                        A.tree ? tree_level_nodes(G, A.Lc) : A.far_ranges, A.ffld,
                        A.partial + (size_t)A.segments * n_beta(e.M) * n, A.counts, A.err, st);
   for (int s = 0; s < e.nslices && r == cudaSuccess; ++s) {
-    r = e.slices[s].launch(A.rec, n, G, A.ent, A.cnt, A.segments, A.partial, A.counts, A.err, st);
+    r = e.slices[s].launch(A.rec, n, G, A.ent, A.cnt, A.shares, A.pre, A.cut + 2 * (size_t)G, A.partial,
+                           A.counts, A.err, st);
     if (marks && r == cudaSuccess) r = cudaEventRecord(marks[2 + s], st);
   }
   return r;

@@ -73,9 +73,9 @@ struct ListSliceEntry {
   int lo = 0, hi = 0, part = 0;
   int warps = 0;  // warps per CTA (all on one target group)
   cudaError_t (*prepare)() = nullptr;  // set the dynamic shared-memory limit
-  // grid (G target groups, C list segments); partial: C blocks [NB][n]
-  cudaError_t (*launch)(const float* rec, int n, int G, const int2* ent, const int* cnt, int C,
-                        double* partial, unsigned long long* counts, int* err,
+  // T CTAs, one share each (near_cut_kernel's pre and start); partial: blocks [NB][n]
+  cudaError_t (*launch)(const float* rec, int n, int G, const int2* ent, const int* cnt, int T,
+                        const unsigned long long* pre, const int* start, double* partial, unsigned long long* counts, int* err,
                         cudaStream_t st) = nullptr;
   cudaError_t (*occupancy)(int* blocks_per_sm) = nullptr;
 };
@@ -85,7 +85,7 @@ struct ListFarEntry {
   // in mcnt (0: none); frad: widest target group whose far field far() and
   // far_tree() leave to loc_far() (0: none)
   cudaError_t (*build)(const float* rec, int n, int G, const float* gdata, float rmax, int2* ent,
-                       int* cnt, int* mcnt, cudaStream_t st) = nullptr;
+                       int* cnt, int* mcnt, int* nsrc, cudaStream_t st) = nullptr;
   // grid (target groups / 4, S source ranges); fpart: S blocks [n_edge][n]
   cudaError_t (*far)(const float* rec, int n, int G, const float* gdata, int S, float frad,
                      double* fpart, unsigned long long* counts, cudaStream_t st) = nullptr;
@@ -136,7 +136,10 @@ struct ListArgs {
   const float* gdata = nullptr;
   int2* ent = nullptr;       // G x G entries (G = groups of kGroup records)
   int* cnt = nullptr;        // G near counts, then G local counts
-  int segments = 1;          // list segments of the near kernels
+  int shares = 1;            // CTAs of a near kernel
+  int segments = 2;          // most shares a group may fall into (>= 2)
+  int* cut = nullptr;        // G near sources, G shares of the group, `shares` first groups
+  unsigned long long* pre = nullptr;  // G + 2 (near_cut_kernel)
   double* partial = nullptr; // segments (+ 1 with local expansions) blocks [NB][n]
   int far_ranges = 1;        // source ranges of the flat far kernel
   double* fpart = nullptr;   // far blocks [n_edge][n]

@@ -348,7 +348,10 @@ __device__ __forceinline__ void finish_block(const FinishArgs& A, int j0, int rb
     const int tt = idx % TG, b = idx / TG, j = j0 + tt;
     double v = 0.0;
     if (j < A.n && A.partial) {
-      v = block_sum(A.partial + (size_t)b * A.n + j, A.nchunks, (size_t)NB * A.n);
+      const double* pb = A.partial + (size_t)b * A.n + j;
+      const size_t bs = (size_t)NB * A.n;
+      v = block_sum(pb, A.gshares ? A.gshares[j / kGroup] : A.nchunks, bs);
+      if (A.local_block >= 0) v += pb[A.local_block * bs];
       // far field of the list form: edge columns only
       if (A.fpart &&
           !(A.rmax > 0.f && A.gdata[(size_t)(j / kGroup) * A.gdata_len + 6] <= A.rmax)) {

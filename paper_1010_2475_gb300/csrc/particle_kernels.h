@@ -15,6 +15,8 @@ struct FinishArgs {
   int nchunks = 0;                  // number of pair partials (0: single particle)
   const double* partial = nullptr;  // [nchunks][NB][n] by sorted position
   const double* fpart = nullptr;    // far-field blocks [nfar][n_edge][n] (list form; nullable):
+  const int* gshares = nullptr;     // list form: near blocks of each group (null: nchunks of all)
+  int local_block = -1;             // block of the local fields (-1: none)
   int nfar = 0, n_edge = 0;         // edge column e = 2 (|beta| - 1) + beta1, beta1 <= 1
   const float* gdata = nullptr;     // with rmax > 0: group records of gdata_len floats; groups of
   int gdata_len = 0;                // radius <= rmax have no far blocks (local expansions)

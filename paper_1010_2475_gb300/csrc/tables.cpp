@@ -78,9 +78,10 @@ void lay_out(FinishTables& t, const std::vector<std::vector<Group>>& rows) {
       t.offs.push_back((int)t.tab.size());
       for (size_t q = 0; q < gs.size() && gs[q]->e.size() > j; ++q) t.tab.push_back(gs[q]->e[j]);
     }
-    for (int k = rb.k0; k < rb.k1; ++k) {
-      for (size_t q = 0; q < gs.size(); ++q)
-        if (gs[q]->k == k) t.rows.push_back({(int)q, gs[q]->l});
+    std::vector<std::vector<RowGroup>> of_row(rb.k1 - rb.k0);
+    for (size_t q = 0; q < gs.size(); ++q) of_row[gs[q]->k - rb.k0].push_back({(int)q, gs[q]->l});
+    for (const auto& r : of_row) {
+      t.rows.insert(t.rows.end(), r.begin(), r.end());
       t.rows_off.push_back((int)t.rows.size());
     }
     t.blocks.push_back(rb);

@@ -71,6 +71,34 @@ def test_group_expansions(mm, order, n, monkeypatch):
         assert any(not np.array_equal(res[nd, "0"][i], res[nd, "1"][i]) for i in range(2))
 
 
+@pytest.mark.parametrize("order,shape,per", [(2, "even", 1), (2, "even", 16), (4, "even", 3),
+                                             (6, "uneven", 1), (6, "uneven", 16), (3, "tiny", 16),
+                                             (8, "uneven", 4)])
+def test_near_shares(mm, order, shape, per, monkeypatch):
+    """Near pairs in equal shares: groups cut anywhere, a share of many groups,
+    one group in as many shares as it may fall into, more CTAs than shares."""
+    n = {"even": 1203, "uneven": 1501, "tiny": 33}[shape]
+    wl = mmvm_inputs.random_disk(n=n, order=order, radius=6.0, sigma=0.5, seed=80 + order)
+    if shape == "uneven":  # long lists in one corner, short ones elsewhere
+        wl.x[:500] = wl.x[:500] * 0.3
+        wl.x[500:] = wl.x[500:] * 12.0
+    nd, nl = mm.pair_variant_counts(order)
+    rows = np.array(sorted({0, n - 1, *range(1, n, max(1, n // 12))}))
+    ox, oM = rhs_regrouped(wl.x, wl.moments, 0.0, order, wl.lam0, wl.nu, rows=rows)
+    sx, sM = abs_scale_rows(wl.x, wl.moments, 0.0, order, wl.lam0, wl.nu, rows)
+    tol = 5e-6 * max(1.0, order / 6.0)
+    monkeypatch.setenv("MMVM_LIST_SEGMENTS", str(per))
+    for v in range(nd, nd + nl):
+        monkeypatch.setenv("MMVM_PAIR_VARIANT", str(v))
+        with mm.Context(order, wl.lam0, wl.nu, mm.MMVM_MIXED_FP32) as ctx:
+            ctx.set_state(wl.x, wl.moments, 0.0)
+            gx, gM = ctx.rhs()
+            near, far_pp, n_m2p, m2p_pairs = mm.mmvm_pair_work(ctx.handle)
+        assert near + far_pp + m2p_pairs == n * n
+        assert vel_error_cond(gx[rows], ox, sx) <= tol
+        assert rhs_error_cond(gM[rows], oM, sM, order, wl.lam0) <= tol
+
+
 # groups of radius 0.6 to 1.2 core sizes, where the remainder of the Gaussian
 # part's Taylor series sets the least separation
 @pytest.mark.parametrize("order,kind,n", [(4, "patches", 20000), (5, "patches", 20000),
