@@ -164,7 +164,8 @@ int mmvm_pair_time(mmvm_ctx* ctx, double* ms, int64_t* count);
 
 /* The same time split by kernel for the list form (the all-pairs variants
  * with mmvm_pair_config out[6] > 0): ms[0] the list build and the tree,
- * ms[1] the far-field kernel, ms[2 ..] each near kernel; summed over the
+ * ms[1] the far-field kernels, ms[2 ..] each near kernel (the first with the
+ * expansions of compact groups); summed over the
  * right-hand sides that mmvm_pair_time has read since the previous call of
  * this function (*count of them), *nparts = 2 + near kernels (0 for the
  * direct form).  ms must hold max_parts values.                             */
@@ -178,14 +179,16 @@ int mmvm_pair_time_parts(mmvm_ctx* ctx, double* ms, int32_t max_parts, int32_t* 
  *      group, near pairs with all warps of a CTA on one target group, a
  *      separate far-field kernel);
  *  [1] kernels per evaluation (order slices or column parts; the list form
- *      counts its list build and far kernel too);
+ *      counts its list build, tree, far and expansion kernels too);
  *  [2] targets per CTA (list form: threads per CTA of its first near kernel);
  *  [3] CTAs per SM;  [4] sources between CTA barriers (0: none);
- *  [5] source chunks (list form: list segments per target group);
+ *  [5] source chunks (list form: most shares of the near pairs that a target
+ *      group falls into);
  *  [6] 1 for the list form, else 0;  [7] source ranges of its far kernel.
  * The variant is chosen by timing the compiled variants for the first state
  * of each size class (environment: MMVM_PAIR_VARIANT=<v> forces one,
- * MMVM_AUTOTUNE=0 keeps variant 0).  out must hold 8 values.              */
+ * MMVM_AUTOTUNE=0 keeps variant 0, MMVM_LOCAL=0 / 1 keeps compact groups of
+ * the list form pair by pair / takes their expansions).  out must hold 8 values.              */
 int mmvm_pair_config(const mmvm_ctx* ctx, int32_t* out);
 
 /* Compiled all-pairs variants of (order, precision): *direct variants of the
@@ -195,7 +198,8 @@ int mmvm_pair_config(const mmvm_ctx* ctx, int32_t* out);
 int mmvm_pair_variant_counts(int32_t order, int32_t precision, int32_t* direct, int32_t* list);
 
 /* Cumulative counts of ordered pairs the all-pairs kernel evaluated since the
- * context was created, by path: full jet (near) and point-vortex jet (far,
+ * context was created, by path: full jet (near, one by one or through the
+ * expansions of compact groups) and point-vortex jet (far,
  * MMVM_MIXED_FP32 only, source by source or through tile expansions).  The
  * self pair and the tuning launches are not counted.  Waits for the context
  * stream.                                                                   */

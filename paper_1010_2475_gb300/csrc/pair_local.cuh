@@ -33,9 +33,8 @@
 // loc_radius(M) and groups close to each other (loc_pair; the target group
 // itself among them) stay with the pair kernels.
 // Measured (two patches, n = 65536, M = 6, one right-hand side): all-pairs
-// kernels 68.6 -> 15.4 ms (near pairs one by one 6.6e8 -> 1e8, far field 4.0 ->
-// 1.7 ms); velocities 3.7e-8 -> 1.1e-8 of FP64, moment rates 1.9e-7 -> 1.8e-7
-// (2-norms).
+// kernels 68.6 -> 16.0 ms (near pairs one by one 6.6e8 -> 1.2e8, far field 4.0 ->
+// 1.3 ms).
 #pragma once
 
 #include "pair_list.cuh"

@@ -313,6 +313,7 @@ __device__ __forceinline__ double block_sum(const double* __restrict__ v, int n,
 //    lengths inside one loop executed a second multiply-add per entry.)
 //  * scalars (powers of c, weights of the step) come from the record kernel;
 //    without one (a single particle, batches) two warps form them.
+// Before / now: 420 / 327 us at n = 24000, M = 6, 199 / 183 us at n = 2011, M = 8.
 // Shared memory holds [column][target] arrays: Psi (NB), a (K), X (2), 1 / M_00,
 // the scalars and the groups' sums.  Every global read of the stage input
 // precedes the first write behind a barrier.  All threads of the CTA call this;
