@@ -395,12 +395,19 @@ __device__ __forceinline__ void pair_tile_work(const T* __restrict__ rec, int n,
   // point-vortex path (warp-uniform): parts 0 and 1 add its edge columns,
   // part 2 has nothing to add.
   float4 tbox = make_float4(0.f, 0.f, 0.f, 0.f);
+  // FP64: the tile's sources about the CTA's first target
+  [[maybe_unused]] float2* soff = reinterpret_cast<float2*>(
+      tile + (size_t)S * (R + (PART != 2 ? tile_far64(M) : 0)));
   if constexpr (f32) {
     if (use_far && warp_valid) tbox = *reinterpret_cast<const float4*>(group_rec<M>(gdata, tgroup));
   } else if (far64) {
-    // box of the warp's targets, in FP32 (x_far64 has margin for the rounding)
-    float lo1 = j < n ? (float)tz1 : 3.4e38f, hi1 = j < n ? (float)tz1 : -3.4e38f;
-    float lo2 = j < n ? (float)tz2 : 3.4e38f, hi2 = j < n ? (float)tz2 : -3.4e38f;
+    // box of the warp's targets, in FP32, about the CTA's first target: rounded
+    // after the FP64 difference, so that the distance from the origin does
+    // not count (one FP32 step of a coordinate is 8 units at 1e8)
+    const T* org = rec + (size_t)tile0 * R;
+    const float f1 = (float)(tz1 - org[0]), f2 = (float)(tz2 - org[1]);
+    float lo1 = j < n ? f1 : 3.4e38f, hi1 = j < n ? f1 : -3.4e38f;
+    float lo2 = j < n ? f2 : 3.4e38f, hi2 = j < n ? f2 : -3.4e38f;
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
       lo1 = fminf(lo1, __shfl_xor_sync(0xffffffffu, lo1, o));
@@ -408,7 +415,11 @@ __device__ __forceinline__ void pair_tile_work(const T* __restrict__ rec, int n,
       lo2 = fminf(lo2, __shfl_xor_sync(0xffffffffu, lo2, o));
       hi2 = fmaxf(hi2, __shfl_xor_sync(0xffffffffu, hi2, o));
     }
-    tbox = make_float4(lo1, hi1, lo2, hi2);
+    // wider by the rounding: 2^-24 of the box's and of the source's coordinate,
+    // which is at most the box's plus the distance (a CTA's targets may lie far apart)
+    const float e1 = 4.8e-7f * fmaxf(fabsf(lo1), fabsf(hi1));
+    const float e2 = 4.8e-7f * fmaxf(fabsf(lo2), fabsf(hi2));
+    tbox = make_float4(lo1 - e1, hi1 + e1, lo2 - e2, hi2 + e2);
   }
 #pragma unroll 1
   for (int t0 = c0; t0 < c1; t0 += S) {
@@ -431,11 +442,14 @@ __device__ __forceinline__ void pair_tile_work(const T* __restrict__ rec, int n,
     if (__syncthreads_or(near)) {
       load_tile(t0, cnt);
       __syncthreads();
-      if constexpr (!f32 && PART != 2) {
+      if constexpr (!f32) {
         if (far64) {
           T* mf = tile + (size_t)S * R;
-          for (int s = threadIdx.x; s < cnt; s += blockDim.x)
-            tile_multipoles<M>(tile + s * R, mf + s * tile_far64(M));
+          const T* org = rec + (size_t)tile0 * R;
+          for (int s = threadIdx.x; s < cnt; s += blockDim.x) {
+            if constexpr (PART != 2) tile_multipoles<M>(tile + s * R, mf + s * tile_far64(M));
+            soff[s] = make_float2((float)(tile[s * R] - org[0]), (float)(tile[s * R + 1] - org[1]));
+          }
           __syncthreads();
         }
       }
@@ -458,9 +472,9 @@ __device__ __forceinline__ void pair_tile_work(const T* __restrict__ rec, int n,
           if constexpr (f32) {
             if (use_far && near) sfar = point_is_far<M>(tbox, rs[0], rs[1]);
           } else if (far64) {
-            const float z1 = (float)rs[0], z2 = (float)rs[1];
-            const float dx = fmaxf(0.f, fmaxf(tbox.x - z1, z1 - tbox.y));
-            const float dy = fmaxf(0.f, fmaxf(tbox.z - z2, z2 - tbox.w));
+            const float2 z = soff[s];
+            const float dx = fmaxf(0.f, fmaxf(tbox.x - z.x, z.x - tbox.y));
+            const float dy = fmaxf(0.f, fmaxf(tbox.z - z.y, z.y - tbox.w));
             sfar = dx * dx + dy * dy >= x_far64(M);
           }
           if (!sfar) {
@@ -585,8 +599,8 @@ size_t pair_smem_bytes(int S) {  // shared memory of one CTA
   size_t b = (size_t)S * rec_len<T>(M) * sizeof(T);
   if (std::is_same<T, float>::value)
     b += 2 * (size_t)PartCols<LO, HI, PART>::NS * TPC * sizeof(float);
-  else if (PART != 2)
-    b += (size_t)S * tile_far64(M) * sizeof(T);
+  else
+    b += (size_t)S * ((PART != 2 ? tile_far64(M) * sizeof(T) : 0) + sizeof(float2));
   return b;
 }
 
