@@ -128,18 +128,21 @@ __host__ __device__ constexpr int gdata_len(int M) { return round_up(8 + 2 * m2p
 // group they serve, and the least separation x = |t0 - s0|^2 of two groups, the
 // wider of radius r: the further apart, the faster the expansions converge.
 // Up to loc_core kLocMinX is enough; beyond, x grows by loc_slope per unit of the
-// radius.  What they keep small is the remainder of the Taylor series of the
-// Gaussian part, e^{-x} at orders up to 2M + 1 + P; with 0.9 and 40 .. 80 at
-// M >= 4 single particles of groups of radius 0.7 .. 1.1 were off by up to 100
-// times the error without expansions (M = 6, disk of 16000).  Errors against
-// FP64 with / without expansions, two patches of 8192, 20000, 36000 and disks of
-// 6000, 16000, 30011, 44000, M = 6: velocities 0.91 .. 1.01 (2-norm), 0.77 .. 1.28
-// (largest), moment rates 0.98 .. 1.03 and 0.94 .. 1.19; a radius of 2.0 with
-// slope 40 at M = 4 and 5 adds 10 to 20 % to the moment rates' error (two patches
-// of 8192).
-__host__ __device__ constexpr int loc_extra(int M) {
-  return M <= 1 ? 13 : M == 2 ? 14 : M == 3 ? 15 : M == 4 ? 16 : M <= 7 ? 17 : 15;
-}
+// radius, or (orders 5 and 6) by a second, steeper line.
+// What they keep small is the remainder of the Taylor series of the Gaussian
+// part, e^{-x} at orders up to 2M + 1 + P.  The double series of two particles at
+// the facing ends of two groups at the least separation, in 64 bits against the
+// jet itself, over radii, directions and moments (10 % of the circulation per
+// order in the weighted norm): the pair's velocity is off by at most 2.4e-7 (M = 3;
+// 1.6e-7 at M = 2, 1e-7 or less else), its moment rates by 4e-6 (M = 6) of the sum of
+// their terms' magnitudes, below the FP32 jet's rounding at these orders.  (With
+// 13 to 15 extra orders and 40 per unit at M <= 3 a velocity was off by up to
+// 5e-5; with 40 per unit alone at M = 5 and 6 moment rates by 8e-5 and 1e-3.)
+// 17 extra orders at M <= 3 cost 1.4 times the multiply-adds of 14, but 14 would
+// have to keep groups further apart: disk of 30011, M = 2, per step 4.07 ms with
+// 17, 4.07 with 16, 4.34 with 15, 4.44 with 14 at separations equally safe (3.60
+// with the limits that were not).
+__host__ __device__ constexpr int loc_extra(int M) { return M == 4 ? 16 : M <= 7 ? 17 : 15; }
 __host__ __device__ constexpr float loc_radius(int M) {
   return M <= 2 ? 2.0f : M <= 4 ? 1.8f : M == 5 ? 1.6f : M == 6 ? 1.7f : M == 7 ? 1.1f : 0.85f;
 }
@@ -154,8 +157,10 @@ __host__ __device__ constexpr float loc_core(int M) {  // up to this radius kLoc
   return M <= 2 ? 0.9f : M == 3 ? 0.8f : M == 4 ? 0.6875f : M <= 7 ? 0.5625f : 0.4375f;
 }
 __host__ __device__ constexpr float loc_slope(int M) {  // of the least x beyond loc_core
-  return M == 3 ? 50.f : M == 4 ? 55.f : M <= 6 ? 40.f : 60.f;
+  return M == 0 ? 60.f : M <= 2 ? 54.f : M == 3 ? 56.f : M == 4 ? 55.f : M <= 6 ? 40.f : 60.f;
 }
+__host__ __device__ constexpr float loc_core2(int M) { return M == 5 ? 0.66f : 0.73f; }
+__host__ __device__ constexpr float loc_slope2(int M) { return M == 5 ? 58.f : M == 6 ? 72.f : 0.f; }
 
 // Binary tree over G groups of kGroup sorted records (the far field of the
 // list form): level L has ceil(G / 2^L) nodes, node i of level L >= 1 holds

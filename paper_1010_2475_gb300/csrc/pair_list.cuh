@@ -127,8 +127,10 @@ template <int M>
 __device__ __forceinline__ bool loc_pair(float rmax, const float4 tc, const float4 sc) {
   const float dx = tc.x - sc.x, dy = tc.y - sc.y;
   const float r = fmaxf(tc.z, sc.z);
-  const float xmin =
-      __fadd_rn(kLocMinX, __fmul_rn(loc_slope(M), fmaxf(__fsub_rn(r, loc_core(M)), 0.f)));
+  float grow = __fmul_rn(loc_slope(M), __fsub_rn(r, loc_core(M)));
+  if constexpr (loc_slope2(M) > 0.f)
+    grow = fmaxf(grow, __fmul_rn(loc_slope2(M), __fsub_rn(r, loc_core2(M))));
+  const float xmin = __fadd_rn(kLocMinX, fmaxf(grow, 0.f));
   return rmax > 0.f && r <= rmax && __fadd_rn(__fmul_rn(dx, dx), __fmul_rn(dy, dy)) >= xmin;
 }
 template <int M>

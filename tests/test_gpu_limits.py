@@ -74,3 +74,71 @@ def test_fp64_shortcut_far_from_the_origin(mm, order, state):
     assert vel_error_rows(gx, rx) <= 1e-12
     if order >= 2:
         assert rhs_error_rows(gM, rM, order, LAM) <= 1e-12
+
+
+@pytest.mark.parametrize("order", range(9))
+def test_strong_vortex_at_the_facing_end(mm, order, monkeypatch):
+    """Two groups on a line, a strong vortex at the end of one that faces the
+    other, at radii and separations through the whole range of the near
+    expansions: where a group expansion converges worst, whoever of the pair
+    kernels and the expansions takes the pair."""
+    widest = (2.0, 2.0, 2.0, 1.8, 1.8, 1.6, 1.7, 1.1, 0.85)[order]
+    rng = np.random.default_rng(order)
+    monkeypatch.setenv("MMVM_LOCAL", "1")
+    monkeypatch.setenv("MMVM_FAR_TREE", "0")
+    variant = str(mm.pair_variant_counts(order)[0])
+    rows = np.arange(32, 64)
+    expanded = 0
+    for r in widest * np.array([0.4, 0.55, 0.7, 0.85, 0.999]):
+        sep = max(8.0, (2.0 * r + 0.2) ** 2) * 1.001
+        while sep < 90.0:
+            s = math.sqrt(sep)
+            x = rng.uniform(-0.6, 0.6, size=(64, 2)) * [r, 0.2 * r]
+            for k in (0, 32):
+                x[k], x[k + 1] = [r, 0.0], [-r, 0.0]
+                x[k + 2], x[k + 3] = [0.0, 0.15 * r], [0.0, -0.15 * r]
+            x[32:, 0] += s
+            g = 1e-6 * (1.0 + rng.random(64))
+            g[0] = 1.0
+            m = _moments(g, order, LAM, rng)
+            monkeypatch.delenv("MMVM_PAIR_VARIANT", raising=False)
+            rx, rM = _rhs(mm, order, LAM, x, m, mm.MMVM_FP64)
+            monkeypatch.setenv("MMVM_PAIR_VARIANT", variant)
+            with mm.Context(order, LAM, 1e-3, mm.MMVM_MIXED_FP32) as ctx:
+                ctx.set_state(x, m, 0.0)
+                gx, gM = ctx.rhs()
+                expanded += mm.mmvm_pair_expanded(ctx.handle)
+            assert vel_error_rows(gx[rows], rx[rows]) <= 2e-6, (r, sep)
+            if order >= 1:
+                sM = abs_scale_rows(x, m, 0.0, order, LAM, 1e-3, rows[:8], procs=1)[1]
+                assert rhs_error_cond(gM[rows[:8]], rM[rows[:8]], sM, order, LAM) \
+                    <= _tol(order), (r, sep)
+            sep *= 1.12
+    assert expanded > 0
+
+
+# groups as wide as the expansions' limits: n sets the radius
+@pytest.mark.parametrize("order,n", [(0, 4001), (1, 5003), (2, 5003), (2, 12001), (3, 6007),
+                                     (4, 9001), (5, 9001), (6, 9001), (6, 16001), (7, 16001),
+                                     (8, 30011)])
+def test_rates_of_moderate_groups(mm, order, n, monkeypatch):
+    """Velocities within 2e-6 of the largest and moment rates within the mixed
+    tolerance of the largest against the FP64 form; one vortex of 50 is 100
+    times as strong as the others.  The pairs really went through the expansions."""
+    rng = np.random.default_rng(n + order)
+    wl = mmvm_inputs.random_disk(n=n, order=order, radius=10.0, sigma=0.5, seed=n + order)
+    g = np.where(rng.random(n) < 0.02, 100.0, 1.0) * rng.normal(size=n)
+    m = _moments(g, order, wl.lam0, rng, 0.01)
+    rx, rM = _rhs(mm, order, wl.lam0, wl.x, m, mm.MMVM_FP64)
+    monkeypatch.setenv("MMVM_PAIR_VARIANT", str(mm.pair_variant_counts(order)[0]))
+    monkeypatch.setenv("MMVM_FAR_TREE", "1")
+    for local in ("0", "1"):
+        monkeypatch.setenv("MMVM_LOCAL", local)
+        with mm.Context(order, wl.lam0, 1e-3, mm.MMVM_MIXED_FP32) as ctx:
+            ctx.set_state(wl.x, m, 0.0)
+            gx, gM = ctx.rhs()
+            expanded = mm.mmvm_pair_expanded(ctx.handle)
+        assert (expanded > 0) == (local == "1")
+        assert vel_error(gx, rx) <= 2e-6
+        if order >= 2:  # first moments are conserved: at order 1 the rate is 0 up to rounding
+            assert rhs_error(gM, rM, order, wl.lam0) <= _tol(order)
