@@ -144,14 +144,17 @@ __host__ __device__ constexpr int gdata_len(int M) { return round_up(8 + 2 * m2p
 // with the limits that were not).
 __host__ __device__ constexpr int loc_extra(int M) { return M == 4 ? 16 : M <= 7 ? 17 : 15; }
 __host__ __device__ constexpr float loc_radius(int M) {
-  return M <= 2 ? 2.0f : M <= 4 ? 1.8f : M == 5 ? 1.6f : M == 6 ? 1.7f : M == 7 ? 1.1f : 0.85f;
+  return M == 0 ? 1.75f : M <= 2 ? 2.0f : M <= 4 ? 1.8f : M == 5 ? 1.6f : M == 6 ? 1.7f : M == 7 ? 1.1f : 0.85f;
 }
-// Widest target group whose far field is taken through its local field: at
-// most 0.3 of the distance to anything beyond x_far(M), so that the Taylor
-// series about its centre loses less than FP32 rounding.
+// Widest target group whose far field is taken through its local field.  A box
+// may have no width (particles on a line), and then a far source beside it is only
+// sqrt(x_far) from the centre: the limits are 0.34 to 0.39 of that, where the Taylor
+// series about the centre, to loc_extra orders per axis, ends within FP32 rounding:
+// velocities 1e-7 or less, moment rates 1.4e-6 or less of their terms' magnitudes (64 bits,
+// over directions and moments; 0.40 to 0.45 at M <= 3 left up to 1.3e-5).
 __host__ __device__ constexpr float loc_field_radius(int M) {
-  return M <= 0 ? 2.0f : M == 1 ? 2.3f : M == 2 ? 2.5f : M == 3 ? 2.8f : M == 4 ? 3.0f
-       : M == 5 ? 3.2f : M == 6 ? 3.4f : M == 7 ? 3.4f : 3.2f;
+  return M <= 0 ? 1.75f : M == 1 ? 2.2f : M == 2 ? 2.45f : M <= 4 ? 2.75f : M == 5 ? 3.2f
+       : M == 6 ? 3.3f : M == 7 ? 3.4f : 3.2f;
 }
 __host__ __device__ constexpr float loc_core(int M) {  // up to this radius kLocMinX is enough
   return M <= 2 ? 0.9f : M == 3 ? 0.8f : M == 4 ? 0.6875f : M <= 7 ? 0.5625f : 0.4375f;

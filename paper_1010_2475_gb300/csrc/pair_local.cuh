@@ -52,6 +52,7 @@ struct Loc {
   static constexpr int NT = Q + NL;           // highest derivative order
   static constexpr int ROWS = 32 + Q + 2;     // table rows (lane + k, k <= Q + 1)
   static_assert(NL <= 31, "one lane per order of the field");
+  static_assert(loc_radius(M) <= loc_field_radius(M), "a near field needs its far field's evaluation");
   // Expansion record of a group: rows k1 of A, rows k1 of S (k2 contiguous,
   // rows padded to 4 floats), then the degree 0 and 1 parts of P_e.
   __host__ __device__ static constexpr int row_len(int top, int k1) { return (top - k1 + 1 + 3) / 4 * 4; }
@@ -557,9 +558,9 @@ __global__ void __launch_bounds__(kLocWarps * 32, 2)
 // multiply-adds per lane instead of 2902 flops per target, a far source 4 (M +
 // 1) instead of 838 flops per target.  The lanes first form the point-vortex
 // edge derivatives of up to 32 nodes or sources (one each), then run through
-// them with one order of the field per lane.  A target group of radius
-// loc_radius sees everything here from sqrt(x_far) away or more, so the field's
-// Taylor series loses less than FP32 rounding.
+// them with one order of the field per lane.  For a target group of radius
+// loc_field_radius or less the field's Taylor series loses less than FP32
+// rounding (common.cuh).
 //
 // A node is taken at a radius of up to 0.2 of the distance, twice that of the
 // target-by-target kernels, which hold every order q <= 3M of the jet to 2e-9:

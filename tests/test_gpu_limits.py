@@ -142,3 +142,33 @@ def test_rates_of_moderate_groups(mm, order, n, monkeypatch):
         assert vel_error(gx, rx) <= 2e-6
         if order >= 2:  # first moments are conserved: at order 1 the rate is 0 up to rounding
             assert rhs_error(gM, rM, order, wl.lam0) <= _tol(order)
+
+
+@pytest.mark.parametrize("order", range(9))
+@pytest.mark.parametrize("frac", [0.7, 0.85, 0.99, 1.05])
+def test_far_field_of_line_groups(mm, order, frac, monkeypatch):
+    """A target group on a line (half length up to the widest that may take a
+    local field) and one strong vortex just beyond the far threshold beside it: the
+    group's box has no width, so the source is as close to its centre as the
+    threshold.  Velocities to 5e-7: a truncation at FP32 rounding (1e-7) and
+    the rounding of a far field."""
+    r = (2.0, 2.3, 2.5, 2.8, 3.0, 3.2, 3.4, 3.4, 3.2)[order] * frac
+    D = math.sqrt(X_FAR[order]) * 1.002
+    rng = np.random.default_rng(10 * order + int(10 * frac))
+    x = np.zeros((64, 2))
+    x[:32, 1] = np.linspace(-r, r, 32)
+    x[32:] = rng.uniform(0.0, 0.02, size=(32, 2)) + [D, -0.01]
+    g = 1e-6 * (1.0 + rng.random(64))
+    g[32] = 1.0
+    m = _moments(g, order, LAM, rng)
+    monkeypatch.setenv("MMVM_PAIR_VARIANT", str(mm.pair_variant_counts(order)[0]))
+    monkeypatch.setenv("MMVM_LOCAL", "1")
+    rows = np.arange(32)
+    rx, rM = _rhs(mm, order, LAM, x, m, mm.MMVM_FP64)
+    sM = abs_scale_rows(x, m, 0.0, order, LAM, 1e-3, rows, procs=1)[1] if order else None
+    for tree in ("0", "1"):
+        monkeypatch.setenv("MMVM_FAR_TREE", tree)
+        gx, gM = _rhs(mm, order, LAM, x, m, mm.MMVM_MIXED_FP32)
+        assert vel_error_rows(gx[rows], rx[rows]) <= 5e-7
+        if order >= 1:
+            assert rhs_error_cond(gM[rows], rM[rows], sM, order, LAM) <= _tol(order)
