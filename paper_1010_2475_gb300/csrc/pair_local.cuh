@@ -562,16 +562,19 @@ __global__ void __launch_bounds__(kLocWarps * 32, 2)
 // loc_field_radius or less the field's Taylor series loses less than FP32
 // rounding (common.cuh).
 //
-// A node is taken at a radius of up to 0.2 of the distance, twice that of the
-// target-by-target kernels, which hold every order q <= 3M of the jet to 2e-9:
-// here the truncation sum_{k>P} C(q+k-1, k) 0.2^k is 1e-9 or less for the
-// velocities (q = 1) and below FP32 rounding for the orders whose far field
-// counts beside the near field (by q = 6, 5 / r^6 of the near field's size).
-constexpr float kLocTheta2 = 0.04f;
+// A node is taken at a radius of up to 0.2 of the distance (0.15 at order 0, which
+// has the fewest terms), twice that of the target-by-target kernels, which hold
+// every order q <= 3M of the jet to 2e-9 of the node's own term of that order.
+// Here a velocity is off by at most 4e-8 (M = 0; 0.2 would leave 5e-7), 2.4e-8 (M =
+// 1), 1e-9 (M = 2) and less (M >= 3) of a source's at the near edge of its node, and
+// the moment rates by 2e-9 (M = 2) of their terms' magnitudes: the high orders, off by up
+// to 1e-5 of their own term, count that little at a distance of sqrt(x_far).
+template <int M>
 __device__ __forceinline__ bool loc_takes(const float4 tb, const float4 c) {
+  constexpr float theta2 = M == 0 ? 0.0225f : 0.04f;
   const float dx = fmaxf(0.f, fmaxf(tb.x - c.x, c.x - tb.y));
   const float dy = fmaxf(0.f, fmaxf(tb.z - c.y, c.y - tb.w));
-  return c.z * c.z <= kLocTheta2 * (dx * dx + dy * dy);
+  return c.z * c.z <= theta2 * (dx * dx + dy * dy);
 }
 
 template <int M>
@@ -702,7 +705,7 @@ __global__ void __launch_bounds__(kLocWarps * 32)
     const float4 box = *reinterpret_cast<const float4*>(nd);
     const float4 cen = *reinterpret_cast<const float4*>(nd + 4);
     const bool far_box = box_dist2(tb, box) >= x_far(M);
-    if (far_box && loc_takes(tb, cen)) {
+    if (far_box && loc_takes<M>(tb, cen)) {
       if (lane == 0) node_s[nq] = top;
       n_m2p += 1;
       n_m2p_pairs += Lv == 0 ? min(kGroup, n - kGroup * i) : (unsigned)cen.w;

@@ -172,3 +172,33 @@ def test_far_field_of_line_groups(mm, order, frac, monkeypatch):
         assert vel_error_rows(gx[rows], rx[rows]) <= 5e-7
         if order >= 1:
             assert rhs_error_cond(gM[rows], rM[rows], sM, order, LAM) <= _tol(order)
+
+
+@pytest.mark.parametrize("order", range(9))
+def test_far_nodes_of_local_fields(mm, order, monkeypatch):
+    """One strong vortex at the edge of its group that faces a compact target
+    group, at every distance from the far threshold on: the widest source
+    groups that are taken through their expansions.  Velocities to 5e-7 as above."""
+    rng = np.random.default_rng(order)
+    monkeypatch.setenv("MMVM_LOCAL", "1")
+    monkeypatch.setenv("MMVM_FAR_TREE", "0")
+    rows = np.arange(32)
+    for ratio in (0.1, 0.14, 0.17, 0.195, 0.21):  # radius / distance of the source group
+        for gap in (1.01, 1.5):
+            D = math.sqrt(X_FAR[order]) * gap
+            r = ratio / (1.0 - ratio) * (D + 0.2)
+            x = rng.uniform(-0.1, 0.1, size=(64, 2))
+            x[32:] = rng.uniform(-0.6, 0.6, size=(32, 2)) * r + [D + 0.1 + r, 0.0]
+            x[32], x[33] = [D + 0.1, 0.0], [D + 0.1 + 2.0 * r, 0.0]
+            x[34], x[35] = [D + 0.1 + r, 0.6 * r], [D + 0.1 + r, -0.6 * r]
+            g = 1e-6 * (1.0 + rng.random(64))
+            g[32] = 1.0
+            m = _moments(g, order, LAM, rng)
+            monkeypatch.delenv("MMVM_PAIR_VARIANT", raising=False)
+            rx, rM = _rhs(mm, order, LAM, x, m, mm.MMVM_FP64)
+            monkeypatch.setenv("MMVM_PAIR_VARIANT", str(mm.pair_variant_counts(order)[0]))
+            gx, gM = _rhs(mm, order, LAM, x, m, mm.MMVM_MIXED_FP32)
+            assert vel_error_rows(gx[rows], rx[rows]) <= 5e-7, (ratio, gap)
+            if order >= 1:
+                sM = abs_scale_rows(x, m, 0.0, order, LAM, 1e-3, rows, procs=1)[1]
+                assert rhs_error_cond(gM[rows], rM[rows], sM, order, LAM) <= _tol(order)
