@@ -118,6 +118,16 @@ __host__ __device__ constexpr int m2p_order(int M) {
 }
 __host__ __device__ constexpr int m2p_terms(int M) { return M + m2p_order(M) + 1; }
 constexpr float kM2PTheta2 = 0.01f;  // theta^2
+// Widest tile or node that is taken through its expansion: its terms reach R^j / j!
+// of a unit circulation, j < m2p_terms(M), and the shifts of the tree form that power
+// too.  The limit keeps them below 1e26, so that circulations up to 1e12 stay inside
+// the FP32 range; without it a term overflowed while its derivative underflowed, and
+// the far field was NaN (M = 6: groups 1e3 core units wide).  Wider ones are opened, or
+// summed source by source.
+__host__ __device__ constexpr float m2p_radius(int M) {
+  return M <= 0 ? 6700.f : M == 1 ? 1130.f : M == 2 ? 430.f : M == 3 ? 240.f : M == 4 ? 185.f
+       : M == 5 ? 135.f : M == 6 ? 118.f : M == 7 ? 104.f : 92.f;
+}
 // Per group of kGroup records (FP32 far field): (min z1, max z1, min z2,
 // max z2) of the hi parts, (centre z1, centre z2, radius, 0), then
 // Re/Im B_j for j < m2p_terms(M); padded to whole float4s.

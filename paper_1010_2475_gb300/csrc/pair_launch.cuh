@@ -222,7 +222,7 @@ __device__ __forceinline__ bool tile_takes_m2p(const float* __restrict__ gdata, 
   const float4 tb = *reinterpret_cast<const float4*>(group_rec<M>(gdata, tgroup));
   const float dx = fmaxf(0.f, fmaxf(tb.x - c.x, c.x - tb.y));
   const float dy = fmaxf(0.f, fmaxf(tb.z - c.y, c.y - tb.w));
-  return c.z * c.z <= kM2PTheta2 * (dx * dx + dy * dy);
+  return c.z <= m2p_radius(M) && c.z * c.z <= kM2PTheta2 * (dx * dx + dy * dy);
 }
 
 // The far group sg summed through its expansion about its centre for this

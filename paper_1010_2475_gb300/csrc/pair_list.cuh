@@ -98,10 +98,11 @@ __device__ __forceinline__ bool box_inside(const float4 tb, const float4 sb) {
   return dx * dx + dy * dy < x_far(M) * 0.999f;
 }
 // tile_takes_m2p for a target box tb and a source group's (centre, radius) c.
+template <int M>
 __device__ __forceinline__ bool takes_m2p(const float4 tb, const float4 c) {
   const float dx = fmaxf(0.f, fmaxf(tb.x - c.x, c.x - tb.y));
   const float dy = fmaxf(0.f, fmaxf(tb.z - c.y, c.y - tb.w));
-  return c.z * c.z <= kM2PTheta2 * (dx * dx + dy * dy);
+  return c.z <= m2p_radius(M) && c.z * c.z <= kM2PTheta2 * (dx * dx + dy * dy);
 }
 
 // ------------------------------------------------------------------ 1. near lists
@@ -521,7 +522,7 @@ __global__ void __launch_bounds__(kFarWarps * 32)
     const float4 sb = *reinterpret_cast<const float4*>(gd);
     const int nsrc = min(kGroup, n - g * kGroup);
     const bool far_tile = box_dist2(tb, sb) >= x_far(M);
-    if (far_tile && takes_m2p(tb, *reinterpret_cast<const float4*>(gd + 4))) {
+    if (far_tile && takes_m2p<M>(tb, *reinterpret_cast<const float4*>(gd + 4))) {
       // the tile through its expansion about its centre
       const float cx = gd[4], cy = gd[5];
       const float d1 = tz1 - cx, d2 = tz2 - cy;
@@ -766,7 +767,7 @@ __global__ void __launch_bounds__(kFarWarps * 32)
     const float4 box = *reinterpret_cast<const float4*>(nd);
     const float4 cen = *reinterpret_cast<const float4*>(nd + 4);
     const bool far_box = box_dist2(tb, box) >= x_far(M);
-    if (far_box && takes_m2p(tb, cen)) {
+    if (far_box && takes_m2p<M>(tb, cen)) {
       // the node (or group) through its expansion about its centre
       const float d1 = tz1 - cen.x, d2 = tz2 - cen.y;
       const float b1 = d1 + tl1, b2 = d2 + tl2;

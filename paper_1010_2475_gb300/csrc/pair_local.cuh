@@ -574,7 +574,7 @@ __device__ __forceinline__ bool loc_takes(const float4 tb, const float4 c) {
   constexpr float theta2 = M == 0 ? 0.0225f : 0.04f;
   const float dx = fmaxf(0.f, fmaxf(tb.x - c.x, c.x - tb.y));
   const float dy = fmaxf(0.f, fmaxf(tb.z - c.y, c.y - tb.w));
-  return c.z * c.z <= theta2 * (dx * dx + dy * dy);
+  return c.z <= m2p_radius(M) && c.z * c.z <= theta2 * (dx * dx + dy * dy);
 }
 
 template <int M>

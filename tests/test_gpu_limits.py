@@ -202,3 +202,31 @@ def test_far_nodes_of_local_fields(mm, order, monkeypatch):
             if order >= 1:
                 sM = abs_scale_rows(x, m, 0.0, order, LAM, 1e-3, rows, procs=1)[1]
                 assert rhs_error_cond(gM[rows], rM[rows], sM, order, LAM) <= _tol(order)
+
+
+@pytest.mark.parametrize("order", range(9))
+@pytest.mark.parametrize("sparse", [False, True])
+def test_domains_many_core_sizes_wide(mm, order, sparse, monkeypatch):
+    """Source groups and tree nodes whose expansions would leave the FP32 range:
+    64 clusters of 32, each 2e3 units wide, over 2e5 units, with (and without) tight
+    groups of targets among them."""
+    rng = np.random.default_rng(order)
+    n = 2048
+    c = 2e5 * rng.uniform(-1.0, 1.0, size=(64, 2))
+    w = np.where(np.arange(64) % 4 == 0, 2e3 if sparse else 0.5, 2e3)
+    x = np.repeat(c, 32, axis=0) + np.repeat(w, 32)[:, None] * rng.uniform(-0.5, 0.5, size=(n, 2))
+    m = _moments(rng.normal(size=n), order, LAM, rng)
+    rows = np.arange(0, n, 97)
+    ox, oM = rhs_regrouped(x, m, 0.0, order, LAM, 1e-3, rows=rows)
+    sx, sM = abs_scale_rows(x, m, 0.0, order, LAM, 1e-3, rows, procs=1)
+    nd, nl = mm.pair_variant_counts(order)
+    for v, tree, local in ((0, "0", "0"), (nd, "0", "0"), (nd, "1", "0"), (nd, "0", "1"),
+                           (nd + nl - 1, "1", "1")):
+        monkeypatch.setenv("MMVM_PAIR_VARIANT", str(v))
+        monkeypatch.setenv("MMVM_FAR_TREE", tree)
+        monkeypatch.setenv("MMVM_LOCAL", local)
+        gx, gM = _rhs(mm, order, LAM, x, m, mm.MMVM_MIXED_FP32)
+        assert np.isfinite(gx).all() and np.isfinite(gM).all(), (v, tree, local)
+        assert vel_error_cond(gx[rows], ox, sx) <= 2e-6, (v, tree, local)
+        if order >= 1:
+            assert rhs_error_cond(gM[rows], oM, sM, order, LAM) <= _tol(order), (v, tree, local)
