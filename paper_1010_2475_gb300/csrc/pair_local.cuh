@@ -234,7 +234,8 @@ __device__ __forceinline__ void loc_upward(float b1, float b2, float l1, float l
                                            float xl, float amp, float s, float* te, float* tf,
                                            Gf&& g, int stride, float xmax) {
   const float rh = 1.f / x;
-  const float rl = (fmaf(-x, rh, 1.f) - xl * rh) * rh;
+  // an x beyond the FP32 range leaves zeros (rh = 0), not inf x 0
+  const float rl = x <= 3.4e38f ? (fmaf(-x, rh, 1.f) - xl * rh) * rh : 0.f;
   const Two r{rh, rl};
   Two v1 = two_mul({b1, l1}, r), v2 = two_mul({b2, l2}, r);
   v1 = {v1.h * s, v1.l * s};

@@ -230,3 +230,26 @@ def test_domains_many_core_sizes_wide(mm, order, sparse, monkeypatch):
         assert vel_error_cond(gx[rows], ox, sx) <= 2e-6, (v, tree, local)
         if order >= 1:
             assert rhs_error_cond(gM[rows], oM, sM, order, LAM) <= _tol(order), (v, tree, local)
+
+
+@pytest.mark.parametrize("order", [0, 2, 6])
+def test_clusters_beyond_the_range_of_squared_distances(mm, order, monkeypatch):
+    """Two clusters 1e20 units apart do not see each other."""
+    rng = np.random.default_rng(order)
+    n = 192
+    x = rng.uniform(-1.0, 1.0, size=(n, 2))
+    m = _moments(rng.normal(size=n), order, LAM, rng)
+    nd, nl = mm.pair_variant_counts(order)
+    for v, tree, local in ((0, "0", "0"), (nd, "0", "0"), (nd, "1", "0"), (nd, "0", "1"),
+                           (nd, "1", "1")):
+        monkeypatch.setenv("MMVM_PAIR_VARIANT", str(v))
+        monkeypatch.setenv("MMVM_FAR_TREE", tree)
+        monkeypatch.setenv("MMVM_LOCAL", local)
+        far = x.copy()
+        far[96:] += [1e20, 0.0]
+        gx, gM = _rhs(mm, order, LAM, far, m, mm.MMVM_MIXED_FP32)
+        ox, oM = rhs_regrouped(x[:96], m[:96], 0.0, order, LAM, 1e-3)
+        sx, sM = abs_scale_rows(x[:96], m[:96], 0.0, order, LAM, 1e-3, np.arange(96), procs=1)
+        assert vel_error_cond(gx[:96], ox, sx) <= 2e-6, (v, tree, local)
+        if order >= 1:
+            assert rhs_error_cond(gM[:96], oM, sM, order, LAM) <= _tol(order), (v, tree, local)
