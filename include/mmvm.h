@@ -186,9 +186,14 @@ int mmvm_pair_time_parts(mmvm_ctx* ctx, double* ms, int32_t max_parts, int32_t* 
  *      group falls into);
  *  [6] 1 for the list form, else 0;  [7] source ranges of its far kernel.
  * The variant is chosen by timing the compiled variants for the first state
- * of each size class (environment: MMVM_PAIR_VARIANT=<v> forces one,
- * MMVM_AUTOTUNE=0 keeps variant 0, MMVM_LOCAL=0 / 1 keeps compact groups of
- * the list form pair by pair / takes their expansions).  out must hold 8 values.              */
+ * of each size class (log2 n) and density class (the radius in core units of 32
+ * particles spread over the bounding box, in powers of two) in the process.
+ * Variants agree within the rounding of the mixed form, not bit by bit: two runs
+ * whose timings differ may differ that much.  Environment: MMVM_PAIR_VARIANT=<v>
+ * forces one, MMVM_AUTOTUNE=0 keeps variant 0, MMVM_FAR_TREE=0 / 1 the flat or the tree
+ * far field, MMVM_LOCAL=0 / 1 compact groups of the list form pair by pair or through
+ * expansions, MMVM_LIST_SEGMENTS=<k> k shares of the near pairs per CTA slot.
+ * out must hold 8 values.                                                   */
 int mmvm_pair_config(const mmvm_ctx* ctx, int32_t* out);
 
 /* Compiled all-pairs variants of (order, precision): *direct variants of the

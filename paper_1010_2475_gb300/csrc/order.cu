@@ -74,7 +74,6 @@ __device__ __forceinline__ unsigned order_key(double x1, double x2, double lo1, 
 // Bounding box of the centres of one CTA's share -> box[4 blockIdx.x ...] = (min1,
 // min2, max1, max2); keys_kernel joins the shares' boxes.  (One CTA for all
 // took 85 us at n = 65536.)
-constexpr int kBoxBlocks = 32;
 __device__ __forceinline__ void warp_box(double& lo1, double& lo2, double& hi1, double& hi2) {
   for (int o = 16; o > 0; o >>= 1) {
     lo1 = fmin(lo1, __shfl_xor_sync(0xffffffffu, lo1, o));
@@ -260,6 +259,12 @@ size_t spatial_order_temp_bytes(int n) {
   return 32 * kBoxBlocks + (size_t)3 * ((size_t)n * 4 + 256) + cub_bytes(n) + 256;
 }
 
+cudaError_t launch_boxes(int n, const double* x, double* boxes, int* count, cudaStream_t st) {
+  *count = std::max(1, std::min(kBoxBlocks, (n + 255) / 256));
+  bbox_kernel<<<*count, 256, 0, st>>>(n, x, boxes);
+  return cudaGetLastError();
+}
+
 cudaError_t launch_spatial_order(int n, const double* x, void* temp, size_t temp_bytes,
                                  int* perm, cudaStream_t st) {
   auto align = [](size_t v) { return (v + 255) & ~(size_t)255; };
@@ -274,8 +279,9 @@ cudaError_t launch_spatial_order(int n, const double* x, void* temp, size_t temp
   off = align(off + (size_t)n * 4);
   size_t cb = cub_bytes(n);
   if (off + cb > temp_bytes) return cudaErrorInvalidValue;
-  const int boxes = std::max(1, std::min(kBoxBlocks, (n + 255) / 256));
-  bbox_kernel<<<boxes, 256, 0, st>>>(n, x, box);
+  int boxes = 0;
+  cudaError_t e = launch_boxes(n, x, box, &boxes, st);
+  if (e != cudaSuccess) return e;
   keys_kernel<<<(n + 255) / 256, 256, 0, st>>>(n, boxes, x, box, kin, iin);
   return cub::DeviceRadixSort::SortPairs(base + off, cb, kin, kout, iin, perm, n, 0, 32, st);
 }

@@ -142,6 +142,10 @@ int finish_scalars(int M);  // doubles launch_prep writes to scal (nullable)
 cudaError_t launch_group_multipole(int M, int n, const void* rec, void* gdata,
                                    const BatchInst* inst, const int* slot_inst,
                                    const int* n_slots, int max_slots, cudaStream_t st);
+// Bounding boxes of the centres: boxes[4 i ...] = (min1, min2, max1, max2) of the
+// i-th share of the particles, *count <= kBoxBlocks of them.
+constexpr int kBoxBlocks = 32;
+cudaError_t launch_boxes(int n, const double* x, double* boxes, int* count, cudaStream_t st);
 // Spatial order: perm[p] = particle at sorted position p (Hilbert order of the
 // centres, ties by index).  temp_bytes() sizes the scratch for n particles.
 size_t spatial_order_temp_bytes(int n);

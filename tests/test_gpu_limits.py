@@ -253,3 +253,20 @@ def test_clusters_beyond_the_range_of_squared_distances(mm, order, monkeypatch):
         assert vel_error_cond(gx[:96], ox, sx) <= 2e-6, (v, tree, local)
         if order >= 1:
             assert rhs_error_cond(gM[:96], oM, sM, order, LAM) <= _tol(order), (v, tree, local)
+
+
+@pytest.mark.parametrize("first", ["sparse", "dense"])
+def test_expansions_follow_the_state(mm, first):
+    """Whether compact groups take expansions depends on the state, not on
+    the state that the first context of the size class held."""
+    order, n = (5, 9001) if first == "sparse" else (3, 9001)
+    rng = np.random.default_rng(order)
+    out = {}
+    for state in (first, {"sparse": "dense", "dense": "sparse"}[first]):
+        x = rng.uniform(-1.0, 1.0, size=(n, 2)) * (2000.0 if state == "sparse" else 10.0)
+        m = _moments(rng.normal(size=n), order, LAM, rng)
+        with mm.Context(order, LAM, 1e-3, mm.MMVM_MIXED_FP32) as ctx:
+            ctx.set_state(x, m, 0.0)
+            ctx.rhs()
+            out[state] = mm.mmvm_pair_expanded(ctx.handle)
+    assert out["dense"] > 0 and out["sparse"] == 0
