@@ -314,8 +314,8 @@ __device__ __forceinline__ double block_sum(const double* __restrict__ v, int n,
 //  * scalars (powers of c, weights of the step) come from the record kernel;
 //    without one (a single particle, batches) two warps form them.
 // Before / now: 420 / 327 us at n = 24000, M = 6, 199 / 183 us at n = 2011, M = 8.
-// Shared memory holds [column][target] arrays: Psi (NB), a (K), X (2), 1 / M_00,
-// the scalars and the groups' sums.  Every global read of the stage input
+// Shared memory holds [column][target] arrays: Psi (NB), a (K), X (2), the
+// scalars and the groups' sums.  Every global read of the stage input
 // precedes the first write behind a barrier.  All threads of the CTA call this;
 // a caller that loops must add a barrier.
 template <int TG>
@@ -325,8 +325,7 @@ __device__ __forceinline__ void finish_block(const FinishArgs& A, int j0, int rb
   double* psi = sm;                 // NB * TG
   double* at = psi + NB * TG;       // K * TG
   double* X = at + K * TG;          // 2 * TG
-  double* m00s = X + 2 * TG;        // TG: 1 / M_00
-  double* cpow = m00s + TG;         // the scalars
+  double* cpow = X + 2 * TG;        // the scalars
   double* cinv = cpow + M + 1;
   double* hs = cinv + M + 1;
   double* gsum = hs + 4;            // max_groups * TG
@@ -367,7 +366,6 @@ __device__ __forceinline__ void finish_block(const FinishArgs& A, int j0, int rb
     psi[b * TG + tt] = v;
   }
   __syncthreads();
-  if (threadIdx.x < TG) m00s[threadIdx.x] = 1.0 / at[threadIdx.x];
   for (int idx = TG + threadIdx.x; idx < TG * K; idx += NT) {
     int s = 0;
     while (tri(s + 1) <= idx / TG) ++s;  // total order of the column
@@ -388,7 +386,8 @@ __device__ __forceinline__ void finish_block(const FinishArgs& A, int j0, int rb
     }
     __syncthreads();  // Psi and the scaled moments
     // 2. centroid sums X_c = sum_m (-1)^{|m|} a_m What_c[m], What_1[m] = -Psi[m+e2],
-    //    What_2[m] = Psi[m+e1]  (eq:xjdot_Final in c = 1 units, self pair excluded);
+    //    What_2[m] = Psi[m+e1]  (eq:xjdot_Final in c = 1 units, self pair excluded),
+    //    over M_00 (the quotient: 1 / M_00 is infinite below 2^-1024);
     //    the columns m of one (target, component) are split over q lanes
     const int q = min(32, NT / (2 * TG));
     if (threadIdx.x < 2 * TG * q) {  // whole warps: 2 TG q is a multiple of 32 here
@@ -402,7 +401,7 @@ __device__ __forceinline__ void finish_block(const FinishArgs& A, int j0, int rb
         acc = fma(a, psi[(comp == 0 ? bcol(m1, m2 + 1) : bcol(m1 + 1, m2)) * TG + tt], acc);
       }
       for (int o = q >> 1; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-      if (part == 0) X[2 * tt + comp] = acc;
+      if (part == 0) X[2 * tt + comp] = acc / at[tt];
     }
     __syncthreads();
   } else if (threadIdx.x < 2 * TG) {
@@ -494,7 +493,7 @@ __device__ __forceinline__ void finish_block(const FinishArgs& A, int j0, int rb
     double ctr = 0.0;
     if (k1c >= 1) ctr += X[2 * tt] * at[mcol(k1c - 1, k2) * TG + tt];
     if (k2 >= 1) ctr += X[2 * tt + 1] * at[mcol(k1c, k2 - 1) * TG + tt];
-    const double dm = fma(ctr, m00s[tt], R) * cinv[kn];  // c^{|k|/2 - 1}
+    const double dm = (R + ctr) * cinv[kn];  // c^{|k|/2 - 1}
     const size_t o = (size_t)j * K + k;
     if (A.mode == 0) {
       A.out_dM[o] = dm;
@@ -508,7 +507,7 @@ __device__ __forceinline__ void finish_block(const FinishArgs& A, int j0, int rb
   }
   if (rb + 1 < rb1) __syncthreads();  // the group sums are reused
   }
-  // 6. centroid velocity xdot_c = c^{-1/2} X_c / M_00 and its stage update
+  // 6. centroid velocity xdot_c = c^{-1/2} X_c and its stage update
   if (rb0 != 0) return;
   // c^{-1/2} (order 0 has only c^0 in its powers, and c^{-1})
   const double cpow1 = M >= 1 ? cpow[1] : sqrt(cinv[0]);
@@ -516,7 +515,7 @@ __device__ __forceinline__ void finish_block(const FinishArgs& A, int j0, int rb
     const int tt = idx >> 1, comp = idx & 1, p = j0 + tt;
     if (p >= A.n) continue;
     const int j = A.perm ? A.perm[p] : p;
-    const double dx = X[idx] * cpow1 * m00s[tt];
+    const double dx = X[idx] * cpow1;
     const size_t ox = (size_t)j * 2 + comp;
     if (A.mode == 0) {
       A.out_dx[ox] = dx;
@@ -701,7 +700,7 @@ cudaError_t launch_prep_batch(int precision, int M, const BatchInst* inst, const
 // Shared memory of a finish CTA of TG targets.
 size_t finish_smem_bytes(int M, int TG, const FinishTab& tab) {
   return sizeof(double) *
-         ((size_t)TG * (n_beta(M) + n_moments(M) + 3 + tab.max_groups) + scal_len(M));
+         ((size_t)TG * (n_beta(M) + n_moments(M) + 2 + tab.max_groups) + scal_len(M));
 }
 
 // Call f(kernel of TG targets) for the run-time TG in {1, 2, 4, 8}.

@@ -270,3 +270,20 @@ def test_expansions_follow_the_state(mm, first):
             ctx.rhs()
             out[state] = mm.mmvm_pair_expanded(ctx.handle)
     assert out["dense"] > 0 and out["sparse"] == 0
+
+
+@pytest.mark.parametrize("n", [2, 300])
+@pytest.mark.parametrize("order", [0, 2])
+def test_circulation_without_a_reciprocal(mm, order, n):
+    """A circulation below 2^-1024 has no finite reciprocal; its velocity is that
+    of any other particle there."""
+    rng = np.random.default_rng(n)
+    x = rng.uniform(-1.0, 1.0, size=(n, 2))
+    m = _moments(rng.normal(size=n), order, LAM, rng, 0.0)
+    m[0] = 0.0
+    m[0, 0] = 4e-309
+    gx, gM = _rhs(mm, order, LAM, x, m, mm.MMVM_FP64)
+    m[0, 0] = 1e-200
+    rx, rM = _rhs(mm, order, LAM, x, m, mm.MMVM_FP64)
+    assert np.isfinite(gx).all() and np.isfinite(gM).all()
+    assert vel_error_rows(gx, rx) <= 1e-12  # 4e-309 keeps 49 bits; products with it round at 5e-324
