@@ -67,7 +67,11 @@ __device__ __forceinline__ void near_source(const T* r, int src, int j, T tz1, T
     l1 = T(0);
     l2 = T(0);
     wm = T(0);
-    if constexpr (!std::is_same<T, float>::value) b1 = T(1e3);  // inside the table form
+    if constexpr (!std::is_same<T, float>::value) {  // the form of the warp's other lanes
+      constexpr double b = 512.0;
+      static_assert(b * b < table_x<T>(3 * M), "the self pair must take the table form");
+      b1 = T(b);
+    }
   }
   PN::run(b1, b2, l1, l2, wm, a, accr);
 }
