@@ -707,32 +707,33 @@ int tune_pair(mmvm_ctx* c, int density) {
     local_choice = 0;
     if (best_v >= 0) {
       mmvm::ListEntry e = mmvm::list_entry(c->M, best_v);
-      double per_pair = 0.0;
-      int rc = time_list_variant(c, e, n, true, false, 0, e0, e1, &per_pair);
-      if (rc) return rc;
-      if (per_pair < best_list) {
-        best_list = per_pair;
-        tree_choice = 1;
-      }
       MMVM_CK(e.far.loc_prepare());
-      for (int tree = 0; tree < 2; ++tree) {
-        rc = time_list_variant(c, e, n, tree != 0, true, 0, e0, e1, &per_pair);
-        if (rc) return rc;
-        if (per_pair < best_list) {
-          best_list = per_pair;
-          tree_choice = tree;
-          local_choice = 1;
-        }
-      }
+      double per_pair = 0.0;
+      int rc = 0;
+      // at the rule's shares and at one per slot: few shares suit the shorter
+      // lists that expansions leave (n = 2011, M = 8: 0.708 and 0.700 ms at the
+      // rule's, 0.70 and 0.66 at one)
+      for (int local = 0; local < 2; ++local)
+        for (int tree = 0; tree < 2; ++tree)
+          for (int seg = 0; seg < 2; ++seg) {
+            if (!local && !tree && !seg) continue;  // timed above
+            rc = time_list_variant(c, e, n, tree != 0, local != 0, seg, e0, e1, &per_pair);
+            if (rc) return rc;
+            if (per_pair < best_list) {
+              best_list = per_pair;
+              tree_choice = tree;
+              local_choice = local;
+            }
+          }
       // shorter lists of close groups remain: the variants rank differently
       struct Timed {
         double per_pair;
         int v, seg;
       };
-      std::vector<Timed> timed{{best_list, best_v, 0}};
+      std::vector<Timed> timed;
       for (int v = 0; v < nl; ++v) {
         mmvm::ListEntry ev = mmvm::list_entry(c->M, v);
-        if (v == best_v || ev.M != c->M) continue;
+        if (ev.M != c->M) continue;
         if (mmvm::list_prepare(ev) != cudaSuccess || mmvm::list_occupancy(ev) < 1) {
           cudaGetLastError();
           continue;
@@ -754,15 +755,16 @@ int tune_pair(mmvm_ctx* c, int density) {
           if (rc) return rc;
           timed.push_back({per_pair, v, seg});
         }
+      best_list = 1e300;
       for (const Timed& t : timed) best_list = std::min(best_list, t.per_pair);
-      // of those within 3 %, the fewest shares: beside other work on the device
+      // of those within 5 %, the fewest shares: beside other work on the device
       // the set-ups cost more (n = 5003, M = 6: 1 and 4 per slot 0.92 and 0.90 ms
       // alone, 2960 and 3190 us per step with three contexts); at equal shares the
       // faster variant at the rule's (the earlier entry)
       const Timed* pick = nullptr;
       auto per_slot = [](const Timed& t) { return t.seg ? t.seg : 2; };  // 0: list_shape's rule
       for (const Timed& t : timed)
-        if (t.per_pair <= 1.03 * best_list && (!pick || per_slot(t) < per_slot(*pick))) pick = &t;
+        if (t.per_pair <= 1.05 * best_list && (!pick || per_slot(t) < per_slot(*pick))) pick = &t;
       best_v = pick->v;
       seg_choice = pick->seg;
       if (best_list < best_full) choice = nv + best_v;
