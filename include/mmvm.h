@@ -179,12 +179,14 @@ int mmvm_pair_time_parts(mmvm_ctx* ctx, double* ms, int32_t max_parts, int32_t* 
  *      group, near pairs with all warps of a CTA on one target group, a
  *      separate far-field kernel);
  *  [1] kernels per evaluation (order slices or column parts; the list form
- *      counts its list build, tree, far and expansion kernels too);
+ *      counts its list build and far kernel too and, with expansions, their four,
+ *      but neither the cut into shares nor the levels of the tree);
  *  [2] targets per CTA (list form: threads per CTA of its first near kernel);
  *  [3] CTAs per SM;  [4] sources between CTA barriers (0: none);
  *  [5] source chunks (list form: most shares of the near pairs that a target
  *      group falls into);
- *  [6] 1 for the list form, else 0;  [7] source ranges of its far kernel.
+ *  [6] list form: 1, with the far field through the tree 2; else 0;  [7] source
+ *      ranges (subtrees) of its far kernel.
  * The variant is chosen by timing the compiled variants for the first state
  * of each size class (log2 n) and density class (the radius in core units of 32
  * particles spread over the bounding box, in powers of two) in the process.

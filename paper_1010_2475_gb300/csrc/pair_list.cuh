@@ -242,8 +242,9 @@ constexpr int kNearFlush = 32;
 // warps' sums cost as much as ~10 rounds of sources, so a CTA should see few
 // groups, and an SM gets one CTA's worth of rounds whatever the lists' lengths.
 // (A CTA per group and segment of its list, the number of segments tuned, against
-// shares, per pass: n = 4096, M = 4 2027 -> 1672 us, n = 2011, M = 8 3935 -> 3383
-// us, n = 5003, M = 6 4771 -> 4218 us, n = 65536, M = 6 60.4 -> 53.9 ms.)
+// shares, per pass alone, with the same limits of the expansions on both sides: n =
+// 4096, M = 4 2027 -> 1672 us, n = 2011, M = 8 3935 -> 3383 us, n = 5003, M = 6 4771 ->
+// 4218 us.)
 //
 // The part is taken in windows of WIN list entries: warp 0 forms the
 // exclusive prefix sums of the entries' near counts, the CTA lists the

@@ -33,7 +33,7 @@
 // loc_radius(M) and groups close to each other (loc_pair; the target group
 // itself among them) stay with the pair kernels.
 // Measured (two patches, n = 65536, M = 6, one right-hand side): all-pairs
-// kernels 68.6 -> 16.0 ms (near pairs one by one 6.6e8 -> 1.2e8, far field 4.0 ->
+// kernels 68.6 -> 16.1 ms (near pairs one by one 6.6e8 -> 1.2e8, far field 4.0 ->
 // 1.3 ms).
 #pragma once
 
